@@ -87,7 +87,7 @@ long long vblock_of(const vl_desc& d, int s) {
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
-    size_t cellwork, coef_v, coef_f, status, u1, u2, cur, fluid_f, counters, select;
+    size_t cellwork, coef_v, coef_f, status, u1, u2, cur, fluid_f, counters, select, todo;
     size_t mlp_w, mlp_m, mlp_v, mlp_g, mlp_acc, mlp_err, mlp_pred, harvest_count, total;
 };
 
@@ -104,7 +104,8 @@ Layout layout_of(const vl_desc& d) {
     L.cur = off; off = align256(off + nc * 3 * sizeof(double));
     L.fluid_f = off; off = align256(off + 2 * nc * 10 * sizeof(float));
     L.counters = off; off = align256(off + VL_NSTATS * sizeof(unsigned long long));
-    L.select = off; off = align256(off + 2 * sizeof(unsigned long long));
+    L.select = off; off = align256(off + 3 * sizeof(unsigned long long));
+    L.todo = off; off = align256(off + nc * 2 * sizeof(unsigned));
     const size_t np = (size_t)VL_MLP_NPARAM * sizeof(float);
     L.mlp_w = off; off = align256(off + np);
     L.mlp_m = off; off = align256(off + np);
@@ -250,6 +251,7 @@ vl_status vlasov_init(const vl_desc* desc, void* const* f_dev, double* fluid_dev
     c->ws.fluid_f = reinterpret_cast<float*>(w + L.fluid_f);
     c->ws.counters = reinterpret_cast<unsigned long long*>(w + L.counters);
     c->ws.fit_select = reinterpret_cast<unsigned long long*>(w + L.select);
+    c->ws.fit_todo = reinterpret_cast<unsigned*>(w + L.todo);
     c->ws.mlp = nullptr;
     c->mlp_w = reinterpret_cast<float*>(w + L.mlp_w);
     c->mlp_m = reinterpret_cast<float*>(w + L.mlp_m);
@@ -572,15 +574,23 @@ vl_status moment_fit_solve(vl_ctx* ctx, int s, const double* vmom, int use_mlp, 
     a.numeric = ctx->status_dev;
     a.wide = a.fp64 ? 0 : ctx->fit_mode[s];
     a.select = nullptr;
+    a.sel = nullptr;
+    a.todo = nullptr;
+    a.ntodo = nullptr;
     cudaStream_t cs = (cudaStream_t)stream;
-    if (d.nvdim == 3 && a.wide < 0) {
-        // the double-float kernel is chosen on the device from the targets
-        st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 2 * sizeof(unsigned long long), cs),
+    // closed-form fits first, the direct kernels take what they leave; a
+    // forced choice of the direct kernel (moment_fit_wide) runs it alone
+    const bool closed = d.nvdim == 3 && (a.fp64 || a.wide < 0) && 2 * a.ncell <= 0xFFFFFFFFLL;
+    if (closed) {
+        st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 3 * sizeof(unsigned long long), cs),
                         "moment_fit (kernel choice)");
         if (st != VL_OK) return st;
-        st = cuda_check(ctx, vl::launch_fit_select(a, ctx->ws.fit_select, cs), "moment_fit (kernel choice)");
-        if (st != VL_OK) return st;
-        a.select = ctx->ws.fit_select;
+        a.select = a.fp64 ? nullptr : ctx->ws.fit_select;
+        a.sel = a.fp64 ? nullptr : ctx->ws.fit_select;
+        a.todo = ctx->ws.fit_todo;
+        a.ntodo = reinterpret_cast<unsigned*>(ctx->ws.fit_select + 2);
+    } else if (a.wide < 0) {
+        a.wide = 1;
     }
     if (use_mlp) {
         vl::MlpInferArgs m;

@@ -42,7 +42,9 @@ struct Workspace {
     double* cur;          // [ncell][3] current density at cell centres
     float* fluid_f;       // [2][ncell][10] FP32 copies of a stage's state and third moments
     unsigned long long* counters;  // [VL_NSTATS]
-    unsigned long long* fit_select;  // [2] device-side choice of the fit kernel (fit_select_kernel)
+    unsigned long long* fit_select;  // [3] device-side choice of the direct fit kernel, then the number of
+                          // fits left to it
+    unsigned* fit_todo;   // [ncell][2] those fits
     float* mlp;           // MLP weights and scratch
 };
 

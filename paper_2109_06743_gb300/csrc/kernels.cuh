@@ -126,17 +126,19 @@ struct FitArgs {
     int wide;               // 1: the fit kernel with the centre-out evaluation, 0: the common
                             // one, -1: chosen on the device from select (moment_fit_wide)
     const unsigned long long* select;  // wide = -1: [2] FP64 bits of the largest n over all
-                            // cells and over the cells that need the wide kernel (fit_select)
+                            // cells and over the cells whose V or F Maxwellian falls by more
+                            // than 60 e-folds from its peak to the farthest corner of the box
+                            // (written by the closed-form kernel)
+    unsigned long long* sel;  // the same words while the closed-form kernel writes them
+    unsigned* todo;         // [2 ncell] fits (2 cell + (0: V, 1: F)) left to the direct kernels
+    unsigned* ntodo;        // their number; null: the direct kernels fit every cell
     int fp64;               // 1: the plain FP64 fit (FP64 mode), 0: double-float on the FP32 pipe
     int* numeric;           // status word (device-visible host memory): set to VL_ENUMERIC when
                             // a target is not finite or has n < 0; may be null
 };
 cudaError_t launch_fit(const FitArgs& a, int nvdim, cudaStream_t st);
-// auto choice of the 2D3V fit kernel: sel[0], sel[1] (zeroed by the caller) get
-// the FP64 bits of the largest n over all cells and over the cells whose V or
-// F Maxwellian falls by more than 60 e-folds from its peak to the farthest
-// corner of the velocity box
-cudaError_t launch_fit_select(const FitArgs& a, unsigned long long* sel, cudaStream_t st);
+// the closed-form fits (closed_fit.cu): sel, ntodo zeroed by the caller
+cudaError_t launch_closed_fit(const FitArgs& a, cudaStream_t st);
 
 // ---- MLP warm start (mlp.cu) ------------------------------------------------------
 struct MlpInferArgs {

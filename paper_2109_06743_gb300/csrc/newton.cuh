@@ -1345,68 +1345,63 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) newton_kernel(FitArgs a) {
         const double nwide = __longlong_as_double((long long)a.select[1]);
         if ((nwide > 1e-10 * nmax) != WIDE) return;
     }
+    // every fit of the species, or those the closed-form kernel left
+    const long long nfit = a.ntodo ? (long long)*a.ntodo : 2 * a.ncell;
+    if (WIDE && a.select && blockIdx.x == 0 && threadIdx.x == 0)
+        atomicAdd(&a.counters[CNT_WIDE_FITS], 2ull * (unsigned long long)a.ncell);
+    const long long per_cta = blockDim.x / kG;
+    if ((long long)blockIdx.x * per_cta >= nfit) return;
     if (threadIdx.x < VL_NSTATS) cnt[threadIdx.x] = 0ull;
     __syncthreads();
     const int gl = glane();
-    const int slot = threadIdx.x / kG;  // 16 cells per CTA
+    const int slot = threadIdx.x / kG;  // 16 fits per CTA
     CellScratch& cs = scratch[slot];
     const unsigned msk = gmask();
-    const long long per_cta = blockDim.x / kG;
     // the trip count is uniform over the CTA, so the four groups of a warp
-    // always call fit_cell together (a group past the last cell takes part
+    // always call fit_cell together (a group past the last fit takes part
     // with have = false)
-    for (long long base = (long long)blockIdx.x * per_cta; base < a.ncell; base += (long long)gridDim.x * per_cta) {
-        const long long cell = base + slot;
-        const bool have = cell < a.ncell;
-        // V targets: the moments of f
+    for (long long base = (long long)blockIdx.x * per_cta; base < nfit; base += (long long)gridDim.x * per_cta) {
+        const bool have = base + slot < nfit;
+        const long long fit = !have ? 0 : (a.ntodo ? (long long)a.todo[base + slot] : base + slot);
+        const long long cell = fit >> 1;
+        const bool fluid = (fit & 1) != 0;
+        // V targets: the moments of f; F targets: the fluid moments rescaled
+        // by n_V / n_F (already done for the fits of the list)
         bool bad = false;
-        if (have)
-            for (int r = 0; r < 2; ++r) {
-                const int c = gl + 8 * r;
-                if (c < 10) {
-                    cs.tgt[c] = a.vmom[cell * 20 + c];
-                    bad = bad || bad_target_pair(a.vmom[cell * 20], cs.tgt[c], c == 0);
-                }
-            }
-        __syncwarp(msk);
-        const double nV = have ? cs.tgt[0] : 0.0;
-        FitWork work = {0u, 0u, 0u, 0u, 0u};
-        int itv = 0, itf = 0;
-        const float* wv = (have && a.warm) ? a.warm + cell * 20 : nullptr;
-        const int stv = fit_cell<N, WIDE>(cs, a, have, have ? a.coef_v + cell * kCoefN : nullptr, wv, &itv, work);
-        __syncwarp(msk);
+        double scale = 1.0, n0 = 0.0;
+        const double* src = fluid ? a.fluid + cell * 10 : a.vmom + cell * 20;
         if (have) {
-            // F targets: the fluid moments rescaled by n_V / n_F
-            const double nF = a.fluid[cell * 10];
-            const double scale = nF > 0.0 ? nV / nF : 0.0;
+            n0 = src[0];
+            if (fluid && !a.ntodo) scale = n0 > 0.0 ? a.vmom[cell * 20] / n0 : 0.0;
             for (int r = 0; r < 2; ++r) {
                 const int c = gl + 8 * r;
                 if (c < 10) {
-                    const double raw = a.fluid[cell * 10 + c];
-                    bad = bad || bad_target_pair(nF, raw, c == 0);
-                    cs.tgt[c] = raw * scale;
+                    const double raw = src[c];
+                    bad = bad || bad_target_pair(n0, raw, c == 0);
+                    cs.tgt[c] = fluid ? raw * scale : raw;
                 }
             }
-            __syncwarp(msk);
+        }
+        __syncwarp(msk);
+        if (have && fluid && !a.ntodo)
             for (int r = 0; r < 2; ++r) {
                 const int c = gl + 8 * r;
                 if (c < 10) a.fluid[cell * 10 + c] = cs.tgt[c];
             }
-        }
         __syncwarp(msk);
-        const float* wf = (have && a.warm) ? a.warm + cell * 20 + 10 : nullptr;
-        const int stf = fit_cell<N, WIDE>(cs, a, have, have ? a.coef_f + cell * kCoefN : nullptr, wf, &itf, work);
+        FitWork work = {0u, 0u, 0u, 0u, 0u};
+        int iters = 0;
+        double* coef = (fluid ? a.coef_f : a.coef_v) + cell * kCoefN;
+        const float* warm = (have && a.warm) ? a.warm + fit * 10 : nullptr;
+        const int st = fit_cell<N, WIDE>(cs, a, have, have ? coef : nullptr, warm, &iters, work);
         bad = __any_sync(msk, bad);
         if (have && gl == 0) {
             if (bad && a.numeric) *reinterpret_cast<volatile int*>(a.numeric) = VL_ENUMERIC;
-            if (WIDE) atomicAdd_block(&cnt[CNT_WIDE_FITS], 2ull);
-            a.status[cell * 2] = stv;
-            a.status[cell * 2 + 1] = stf;
-            atomicAdd_block(&cnt[CNT_ITERS], (unsigned long long)(itv + itf));
-            const unsigned long long fb = (stv == 1) + (stf == 1);
-            if (fb) atomicAdd_block(&cnt[CNT_FALLBACK], fb);
-            const unsigned long long inv = (stv == 2) + (stf == 2);
-            if (inv) atomicAdd_block(&cnt[CNT_INVALID], inv);
+            if (WIDE && !a.select) atomicAdd_block(&cnt[CNT_WIDE_FITS], 1ull);
+            a.status[fit] = st;
+            atomicAdd_block(&cnt[CNT_ITERS], (unsigned long long)iters);
+            if (st == 1) atomicAdd_block(&cnt[CNT_FALLBACK], 1ull);
+            if (st == 2) atomicAdd_block(&cnt[CNT_INVALID], 1ull);
             atomicAdd_block(&cnt[CNT_EVAL_M], (unsigned long long)work.m);
             atomicAdd_block(&cnt[CNT_EVAL_G], (unsigned long long)work.g);
             atomicAdd_block(&cnt[CNT_EVAL_SLOW], (unsigned long long)work.slow);
@@ -1420,16 +1415,20 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) newton_kernel(FitArgs a) {
         atomicAdd(&a.counters[threadIdx.x], cnt[threadIdx.x]);
 }
 
-// One CTA per 16 cells: fits take uneven time (one to several Newton
+// One CTA per 16 fits: fits take uneven time (one to several Newton
 // iterations), so the hardware's CTA scheduler, which starts a new CTA
 // wherever one finishes, balances the load better than a fixed persistent
-// share per CTA (grids beyond 2^31 - 1 CTAs fall back to looping).
+// share per CTA (grids beyond 2^31 - 1 CTAs fall back to looping). The fits
+// left by the closed-form kernel are few and their number is on the device:
+// at most kListBlocks CTAs loop over them.
 // With wide = -1 both kernels are launched and the one not chosen by the
 // device-side selection (a.select) returns at once.
+constexpr long long kListBlocks = 152 * 8;
 template <int N>
 cudaError_t launch_n(const FitArgs& a, cudaStream_t st) {
-    long long blocks = (a.ncell + 15) / 16;
+    long long blocks = (2 * a.ncell + 15) / 16;
     if (blocks > 0x7FFFFFFFLL) blocks = 0x7FFFFFFFLL;
+    if (a.ntodo && blocks > kListBlocks) blocks = kListBlocks;
     FitArgs b = a;
     if (a.wide >= 0) b.select = nullptr;
     if (a.wide != 0) {

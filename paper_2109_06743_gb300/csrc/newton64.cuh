@@ -676,47 +676,44 @@ template <int N>
 __global__ void __launch_bounds__(32 * kCellsPerCta) newton64_kernel(FitArgs a) {
     __shared__ Cell cells[kCellsPerCta];
     __shared__ unsigned long long cnt[VL_NSTATS];
+    // every fit of the species, or those the closed-form kernel left
+    const long long nfit = a.ntodo ? (long long)*a.ntodo : 2 * a.ncell;
+    if ((long long)blockIdx.x * kCellsPerCta >= nfit) return;
     if (threadIdx.x < VL_NSTATS) cnt[threadIdx.x] = 0ull;
     __syncthreads();
     const int lane = lane_id();
     const int slot = threadIdx.x >> 5;
     Cell& cs = cells[slot];
-    for (long long cell = (long long)blockIdx.x * kCellsPerCta + slot; cell < a.ncell;
-         cell += (long long)gridDim.x * kCellsPerCta) {
-        // V targets: the moments of f
-        if (lane < 10) cs.tgt[lane] = a.vmom[cell * 20 + lane];
+    for (long long k = (long long)blockIdx.x * kCellsPerCta + slot; k < nfit; k += (long long)gridDim.x * kCellsPerCta) {
+        const long long fit = a.ntodo ? (long long)a.todo[k] : k;
+        const long long cell = fit >> 1;
+        const bool fluid = (fit & 1) != 0;
+        // V targets: the moments of f; F targets: the fluid moments rescaled
+        // by n_V / n_F (already done for the fits of the list)
+        const double* src = fluid ? a.fluid + cell * 10 : a.vmom + cell * 20;
+        if (lane < 10) cs.tgt[lane] = src[lane];
         __syncwarp();
-        bool bad = lane == 0 && bad_targets(cs.tgt, 10);
-        const double nV = cs.tgt[0];
+        const bool bad = lane == 0 && bad_targets(cs.tgt, 10);
+        if (fluid && !a.ntodo) {
+            const double nF = cs.tgt[0];
+            const double scale = nF > 0.0 ? a.vmom[cell * 20] / nF : 0.0;
+            __syncwarp();
+            if (lane < 10) {
+                cs.tgt[lane] *= scale;
+                a.fluid[cell * 10 + lane] = cs.tgt[lane];
+            }
+        }
+        __syncwarp();
         Work64 work = {0u, 0u, 0u};
-        int itv = 0, itf = 0;
-        const float* wv = a.warm ? a.warm + cell * 20 : nullptr;
-        const int stv = fit_cell64<N>(cs, a, a.coef_v + cell * kCoefN, wv, &itv, work);
-        // F targets: the fluid moments rescaled by n_V / n_F
-        const double nF = a.fluid[cell * 10];
+        int iters = 0;
+        const float* warm = a.warm ? a.warm + fit * 10 : nullptr;
+        const int st = fit_cell64<N>(cs, a, (fluid ? a.coef_f : a.coef_v) + cell * kCoefN, warm, &iters, work);
         if (lane == 0) {
-            double raw[10];
-            for (int q = 0; q < 10; ++q) raw[q] = a.fluid[cell * 10 + q];
-            bad = bad || bad_targets(raw, 10);
-        }
-        const double scale = nF > 0.0 ? nV / nF : 0.0;
-        __syncwarp();
-        if (lane < 10) {
-            cs.tgt[lane] = a.fluid[cell * 10 + lane] * scale;
-        }
-        __syncwarp();
-        if (lane < 10) a.fluid[cell * 10 + lane] = cs.tgt[lane];
-        const float* wf = a.warm ? a.warm + cell * 20 + 10 : nullptr;
-        const int stf = fit_cell64<N>(cs, a, a.coef_f + cell * kCoefN, wf, &itf, work);
-        if (lane == 0) {
-            a.status[cell * 2] = stv;
-            a.status[cell * 2 + 1] = stf;
+            a.status[fit] = st;
             if (bad && a.numeric) *reinterpret_cast<volatile int*>(a.numeric) = VL_ENUMERIC;
-            atomicAdd_block(&cnt[CNT_ITERS], (unsigned long long)(itv + itf));
-            const unsigned long long fb = (stv == 1) + (stf == 1);
-            if (fb) atomicAdd_block(&cnt[CNT_FALLBACK], fb);
-            const unsigned long long inv = (stv == 2) + (stf == 2);
-            if (inv) atomicAdd_block(&cnt[CNT_INVALID], inv);
+            atomicAdd_block(&cnt[CNT_ITERS], (unsigned long long)iters);
+            if (st == 1) atomicAdd_block(&cnt[CNT_FALLBACK], 1ull);
+            if (st == 2) atomicAdd_block(&cnt[CNT_INVALID], 1ull);
             atomicAdd_block(&cnt[CNT_EVAL64_M], (unsigned long long)work.m);
             atomicAdd_block(&cnt[CNT_EVAL64_G], (unsigned long long)work.g);
             if (work.warm) atomicAdd_block(&cnt[CNT_WARM], (unsigned long long)work.warm);
@@ -730,8 +727,9 @@ __global__ void __launch_bounds__(32 * kCellsPerCta) newton64_kernel(FitArgs a) 
 
 template <int N>
 cudaError_t launch64(const FitArgs& a, cudaStream_t st) {
-    long long blocks = (a.ncell + kCellsPerCta - 1) / kCellsPerCta;
+    long long blocks = (2 * a.ncell + kCellsPerCta - 1) / kCellsPerCta;
     if (blocks > 0x7FFFFFFFLL) blocks = 0x7FFFFFFFLL;
+    if (a.ntodo && blocks > 152 * 16) blocks = 152 * 16;  // the list is short, its length on the device
     if (blocks < 1) return cudaSuccess;
     newton64_kernel<N><<<(unsigned)blocks, 32 * kCellsPerCta, 0, st>>>(a);
     count_launch();
