@@ -11,11 +11,14 @@
 // C_ab = ((row a of E2) x B)_b, E3 = int v v v f taken from the Vlasov solver
 // and reconstructed with the same CWENO polynomials as U. Fluxes are the
 // central-upwind (local Lax-Friedrichs) flux with the ten-moment wave speed
-// |u_d| + sqrt(3 Theta_dd) of the two neighbouring cells. One thread per cell
-// and stage. The state stays in FP64; the reconstruction, fluxes and sources
-// (the right-hand side L) are computed in R = double in FP64 mode and in
-// R = float in FP32 mode (on GB300 the FP64 pipe runs at ~1/58 of the FP32
-// pipe), and the Runge-Kutta combination U0 + dt L is formed in FP64.
+// |u_d| + sqrt(3 Theta_dd) of the two neighbouring cells. The state stays in
+// FP64; the reconstruction, fluxes and sources (the right-hand side L) are
+// computed in R = double in FP64 mode and in R = float in FP32 mode (on GB300
+// the FP64 pipe runs at ~1/58 of the FP32 pipe), and the Runge-Kutta
+// combination U0 + dt L is formed in FP64.
+//
+// 2D3V: one CTA per tile of cells and stage (fluid_tile_kernel); 1D1V: one
+// thread per cell.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -58,89 +61,13 @@ __device__ __forceinline__ void cweno3_point(R um, R u0, R up, R* left, R* right
     *right = wl * lr + wr * rr + wc * cr;
 }
 
-struct FluidCtx {
-    const FluidArgs* a;
-    int nc, nq, qoff;
-    bool use0, use1;  // wq0 != 0, wq1 != 0 (decided once per thread)
-};
-
-// sign of a component under y -> -y (v_y -> -v_y)
-__device__ __forceinline__ double parity_state(int k) {
-    // n nux nuy nuz xx xy xz yy yz zz
-    return (k == 2 || k == 5 || k == 8) ? -1.0 : 1.0;
-}
-__device__ __forceinline__ double parity_q(int k) {
-    // xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
-    return (k == 1 || k == 4 || k == 6 || k == 8) ? -1.0 : 1.0;
-}
-
-// resolve (ix, iy) with periodic x and periodic-or-wall y; returns the
-// linear cell index and the mirror flag
-__device__ __forceinline__ long long resolve(const FluidArgs& a, int ix, int iy, bool* mir) {
-    ix %= a.nx;
-    if (ix < 0) ix += a.nx;
-    *mir = false;
-    if (iy < 0 || iy >= a.ny) {
-        if (a.bc_y == 1) {
-            iy = iy < 0 ? -1 - iy : 2 * a.ny - 1 - iy;
-            *mir = true;
-        } else {
-            iy %= a.ny;
-            if (iy < 0) iy += a.ny;
-        }
-    }
-    return (long long)iy * a.nx + ix;
-}
-
-// In FP32 mode the stage input and the weighted third moments are converted
-// to float once per stage (fluid_prep_kernel) instead of at each of the ~16
-// stencil reads of every value (FP64-to-FP32 conversions run on the FP64
-// pipe); the values are the same.
-template <typename R>
-__device__ __forceinline__ R state_at(const FluidCtx& c, int k, int ix, int iy) {
-    bool mir;
-    long long id = resolve(*c.a, ix, iy, &mir);
-    R v = (sizeof(R) == 4 && c.a->Usf) ? (R)c.a->Usf[id * c.nc + k] : (R)c.a->Us[id * c.nc + k];
-    return (mir && c.a->nvdim == 3) ? v * (R)parity_state(k) : v;
-}
-
-// Q = wq0 q0 + wq1 q1 (the weights are 0, 1/2 or 1, exact in R)
-template <typename R>
-__device__ __forceinline__ R q_value(const FluidArgs& a, const FluidCtx& c, long long id, int k) {
-    R v = R(0);
-    if (c.use0) v += (R)a.wq0 * (R)a.q0[id * a.nmom + c.qoff + k];
-    if (c.use1) v += (R)a.wq1 * (R)a.q1[id * a.nmom + c.qoff + k];
-    return v;
-}
-
-template <typename R>
-__device__ __forceinline__ R q_at(const FluidCtx& c, int k, int ix, int iy) {
-    bool mir;
-    long long id = resolve(*c.a, ix, iy, &mir);
-    const FluidArgs& a = *c.a;
-    const R v = (sizeof(R) == 4 && a.Qf) ? (R)a.Qf[id * c.nq + k] : q_value<R>(a, c, id, k);
-    return (mir && a.nvdim == 3) ? v * (R)parity_q(k) : v;
-}
-
-template <typename R>
-__device__ __forceinline__ R wave_speed(int nvdim, int dir, const R* u) {
-    R n = u[0];
-    if (!(n > R(0))) return R(0);
-    R ud = u[1 + dir] / n;
-    R e2 = nvdim == 1 ? u[2] : u[4 + s2(dir, dir)];
-    R th = e2 / n - ud * ud;
-    if (th < R(0)) th = R(0);
-    return fabs(ud) + sqrt(R(3) * th);
-}
-
-template <typename R>
-__device__ __forceinline__ R flux_of(int nvdim, int dir, int k, const R* u, const R* q) {
-    if (nvdim == 1) return k == 0 ? u[1] : (k == 1 ? u[2] : q[0]);
-    if (k == 0) return u[1 + dir];
-    if (k < 4) return u[4 + s2(dir, k - 1)];
-    const int ab[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
-    return q[s3(dir, ab[k - 4][0], ab[k - 4][1])];
-}
+// index of the flux of component k in direction dir: a state component (n:
+// nu_d; nu_a: E2_da) or 10 + a third moment (E2_ab: E3_dab)
+static __constant__ signed char kFluxVar[2][10] = {{1, 4, 5, 6, 10, 11, 12, 13, 14, 15},
+                                                   {2, 5, 7, 8, 11, 13, 14, 16, 17, 18}};
+// sign of a component under y -> -y (v_y -> -v_y): the state n nux nuy nuz xx
+// xy xz yy yz zz, then the third moments xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
+static __constant__ signed char kParity[20] = {1, 1, -1, 1, 1, -1, 1, 1, -1, 1, 1, -1, 1, 1, -1, 1, -1, 1, -1, 1};
 
 // Gradient-closure model (Sec. 2.3): with zero heat flux the third moment
 // is that of the Maxwellian with the state's n, u and E2,
@@ -166,220 +93,154 @@ __device__ __forceinline__ void closure_e3(const R* s, R* e3) {
                                   R(2) * n * v[k] * v[a] * v[b];
 }
 
-// theta = E2 / n - u u of cell (ix, iy), ghosts as for the state
-template <typename R>
-__device__ __forceinline__ void theta_cell(const FluidCtx& c, int ix, int iy, R* th) {
-    R s[10];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) s[k] = state_at<R>(c, k, ix, iy);
-    const R n = s[0];
-    const R inv = n > R(0) ? R(1) / n : R(0);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = a; b < 3; ++b) th[s2(a, b)] = s[4 + s2(a, b)] * inv - (s[1 + a] * inv) * (s[1 + b] * inv);
-}
+// One RK stage over a tile of TX x TY cells, in shared-memory phases:
+//   1. the stage input and the weighted third moments of the tile and two
+//      halo cells per side (periodic images, mirror cells beyond a wall),
+//      converted to R once;
+//   2. the reconstruction of every component in every cell a flux of the tile
+//      reads, once per direction (left and right interface values), and the
+//      wave speeds; with CLOSURE the third moments of the interface states;
+//   3. the flux differences, one (cell, component) per thread;
+//   4. the sources, one thread per cell (with CLOSURE also the heat flux from
+//      theta of the tile and its neighbours);
+//   5. the Runge-Kutta combination, one (cell, component) per thread, so that
+//      the FP64 state is read and written in contiguous runs.
+// What bounds it: the reconstruction's arithmetic (four divisions a point).
+// One thread per cell formed every point three times (for its own and both
+// neighbours' fluxes) in one serial chain of about 20 k instructions, 60 us
+// per stage however small the grid; here a point is formed 1.25-1.4 times and
+// 256 threads share a tile. Measured (GB300): one FP32 step (three stages) of
+// 128 x 64 cells 180 -> 37 us; the closure model's step of 64 x 64 cells in
+// FP64, both species and fields, 1257 -> 330 us; same bits. Tiles of 8 x 8
+// cells where they fill the chip twice (1.25 points formed per point used),
+// else 8 x 4 (1.38, but more CTAs).
+constexpr int kTileThreads = 256;
+template <typename R, int TX, int TY>
+struct FluidTile {
+    static constexpr int HX = TX + 4, HY = TY + 4;          // with halo
+    static constexpr int PX = (TX + 2) * TY, PY = TX * (TY + 2);  // reconstructed points per direction
+    R s[20][HX * HY];
+    R x[20][2][PX], y[20][2][PY];  // [component][left, right interface value][point]
+    R wx[PX], wy[PY];              // wave speeds
+    R l[10][TX * TY];
+};
 
-// value of component k of the state (q = false) or of the third moments
-// (q = true) in a resolved cell (id, mirror flag)
-template <typename R>
-__device__ __forceinline__ R value_at(const FluidCtx& c, bool q, int k, long long id, bool mir) {
-    const FluidArgs& a = *c.a;
-    R v;
-    if (!q) v = (sizeof(R) == 4 && a.Usf) ? (R)a.Usf[id * c.nc + k] : (R)a.Us[id * c.nc + k];
-    else v = (sizeof(R) == 4 && a.Qf) ? (R)a.Qf[id * c.nq + k] : q_value<R>(a, c, id, k);
-    if (mir && a.nvdim == 3) v *= (R)(q ? parity_q(k) : parity_state(k));
-    return v;
-}
-
-// Numerical fluxes through the two interfaces of a cell in direction dir
-// (Hm: with the neighbour below, Hp: with the neighbour above). The five
-// cells of the stencil are resolved once; each of the three middle cells is
-// reconstructed once (its left and right interface values), which serves
-// both interfaces.
-// The numerical fluxes of cell_fluxes with the third moments from f (no
-// closure), one flux component at a time so that few values are live: the
-// interface states of component k (for the dissipation term) and of the
-// component whose value is k's flux (state component 1+dir, 4+(dir,k-1) or
-// third moment (dir,a,b)). The wave speeds come from the cell averages.
-template <typename R, int NV>
-__device__ __forceinline__ void cell_fluxes_lean(const FluidCtx& c, int dir, int ix, int iy, R* Hm, R* Hp) {
-    constexpr int NC = NV == 1 ? 3 : 10;
-    long long id[5];
-    bool mir[5];
-#pragma unroll
-    for (int o = 0; o < 5; ++o)
-        id[o] = resolve(*c.a, ix + (dir == 0 ? o - 2 : 0), iy + (dir == 1 ? o - 2 : 0), &mir[o]);
-    // wave speeds |u_d| + sqrt(3 Theta_dd) of cells -1, 0, +1
-    R ws[3];
-    const int kd = NV == 1 ? 2 : 4 + s2(dir, dir);
-#pragma unroll
-    for (int o = 0; o < 3; ++o) {
-        const R n = value_at<R>(c, false, 0, id[o + 1], mir[o + 1]);
-        const R nu = value_at<R>(c, false, 1 + dir, id[o + 1], mir[o + 1]);
-        const R e2 = value_at<R>(c, false, kd, id[o + 1], mir[o + 1]);
+template <typename R, bool CLOSURE, int TX, int TY>
+__global__ void __launch_bounds__(kTileThreads) fluid_tile_kernel(FluidArgs a) {
+    typedef FluidTile<R, TX, TY> Tile;
+    constexpr int HX = Tile::HX, HY = Tile::HY, PX = Tile::PX, PY = Tile::PY, NV = CLOSURE ? 10 : 20;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Tile& t = *reinterpret_cast<Tile*>(smem_raw);
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int nx = a.nx, ny = a.ny;
+    const bool use0 = a.wq0 != 0.0, use1 = a.wq1 != 0.0;
+    const int tid = threadIdx.x;
+    for (int e = tid; e < HX * HY * 10; e += kTileThreads) {
+        const int k = e % 10, p = e / 10, lx = p % HX, ly = p / HX;
+        if ((lx < 2 || lx >= TX + 2) && (ly < 2 || ly >= TY + 2)) continue;  // corners are not read
+        int ix = x0 + lx - 2, iy = y0 + ly - 2;
+        ix %= nx;
+        if (ix < 0) ix += nx;
+        bool mir = false;
+        if (iy < 0 || iy >= ny) {
+            if (a.bc_y == 1) {
+                iy = iy < 0 ? -1 - iy : 2 * ny - 1 - iy;
+                iy = iy < 0 ? 0 : iy;  // only rows beyond the last tile's own halo
+                mir = true;
+            } else {
+                iy %= ny;
+                if (iy < 0) iy += ny;
+            }
+        }
+        const long long id = (long long)iy * nx + ix;
+        R v = (R)a.Us[id * 10 + k];
+        t.s[k][p] = mir ? v * (R)kParity[k] : v;
+        if (!CLOSURE) {
+            // Q = wq0 q0 + wq1 q1 (the weights are 0, 1/2 or 1, exact in R)
+            v = R(0);
+            if (use0) v += (R)a.wq0 * (R)a.q0[id * 20 + 10 + k];
+            if (use1) v += (R)a.wq1 * (R)a.q1[id * 20 + 10 + k];
+            t.s[10 + k][p] = mir ? v * (R)kParity[10 + k] : v;
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < NV * PX; e += kTileThreads) {
+        const int k = e / PX, p = e % PX, c = (p / (TX + 2) + 2) * HX + p % (TX + 2) + 1;
+        const R* u = t.s[k] + c;
+        cweno3_point<R>(u[-1], u[0], u[1], &t.x[k][0][p], &t.x[k][1][p]);
+    }
+    for (int e = tid; e < NV * PY; e += kTileThreads) {
+        const int k = e / PY, p = e % PY, c = (p / TX + 1) * HX + p % TX + 2;
+        const R* u = t.s[k] + c;
+        cweno3_point<R>(u[-HX], u[0], u[HX], &t.y[k][0][p], &t.y[k][1][p]);
+    }
+    // wave speeds |u_d| + sqrt(3 Theta_dd) from the cell averages
+    for (int e = tid; e < PX + PY; e += kTileThreads) {
+        const int dir = e < PX ? 0 : 1, p = dir ? e - PX : e;
+        const int c = dir ? (p / TX + 1) * HX + p % TX + 2 : (p / (TX + 2) + 2) * HX + p % (TX + 2) + 1;
+        const R n = t.s[0][c];
         R w = R(0);
         if (n > R(0)) {
-            const R ud = nu / n;
-            R th = e2 / n - ud * ud;
+            const R ud = t.s[1 + dir][c] / n;
+            R th = t.s[dir ? 7 : 4][c] / n - ud * ud;
             if (th < R(0)) th = R(0);
             w = fabs(ud) + sqrt(R(3) * th);
         }
-        ws[o] = w;
+        if (dir) t.wy[p] = w;
+        else t.wx[p] = w;
     }
-    const R sm = fmax(ws[0], ws[1]), sp = fmax(ws[1], ws[2]);
-    // interface states of one component: the right value of cell -1, the
-    // left and right values of cell 0 and the left value of cell +1
-    auto recon = [&](bool q, int k, R& rm, R& l0, R& r0, R& lp) {
-        const R a0 = value_at<R>(c, q, k, id[0], mir[0]), a1 = value_at<R>(c, q, k, id[1], mir[1]);
-        const R a2 = value_at<R>(c, q, k, id[2], mir[2]), a3 = value_at<R>(c, q, k, id[3], mir[3]);
-        const R a4 = value_at<R>(c, q, k, id[4], mir[4]);
-        R l, r;
-        cweno3_point<R>(a0, a1, a2, &l, &r);
-        rm = r;
-        cweno3_point<R>(a1, a2, a3, &l0, &r0);
-        cweno3_point<R>(a2, a3, a4, &lp, &r);
-    };
+    __syncthreads();
+    if (CLOSURE) {
+        for (int e = tid; e < 2 * (PX + PY); e += kTileThreads) {
+            const int side = e & 1, q = e >> 1, dir = q < PX ? 0 : 1, p = dir ? q - PX : q;
+            R s[10], e3[10];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        R um, u0, up, cp;
-        recon(false, k, um, u0, up, cp);
-        // the flux of component k
-        bool fq;
-        int fk;
-        if (NV == 1) {
-            fq = k == 2;
-            fk = k == 0 ? 1 : (k == 1 ? 2 : 0);
-        } else if (k == 0) {
-            fq = false;
-            fk = 1 + dir;
-        } else if (k < 4) {
-            fq = false;
-            fk = 4 + s2(dir, k - 1);
-        } else {
-            const int ab[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
-            fq = true;
-            fk = s3(dir, ab[k - 4][0], ab[k - 4][1]);
+            for (int k = 0; k < 10; ++k) s[k] = dir ? t.y[k][side][p] : t.x[k][side][p];
+            closure_e3<R>(s, e3);
+#pragma unroll
+            for (int k = 0; k < 10; ++k) {
+                if (dir) t.y[10 + k][side][p] = e3[k];
+                else t.x[10 + k][side][p] = e3[k];
+            }
         }
-        R fm, f0, fp, fc;
-        recon(fq, fk, fm, f0, fp, fc);
-        Hm[k] = R(0.5) * (fm + f0) - R(0.5) * sm * (u0 - um);
-        Hp[k] = R(0.5) * (fp + fc) - R(0.5) * sp * (cp - up);
+        __syncthreads();
     }
-}
-
-template <typename R, int NV>
-__device__ __forceinline__ void cell_fluxes(const FluidCtx& c, int dir, int ix, int iy, R* Hm, R* Hp) {
-    constexpr int NC = NV == 1 ? 3 : 10, NQ = NV == 1 ? 1 : 10;
-    long long id[5];
-    bool mir[5];
+    // Walls: the interface beyond the last row is the wall itself (mirror
+    // ghosts already give its flux).
+    const R invhx = (R)a.invdx, invhy = (R)a.invdy;
+    for (int e = tid; e < 10 * TX * TY; e += kTileThreads) {
+        const int k = e / (TX * TY), cell = e % (TX * TY), cx = cell % TX, cy = cell / TX;
+        R L = R(0);
 #pragma unroll
-    for (int o = 0; o < 5; ++o)
-        id[o] = resolve(*c.a, ix + (dir == 0 ? o - 2 : 0), iy + (dir == 1 ? o - 2 : 0), &mir[o]);
-    // uE[p][side]: reconstruction in cell p-1 (p = 0, 1, 2 for cells -1, 0, +1)
-    R um[10], u0[10], up[10], cm[10], c0[10], cp[10];  // left/right states of the two interfaces
-    R qm_[10], q0_[10], qp_[10], qmm[10];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        const R a0 = value_at<R>(c, false, k, id[0], mir[0]), a1 = value_at<R>(c, false, k, id[1], mir[1]);
-        const R a2 = value_at<R>(c, false, k, id[2], mir[2]), a3 = value_at<R>(c, false, k, id[3], mir[3]);
-        const R a4 = value_at<R>(c, false, k, id[4], mir[4]);
-        R l, r;
-        cweno3_point<R>(a0, a1, a2, &l, &r);  // cell -1
-        um[k] = r;                            // left state of the lower interface
-        cweno3_point<R>(a1, a2, a3, &l, &r);  // cell 0
-        u0[k] = l;                            // right state of the lower interface
-        up[k] = r;                            // left state of the upper interface
-        cweno3_point<R>(a2, a3, a4, &l, &r);  // cell +1
-        cp[k] = l;                            // right state of the upper interface
-        cm[k] = a1;
-        c0[k] = a2;
-        qmm[k] = a3;  // cell averages of cell +1 (wave speed)
-    }
-    if (c.a->closure) {
-        closure_e3<R>(um, qm_);
-        closure_e3<R>(u0, q0_);
-        closure_e3<R>(up, qp_);
-    }
-    R qcp[10];
-    if (c.a->closure) {
-        closure_e3<R>(cp, qcp);
-    } else {
-#pragma unroll
-        for (int k = 0; k < NQ; ++k) {
-            const R a0 = value_at<R>(c, true, k, id[0], mir[0]), a1 = value_at<R>(c, true, k, id[1], mir[1]);
-            const R a2 = value_at<R>(c, true, k, id[2], mir[2]), a3 = value_at<R>(c, true, k, id[3], mir[3]);
-            const R a4 = value_at<R>(c, true, k, id[4], mir[4]);
-            R l, r;
-            cweno3_point<R>(a0, a1, a2, &l, &r);
-            qm_[k] = r;
-            cweno3_point<R>(a1, a2, a3, &l, &r);
-            q0_[k] = l;
-            qp_[k] = r;
-            cweno3_point<R>(a2, a3, a4, &l, &r);
-            qcp[k] = l;
+        for (int dir = 0; dir < 2; ++dir) {
+            const int p = dir ? (cy + 1) * TX + cx : cy * (TX + 2) + cx + 1, st = dir ? TX : 1;
+            const R* ul = dir ? t.y[k][0] : t.x[k][0];
+            const R* ur = dir ? t.y[k][1] : t.x[k][1];
+            const int f = kFluxVar[dir][k];
+            const R* fl = dir ? t.y[f][0] : t.x[f][0];
+            const R* fr = dir ? t.y[f][1] : t.x[f][1];
+            const R* ws = dir ? t.wy : t.wx;
+            const R sm = fmax(ws[p - st], ws[p]), sp = fmax(ws[p], ws[p + st]);
+            const R Hm = R(0.5) * (fr[p - st] + fl[p]) - R(0.5) * sm * (ul[p] - ur[p - st]);
+            const R Hp = R(0.5) * (fr[p] + fl[p + st]) - R(0.5) * sp * (ul[p + st] - ur[p]);
+            L -= (Hp - Hm) * (dir ? invhy : invhx);
         }
+        t.l[k][cell] = L;
     }
-    constexpr int nvdim = NV;
-    const R sm = fmax(wave_speed<R>(nvdim, dir, cm), wave_speed<R>(nvdim, dir, c0));
-    const R sp = fmax(wave_speed<R>(nvdim, dir, c0), wave_speed<R>(nvdim, dir, qmm));
+    __syncthreads();
+    for (int cell = tid; cell < TX * TY; cell += kTileThreads) {
+        const int cx = cell % TX, cy = cell / TX, ix = x0 + cx, iy = y0 + cy;
+        if (ix >= nx || iy >= ny) continue;
+        const int c = (cy + 2) * HX + cx + 2;
+        R u[10], eb[6], L[10];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        Hm[k] = R(0.5) * (flux_of<R>(nvdim, dir, k, um, qm_) + flux_of<R>(nvdim, dir, k, u0, q0_)) -
-                R(0.5) * sm * (u0[k] - um[k]);
-        Hp[k] = R(0.5) * (flux_of<R>(nvdim, dir, k, up, qp_) + flux_of<R>(nvdim, dir, k, cp, qcp)) -
-                R(0.5) * sp * (cp[k] - up[k]);
-    }
-}
-
-// One thread per cell and stage; NV = 1 (1D1V: three components) or 3
-// (2D3V: ten), a compile-time count so that the per-component arrays stay in
-// registers.
-#ifndef VL_FLUID_MIN_BLOCKS_F32
-#define VL_FLUID_MIN_BLOCKS_F32 8
-#endif
-#ifndef VL_FLUID_MIN_BLOCKS_F64
-#define VL_FLUID_MIN_BLOCKS_F64 1
-#endif
-template <typename R, int NV, bool CLOSURE>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? VL_FLUID_MIN_BLOCKS_F32 : VL_FLUID_MIN_BLOCKS_F64)
-    fluid_stage_kernel(FluidArgs a) {
-    constexpr int NC = NV == 1 ? 3 : 10;
-    long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (cell >= (long long)a.nx * a.ny) return;
-    const int ix = (int)(cell % a.nx), iy = (int)(cell / a.nx);
-    FluidCtx c;
-    c.a = &a;
-    c.nc = NC;
-    c.nq = NV == 1 ? 1 : 10;
-    c.qoff = NV == 1 ? 3 : 10;
-    c.use0 = a.wq0 != 0.0;
-    c.use1 = a.wq1 != 0.0;
-    R L[10];
+        for (int k = 0; k < 10; ++k) {
+            u[k] = t.s[k][c];
+            L[k] = t.l[k][cell];
+        }
 #pragma unroll
-    for (int k = 0; k < NC; ++k) L[k] = R(0);
-    constexpr int ndir = NV == 1 ? 1 : 2;
-    R Hm[10], Hp[10];
-#pragma unroll
-    for (int dir = 0; dir < ndir; ++dir) {
-        const R invh = (R)(1.0 / (dir == 0 ? a.dx : a.dy));
-        if (CLOSURE) cell_fluxes<R, NV>(c, dir, ix, iy, Hm, Hp);
-        else cell_fluxes_lean<R, NV>(c, dir, ix, iy, Hm, Hp);
-        // walls: the interface beyond the last row is the wall itself
-        // (mirror ghosts already give its flux); nothing special needed
-#pragma unroll
-        for (int k = 0; k < NC; ++k) L[k] -= (Hp[k] - Hm[k]) * invh;
-    }
-    R u[10], eb[6];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) u[k] = (R)a.Us[cell * NC + k];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) eb[k] = (R)a.eb[cell * 6 + k];
-    const R qm = (R)a.qm;
-    if (NV == 1) {
-        L[1] += qm * u[0] * eb[0];
-        L[2] += qm * R(2) * u[1] * eb[0];
-    } else {
+        for (int k = 0; k < 6; ++k) eb[k] = (R)a.eb[((long long)iy * nx + ix) * 6 + k];
+        const R qm = (R)a.qm;
         const R* E = eb;
         const R* B = eb + 3;
         const R* nu = u + 1;
@@ -404,71 +265,152 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? VL_FLUID_MIN_BLOCKS_F32 
             for (int q = p; q < 3; ++q) L[4 + s2(p, q)] += qm * (nu[p] * E[q] + nu[q] * E[p] + C[p][q] + C[q][p]);
         if (CLOSURE) {
             // heat flux of the closure: -(1/m) div Q = chi_k0 n v_t lap theta,
-            // v_t = sqrt(tr(theta) / 3), five-point Laplacian
-            R t0[6], tw[6], te[6], ts[6], tn[6];
-            theta_cell<R>(c, ix, iy, t0);
-            theta_cell<R>(c, ix - 1, iy, tw);
-            theta_cell<R>(c, ix + 1, iy, te);
-            theta_cell<R>(c, ix, iy - 1, ts);
-            theta_cell<R>(c, ix, iy + 1, tn);
-            const R tr = t0[0] + t0[3] + t0[5];
+            // theta = E2 / n - u u, v_t = sqrt(tr(theta) / 3), five-point Laplacian
+            R th[5][6];
+            const int at[5] = {c, c - 1, c + 1, c - HX, c + HX};
+#pragma unroll
+            for (int o = 0; o < 5; ++o) {
+                const R n = t.s[0][at[o]];
+                const R inv = n > R(0) ? R(1) / n : R(0);
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int q = p; q < 3; ++q)
+                        th[o][s2(p, q)] =
+                            t.s[4 + s2(p, q)][at[o]] * inv - (t.s[1 + p][at[o]] * inv) * (t.s[1 + q][at[o]] * inv);
+            }
+            const R tr = th[0][0] + th[0][3] + th[0][5];
             const R vt = sqrt(tr > R(0) ? tr / R(3) : R(0));
             const R coef = (R)a.chi_k0 * u[0] * vt;
-            const R ix2 = (R)(1.0 / (a.dx * a.dx)), iy2 = (R)(1.0 / (a.dy * a.dy));
+            const R ix2 = (R)a.invdx2, iy2 = (R)a.invdy2;
 #pragma unroll
             for (int k = 0; k < 6; ++k)
-                L[4 + k] += coef * ((te[k] - R(2) * t0[k] + tw[k]) * ix2 + (tn[k] - R(2) * t0[k] + ts[k]) * iy2);
+                L[4 + k] += coef * ((th[2][k] - R(2) * th[0][k] + th[1][k]) * ix2 +
+                                    (th[4][k] - R(2) * th[0][k] + th[3][k]) * iy2);
         }
-    }
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        double us = a.Us[cell * NC + k];
-        double u0 = a.a0 != 0.0 ? a.U0[cell * NC + k] : 0.0;
-        a.Uout[cell * NC + k] = a.a0 * u0 + a.a1 * (us + a.dt * (double)L[k]);
+        for (int k = 0; k < 10; ++k) t.l[k][cell] = L[k];
+    }
+    __syncthreads();
+    for (int e = tid; e < 10 * TX * TY; e += kTileThreads) {
+        const int k = e % 10, cell = e / 10, ix = x0 + cell % TX, iy = y0 + cell / TX;
+        if (ix >= nx || iy >= ny) continue;
+        const long long o = ((long long)iy * nx + ix) * 10 + k;
+        const double us = a.Us[o];
+        const double u0 = a.a0 != 0.0 ? a.U0[o] : 0.0;
+        a.Uout[o] = a.a0 * u0 + a.a1 * (us + a.dt * (double)t.l[k][cell]);
     }
 }
 
-// FP32 copies of the stage input and of the weighted third moments
-__global__ void fluid_prep_kernel(FluidArgs a) {
-    long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (cell >= (long long)a.nx * a.ny) return;
-    FluidCtx c;
-    c.a = &a;
-    c.nc = a.nvdim == 1 ? 3 : 10;
-    c.nq = a.nvdim == 1 ? 1 : 10;
-    c.qoff = a.nvdim == 1 ? 3 : 10;
-    c.use0 = a.wq0 != 0.0;
-    c.use1 = a.wq1 != 0.0;
-    for (int k = 0; k < c.nc; ++k) a.Usf[cell * c.nc + k] = (float)a.Us[cell * c.nc + k];
-    if (a.Qf)
-        for (int k = 0; k < c.nq; ++k) a.Qf[cell * c.nq + k] = q_value<float>(a, c, cell, k);
+// 1D1V (three components n, nu, E2; periodic): one thread per cell and stage.
+template <typename R>
+__global__ void __launch_bounds__(128) fluid1d_stage_kernel(FluidArgs a) {
+    const int ix = blockIdx.x * blockDim.x + threadIdx.x, nx = a.nx;
+    if (ix >= nx) return;
+    const bool use0 = a.wq0 != 0.0, use1 = a.wq1 != 0.0;
+    int id[5];
+#pragma unroll
+    for (int o = 0; o < 5; ++o) {
+        id[o] = (ix + o - 2) % nx;
+        if (id[o] < 0) id[o] += nx;
+    }
+    auto value = [&](bool q, int k, int c) -> R {
+        if (!q) return (R)a.Us[(long long)c * 3 + k];
+        R v = R(0);
+        if (use0) v += (R)a.wq0 * (R)a.q0[(long long)c * 4 + 3 + k];
+        if (use1) v += (R)a.wq1 * (R)a.q1[(long long)c * 4 + 3 + k];
+        return v;
+    };
+    // wave speeds |u| + sqrt(3 Theta) of cells -1, 0, +1
+    R ws[3];
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+        const R n = value(false, 0, id[o + 1]);
+        const R nu = value(false, 1, id[o + 1]);
+        const R e2 = value(false, 2, id[o + 1]);
+        R w = R(0);
+        if (n > R(0)) {
+            const R ud = nu / n;
+            R th = e2 / n - ud * ud;
+            if (th < R(0)) th = R(0);
+            w = fabs(ud) + sqrt(R(3) * th);
+        }
+        ws[o] = w;
+    }
+    const R sm = fmax(ws[0], ws[1]), sp = fmax(ws[1], ws[2]);
+    // interface states of one component: the right value of cell -1, the
+    // left and right values of cell 0 and the left value of cell +1
+    auto recon = [&](bool q, int k, R& rm, R& l0, R& r0, R& lp) {
+        const R a0 = value(q, k, id[0]), a1 = value(q, k, id[1]), a2 = value(q, k, id[2]), a3 = value(q, k, id[3]),
+                a4 = value(q, k, id[4]);
+        R l, r;
+        cweno3_point<R>(a0, a1, a2, &l, &r);
+        rm = r;
+        cweno3_point<R>(a1, a2, a3, &l0, &r0);
+        cweno3_point<R>(a2, a3, a4, &lp, &r);
+    };
+    const R invh = (R)a.invdx;
+    R L[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        R um, u0, up, cp, fm, f0, fp, fc;
+        recon(false, k, um, u0, up, cp);
+        recon(k == 2, k == 2 ? 0 : k + 1, fm, f0, fp, fc);
+        const R Hm = R(0.5) * (fm + f0) - R(0.5) * sm * (u0 - um);
+        const R Hp = R(0.5) * (fp + fc) - R(0.5) * sp * (cp - up);
+        L[k] = R(0);
+        L[k] -= (Hp - Hm) * invh;
+    }
+    R u[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[k] = (R)a.Us[(long long)ix * 3 + k];
+    const R E = (R)a.eb[(long long)ix * 6], qm = (R)a.qm;
+    L[1] += qm * u[0] * E;
+    L[2] += qm * R(2) * u[1] * E;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const long long o = (long long)ix * 3 + k;
+        const double us = a.Us[o];
+        const double u0 = a.a0 != 0.0 ? a.U0[o] : 0.0;
+        a.Uout[o] = a.a0 * u0 + a.a1 * (us + a.dt * (double)L[k]);
+    }
+}
+
+template <typename R, bool CLOSURE, int TX, int TY>
+static cudaError_t launch_tile(const FluidArgs& a, cudaStream_t st) {
+    auto* k = fluid_tile_kernel<R, CLOSURE, TX, TY>;
+    const int smem = (int)sizeof(FluidTile<R, TX, TY>);
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((a.nx + TX - 1) / TX), (unsigned)((a.ny + TY - 1) / TY));
+    k<<<grid, kTileThreads, smem, st>>>(a);
+    count_launch();
+    return cudaGetLastError();
 }
 
 cudaError_t launch_fluid_stage(const FluidArgs& args, cudaStream_t st) {
     FluidArgs a = args;
-    long long n = (long long)a.nx * a.ny;
-    int threads = 128;
-    if (a.precision == 64) {
-        a.Usf = nullptr;
-        a.Qf = nullptr;
-    }
-    if (a.Usf) {
-        fluid_prep_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(a);
-        count_launch();
-    }
-    const unsigned grid = (unsigned)((n + threads - 1) / threads);
+    a.invdx = 1.0 / a.dx;
+    a.invdy = 1.0 / a.dy;
+    a.invdx2 = 1.0 / (a.dx * a.dx);
+    a.invdy2 = 1.0 / (a.dy * a.dy);
     if (a.nvdim == 1) {
-        if (a.precision == 64) fluid_stage_kernel<double, 1, false><<<grid, threads, 0, st>>>(a);
-        else fluid_stage_kernel<float, 1, false><<<grid, threads, 0, st>>>(a);
-    } else if (a.closure) {
-        if (a.precision == 64) fluid_stage_kernel<double, 3, true><<<grid, threads, 0, st>>>(a);
-        else fluid_stage_kernel<float, 3, true><<<grid, threads, 0, st>>>(a);
-    } else {
-        if (a.precision == 64) fluid_stage_kernel<double, 3, false><<<grid, threads, 0, st>>>(a);
-        else fluid_stage_kernel<float, 3, false><<<grid, threads, 0, st>>>(a);
+        const unsigned grid = (unsigned)((a.nx + 127) / 128);
+        if (a.precision == 64) fluid1d_stage_kernel<double><<<grid, 128, 0, st>>>(a);
+        else fluid1d_stage_kernel<float><<<grid, 128, 0, st>>>(a);
+        count_launch();
+        return cudaGetLastError();
     }
-    count_launch();
-    return cudaGetLastError();
+    // 8 x 8 tiles once there are two per SM
+    const bool large = (long long)((a.nx + 7) / 8) * ((a.ny + 7) / 8) >= 2 * 152;
+    if (a.closure) {
+        if (a.precision == 64)
+            return large ? launch_tile<double, true, 8, 8>(a, st) : launch_tile<double, true, 8, 4>(a, st);
+        return large ? launch_tile<float, true, 8, 8>(a, st) : launch_tile<float, true, 8, 4>(a, st);
+    }
+    if (a.precision == 64)
+        return large ? launch_tile<double, false, 8, 8>(a, st) : launch_tile<double, false, 8, 4>(a, st);
+    return large ? launch_tile<float, false, 8, 8>(a, st) : launch_tile<float, false, 8, 4>(a, st);
 }
 
 }  // namespace vl
