@@ -104,7 +104,7 @@ Layout layout_of(const vl_desc& d) {
     L.cur = off; off = align256(off + nc * 3 * sizeof(double));
     L.counters = off; off = align256(off + VL_NSTATS * sizeof(unsigned long long));
     L.select = off; off = align256(off + 3 * sizeof(unsigned long long));
-    L.todo = off; off = align256(off + nc * 2 * sizeof(unsigned));
+    L.todo = off; off = align256(off + nc * 2 * sizeof(unsigned long long));
     const size_t np = (size_t)VL_MLP_NPARAM * sizeof(float);
     L.mlp_w = off; off = align256(off + np);
     L.mlp_m = off; off = align256(off + np);
@@ -249,7 +249,7 @@ vl_status vlasov_init(const vl_desc* desc, void* const* f_dev, double* fluid_dev
     c->ws.cur = reinterpret_cast<double*>(w + L.cur);
     c->ws.counters = reinterpret_cast<unsigned long long*>(w + L.counters);
     c->ws.fit_select = reinterpret_cast<unsigned long long*>(w + L.select);
-    c->ws.fit_todo = reinterpret_cast<unsigned*>(w + L.todo);
+    c->ws.fit_todo = reinterpret_cast<unsigned long long*>(w + L.todo);
     c->ws.mlp = nullptr;
     c->mlp_w = reinterpret_cast<float*>(w + L.mlp_w);
     c->mlp_m = reinterpret_cast<float*>(w + L.mlp_m);
@@ -565,6 +565,7 @@ vl_status moment_fit_solve(vl_ctx* ctx, int s, const double* vmom, int use_mlp, 
     a.ncell = ncell_of(d);
     a.nv = d.nv[s][0];
     fill_box(d, s, a.vmin, a.dv);
+    for (int q = 0; q < 3; ++q) a.inv_dv[q] = 1.0 / a.dv[q];
     for (int q = 0; q < 3; ++q) a.vmax[q] = a.vmin[q] + a.dv[q] * (d.nvdim == 3 || q == 0 ? d.nv[s][q] : 1);
     a.tol = d.fit_tol;
     a.max_iter = d.fit_max_iter;
@@ -578,17 +579,18 @@ vl_status moment_fit_solve(vl_ctx* ctx, int s, const double* vmom, int use_mlp, 
     cudaStream_t cs = (cudaStream_t)stream;
     // closed-form fits first, the direct kernels take what they leave; a
     // forced choice of the direct kernel (moment_fit_wide) runs it alone
-    const bool closed = d.nvdim == 3 && (a.fp64 || a.wide < 0) && 2 * a.ncell <= 0xFFFFFFFFLL;
-    if (closed) {
-        st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 3 * sizeof(unsigned long long), cs),
-                        "moment_fit (kernel choice)");
-        if (st != VL_OK) return st;
-        a.select = a.fp64 ? nullptr : ctx->ws.fit_select;
-        a.sel = a.fp64 ? nullptr : ctx->ws.fit_select;
-        a.todo = ctx->ws.fit_todo;
-        a.ntodo = reinterpret_cast<unsigned*>(ctx->ws.fit_select + 2);
-    } else if (a.wide < 0) {
-        a.wide = 1;
+    if (d.nvdim == 3 && (a.fp64 || a.wide < 0)) {
+        const bool closed = a.nv >= vl::kClosedMin;
+        if (closed || !a.fp64) {
+            st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 3 * sizeof(unsigned long long), cs),
+                            "moment_fit (kernel choice)");
+            if (st != VL_OK) return st;
+        }
+        if (!a.fp64) a.select = a.sel = ctx->ws.fit_select;
+        if (closed) {
+            a.todo = ctx->ws.fit_todo;
+            a.ntodo = reinterpret_cast<unsigned*>(ctx->ws.fit_select + 2);
+        }
     }
     if (use_mlp) {
         vl::MlpInferArgs m;

@@ -10,16 +10,18 @@
 // step (delta_0, delta_1, delta_2) is P <- P - 2 delta_2, m <- m + P^-1
 // delta_1, L <- L + delta_0 + delta_1 . P^-1 delta_1 / 2.
 //
-// What the closed form refuses, a step that fails the descent test and a fit
-// that does not converge go on a list; the direct kernels then fit those from
-// their start as before. Results agree to the fit tolerance either way.
+// What the closed form refuses, a step that fails the descent test, a fit that
+// does not converge and (FP32 mode) one whose line parameters would round
+// differently (rounds_alike) go on a list; the direct kernels then fit those
+// from their start as before. Results agree to the fit tolerance either way.
 //
 // Why one thread per fit: an evaluation is about 5 k operations with little
 // parallelism inside (three axes, two sides), against 152 k for the direct
 // sums by eight lanes; 65536 fits fill the chip 14 warps deep per SM.
-// Measured (GB300, cold starts): 65536 fits of 16^3 Harris ions 2.16-2.28 ->
-// 0.29 ms, 65536 network-started fits of 12^3 asymmetric-sheet electrons 2.11
-// -> 0.55 ms, 16384 fits in FP64 mode 5.08 -> 0.45 ms.
+// Measured (GB300), closed form and list: 65536 cold fits of 16^3 Harris ions
+// 2.23 -> 0.43 ms (0.29 + 0.14), 65536 network-started fits of 12^3
+// asymmetric-sheet electrons 2.14 -> 0.78 ms, 16384 fits in FP64 mode 5.08 ->
+// 0.44 ms.
 #pragma once
 
 #include "closed_form.cuh"
@@ -101,6 +103,7 @@ CF_FN double log_of(double x) { return log(x); }
 struct FitCount {
     int iters;
     unsigned evals, grams;
+    float last, res, prev;  // size of the last Newton step, residuals after and before it (relative to n)
 };
 
 // thresholds of the direct kernels: damping test above kDamp n, Gram sums with
@@ -165,6 +168,7 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
         }
         if (gmax <= tolj) {
             cnt.iters += it;
+            cnt.res = (float)rel;
             return true;
         }
         if (it >= max_iter) return false;
@@ -191,8 +195,15 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
                 Gc[4 + sym(a, c)] = Gj[4 + sym(a, c)] - m[a] * Gj[1 + c] - m[c] * Gc[1 + a];
         if (!newton_direction<J>(e.C, Gc, dl)) return false;
         gd = J(0);
+        J big = J(0);
         CF_UNROLL
-        for (int q = 0; q < 10; ++q) gd += Gc[q] * dl[q];
+        for (int q = 0; q < 10; ++q) {
+            gd += Gc[q] * dl[q];
+            const J v = fabs(dl[q]);
+            big = v > big ? v : big;
+        }
+        cnt.last = (float)big;
+        cnt.prev = (float)rel;
         check = far;
         gram = more_steps(rel, (J)tol, J(0));
         // the step
@@ -314,6 +325,43 @@ CF_FN bool from_eta(const typename Jac<T>::type (&eta)[10], Maxw<T>& g) {
 CF_FN double wide_of(df2 a) { return (double)a.hi + (double)a.lo; }
 CF_FN double wide_of(double a) { return a; }
 
+// FP32 mode: the exchange rounds a fit's line parameters (fit.cu) to float,
+// and one unit in the last place of L moves the whole Maxwellian by 5e-7. Two
+// fits of the same targets differ by the rounding of their sums, by a few 1e-6
+// of the last Newton step (FP32 Jacobian) and, where a residual lies at the
+// tolerance, by one step more or less (measured against the direct kernels
+// over 1.6e5 fits: 5e-13, 1.8e-6 of the step, the residual or the step). A fit
+// with a parameter that close to a rounding boundary is decided by the direct
+// kernel, so that f does not depend on which kernel made a fit (about two
+// fits in ten thousand; small off-diagonal parameters, whose last place moves
+// nothing by 1e-8, do not count).
+template <typename T>
+CF_FN bool rounds_alike(const Maxw<T>& g, const FitBox<T>& b, const double (&u0)[3], const double (&sg)[3], double tol,
+                        const FitArgs& a, const FitCount& fc) {
+    const double last = fc.last, res = fc.res;
+    double eps = 8e-13 + 2e-6 * last;
+    if (res > 0.9 * tol) eps += res;
+    if ((double)fc.prev < 1.1 * tol) eps += 2.2 * last;
+    auto alike = [](double p, double d) { return (float)(p - d) == (float)(p + d); };
+    auto small = [&](double p, double d) { return fabs(p) < 0.015625 || alike(p, d); };
+    const double e2 = 1.5 * eps, e4 = 3.0 * eps;
+    double h[3], P[6];
+    bool ok = alike(wide_of(g.L), e2);
+    CF_UNROLL
+    for (int q = 0; q < 3; ++q) {
+        h[q] = wide_of(b.h[q]);
+        const double is = sg[q] * a.inv_dv[q];
+        ok = ok && alike((u0[q] - a.vmin[q]) * a.inv_dv[q] - 0.5 + is * wide_of(g.m[q]), e2 * is);
+    }
+    CF_UNROLL
+    for (int p = 0; p < 3; ++p)
+        CF_UNROLL
+        for (int q = p; q < 3; ++q) P[sym(p, q)] = h[p] * h[q] * wide_of(g.P[sym(p, q)]);
+    const double iz = 1.0 / P[5], gx = -P[2] * iz, gy = -P[4] * iz;
+    ok = ok && alike(0.5 * P[5], e2 * P[5]) && alike(P[0] + P[2] * gx, e4 * P[0]) && alike(P[3] + P[4] * gy, e4 * P[3]);
+    return ok && small(gx, e4) && small(gy, e4) && small(P[1] + P[2] * gy, e4 * h[0] * h[1]);
+}
+
 #ifdef __CUDACC__
 
 // Thread g fits Maxwellian g & 1 (0: the moments of f, 1: the fluid's,
@@ -329,7 +377,8 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
     __syncthreads();
     const long long fit = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool have = fit < 2 * a.ncell;
-    FitCount fc = {0, 0u, 0u};
+    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 1.f};
+    bool left = false;
     unsigned warm = 0u;
     unsigned long long top = 0ull, wide = 0ull;
     if (have) {
@@ -381,6 +430,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
                 }
                 good = from_eta<T>(eta, g) && closed_newton<T>(g, b, a.nv, Tt, t[0], a.tol, a.max_iter, fc);
             }
+            if (!kF64 && good) good = rounds_alike<T>(g, b, u0, sg, a.tol, a, fc);
             if (good) {
                 warm = started ? 1u : 0u;
                 coef[0] = wide_of(g.L);
@@ -420,9 +470,18 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
                 }
             }
         }
-        if (!good) {
-            fc = {0, 0u, 0u};
-            a.todo[atomicAdd(a.ntodo, 1u)] = (unsigned)fit;
+        left = !good;
+        if (left) fc = {0, 0u, 0u, 0.f, 0.f, 1.f};
+    }
+    if (kF64) {
+        if (left) a.todo[atomicAdd(a.ntodo, 1u)] = (unsigned long long)fit;
+    } else {
+        // eight lanes hold four cells: V fits on the even ones, F on the odd
+        const unsigned m = __ballot_sync(0xffffffffu, left) >> (threadIdx.x & 24);
+        const int w = threadIdx.x & 7;
+        if (w < 2) {
+            const unsigned v = m >> w, keep = (v & 1u) | ((v >> 1) & 2u) | ((v >> 2) & 4u) | ((v >> 3) & 8u);
+            if (keep) a.todo[atomicAdd(a.ntodo, 1u)] = (unsigned long long)((fit >> 3) * 2 + w) << 4 | keep;
         }
     }
     // CTA totals, then one atomic per counter

@@ -42,8 +42,8 @@ struct Workspace {
     double* cur;          // [ncell][3] current density at cell centres
     unsigned long long* counters;  // [VL_NSTATS]
     unsigned long long* fit_select;  // [3] device-side choice of the direct fit kernel, then the number of
-                          // fits left to it
-    unsigned* fit_todo;   // [ncell][2] those fits
+                          // entries left to it
+    unsigned long long* fit_todo;  // [2 ncell] those fits
     float* mlp;           // MLP weights and scratch
 };
 

@@ -128,16 +128,24 @@ struct FitArgs {
     const unsigned long long* select;  // wide = -1: [2] FP64 bits of the largest n over all
                             // cells and over the cells whose V or F Maxwellian falls by more
                             // than 60 e-folds from its peak to the farthest corner of the box
-                            // (written by the closed-form kernel)
-    unsigned long long* sel;  // the same words while the closed-form kernel writes them
-    unsigned* todo;         // [2 ncell] fits (2 cell + (0: V, 1: F)) left to the direct kernels
+                            // (written by the closed-form kernel or fit_select_kernel)
+    unsigned long long* sel;  // the same words, for the kernel that writes them
+    unsigned long long* todo;  // what the closed-form kernel leaves to the direct kernels. FP64 mode:
+                            // fits, 2 cell + (0: V, 1: F). FP32 mode: units of four cells' V or F
+                            // fits, (2 (cell / 4) + (0: V, 1: F)) * 16 + a bit per cell to be kept
     unsigned* ntodo;        // their number; null: the direct kernels fit every cell
+    double inv_dv[3];
     int fp64;               // 1: the plain FP64 fit (FP64 mode), 0: double-float on the FP32 pipe
     int* numeric;           // status word (device-visible host memory): set to VL_ENUMERIC when
                             // a target is not finite or has n < 0; may be null
 };
 cudaError_t launch_fit(const FitArgs& a, int nvdim, cudaStream_t st);
-// the closed-form fits (closed_fit.cu): sel, ntodo zeroed by the caller
+// the closed-form fits (closed_fit.cu): sel, ntodo zeroed by the caller. For
+// blocks of kClosedMin^3 and more: an 8^3 block of +-5 thermal speeds resolves
+// them with 0.8 cells each, where the Poisson modes of the tails' corners
+// matter and most fits are refused (measured with the closed form tried first:
+// 8192 FP32 fits of Harris ions 222 -> 307 us, 16384 FP64 fits 3.34 -> 3.63 ms)
+constexpr int kClosedMin = 12;
 cudaError_t launch_closed_fit(const FitArgs& a, cudaStream_t st);
 
 // ---- MLP warm start (mlp.cu) ------------------------------------------------------

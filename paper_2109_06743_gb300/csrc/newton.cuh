@@ -71,22 +71,44 @@ struct CellScratch {
     double Jd[100];     // precise-mode Gram matrix
 };
 
-__device__ __forceinline__ int glane() { return threadIdx.x & (kG - 1); }
-__device__ __forceinline__ unsigned gmask() { return 0xFFu << ((threadIdx.x & 31) & ~(kG - 1)); }
-__device__ __forceinline__ int gbase() { return (threadIdx.x & 31) & ~(kG - 1); }
+// S = 1: 8 lanes per cell, four cells per warp (a unit is a warp). S = 4: a
+// warp per cell, four lanes in the place of each of the 8; they share the
+// lines of the lane's run and repeat the rest, so that every sum is formed in
+// the same order and a fit has the same bits (a unit is a CTA of four warps).
+template <int S>
+__device__ __forceinline__ int glane() { return (threadIdx.x / S) & (kG - 1); }
+template <int S>
+__device__ __forceinline__ unsigned gmask() {
+    return S == 1 ? 0xFFu << ((threadIdx.x & 31) & ~(kG - 1)) : 0xffffffffu;
+}
+template <int S>
+__device__ __forceinline__ int gbase() { return S == 1 ? (threadIdx.x & 31) & ~(kG - 1) : 0; }
+// one thread per cell
+template <int S>
+__device__ __forceinline__ bool glead() { return (threadIdx.x & (kG * S - 1)) == 0; }
+// vote of the unit's four cells
+template <int S>
+__device__ __forceinline__ bool unit_any(bool x) {
+    if constexpr (S == 1) return __any_sync(0xffffffffu, x) != 0;
+    else return __syncthreads_or(x) != 0;
+}
 
-__device__ __forceinline__ float gbcastf(float v, int src) { return __shfl_sync(gmask(), v, gbase() + src); }
-__device__ __forceinline__ double gbcastd(double v, int src) { return __shfl_sync(gmask(), v, gbase() + src); }
+template <int S>
+__device__ __forceinline__ float gbcastf(float v, int src) { return __shfl_sync(gmask<S>(), v, gbase<S>() + src * S); }
+template <int S>
+__device__ __forceinline__ double gbcastd(double v, int src) { return __shfl_sync(gmask<S>(), v, gbase<S>() + src * S); }
 
+template <int S>
 __device__ __forceinline__ float gsumf(float v) {
 #pragma unroll
-    for (int o = kG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask(), v, o);
-    return gbcastf(v, 0);
+    for (int o = kG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask<S>(), v, o * S);
+    return gbcastf<S>(v, 0);
 }
+template <int S>
 __device__ __forceinline__ double gsumd(double v) {
 #pragma unroll
-    for (int o = kG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask(), v, o);
-    return gbcastd(v, 0);
+    for (int o = kG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask<S>(), v, o * S);
+    return gbcastd<S>(v, 0);
 }
 
 // running double-float sum: s plus the accumulated error terms e
@@ -126,15 +148,24 @@ __device__ __forceinline__ void acc2_add_mag(acc2& A, float hi, float lo) {
     A.e = __fadd_rn(A.e, __fadd_rn(__fsub_rn(small, __fsub_rn(s, big)), lo));
     A.s = s;
 }
+template <int S>
 __device__ __forceinline__ df2 gsum_acc(acc2 a) {
 #pragma unroll
     for (int o = kG / 2; o > 0; o >>= 1) {
-        float s = __shfl_xor_sync(gmask(), a.s, o);
-        float e = __shfl_xor_sync(gmask(), a.e, o);
+        float s = __shfl_xor_sync(gmask<S>(), a.s, o * S);
+        float e = __shfl_xor_sync(gmask<S>(), a.e, o * S);
         acc2_add(a, s, e);
     }
     df2 r = df2_qtwo_sum(a.s, a.e);
-    return {gbcastf(r.hi, 0), gbcastf(r.lo, 0)};
+    return {gbcastf<S>(r.hi, 0), gbcastf<S>(r.lo, 0)};
+}
+// the line sums of lane s of the four that stand for one
+__device__ __forceinline__ acc2 from_sub(acc2 a, int s) {
+    const int src = (threadIdx.x & 28) + s;
+    return {__shfl_sync(0xffffffffu, a.s, src), __shfl_sync(0xffffffffu, a.e, src)};
+}
+__device__ __forceinline__ float from_sub(float a, int s) {
+    return __shfl_sync(0xffffffffu, a, (threadIdx.x & 28) + s);
 }
 
 // a * b as an unnormalised pair: p = fl(a.hi b.hi) and the FP32 sum of the
@@ -182,9 +213,9 @@ __device__ __noinline__ void index_coeffs(const df2* e, const df2* wc, const df2
 // Can float recurrences represent every value and one-cell step of the
 // block? (the minimum of a concave quadratic over a box is at a corner;
 // one-cell steps are linear in position, extreme at the corners)
-template <int N>
+template <int N, int S>
 __device__ bool edge_ok(const df2* kcd) {
-    const int gl = glane();
+    const int gl = glane<S>();
     constexpr float hN = 0.5f * (N - 1);
     float k[10];
 #pragma unroll
@@ -207,7 +238,7 @@ __device__ bool edge_ok(const df2* kcd) {
         float d2 = k[7] * (2.f * yy + 1.f) + k[2] - hN * k[5] + k[8] * z;
         ok = ok && fabsf(d2) < 80.f;
     }
-    return __all_sync(gmask(), ok);
+    return __all_sync(gmask<S>(), ok);
 }
 
 __device__ __forceinline__ void gram_line(float* g, const float* T, float cj, float ck) {
@@ -287,9 +318,9 @@ __device__ __forceinline__ void plane_flush(acc2 (&m)[10], float (&g)[GRAM ? 35 
 // (cs.g) from the high parts of the same values, in one pass over the block;
 // every line starts at v_x's lowest cell and every run of line starts at
 // v_y's lowest, so every value of the block must be in the float range.
-template <int N, bool GRAM>
+template <int N, bool GRAM, int S>
 __device__ __noinline__ void eval_edge(CellScratch& cs, const df2* kc) {
-    const int gl = glane();
+    const int gl = glane<S>();
     constexpr float hN = 0.5f * (N - 1);
     constexpr int R = (N * N) / kG;
     const int l0 = gl * R, l1 = l0 + R;
@@ -311,83 +342,162 @@ __device__ __noinline__ void eval_edge(CellScratch& cs, const df2* kc) {
 #pragma unroll
     for (int q = 0; q < (GRAM ? 15 : 1); ++q) G[q] = 0.f;
     df2 Ms = {0.f, 0.f}, rs = {0.f, 0.f}, rl = {0.f, 0.f};
+    if constexpr (S > 1) {
+        // S lines at a time, one per lane: starts in turn by every lane, the
+        // lines side by side, then their sums in turn
+        const int sub = threadIdx.x & (S - 1);
 #pragma unroll 1
-    for (int l = l0; l < l1; ++l) {
-        const int j = l % N, k = l / N;
-        const float cj = (float)j - hN, ck = (float)k - hN;
-        if (l == l0 || j == 0) {
-            // B = kx + kxy cj + kxz ck; C = k0 + ky cj + kz ck + kyy cj^2 + kyz cj ck + kzz ck^2
-            df2 B = dadd(kc[1], dadd(df2_mulf(kc[5], cj), df2_mulf(kc[6], ck)));
-            df2 C = dadd(kc[0], dadd(df2_mulf(kc[2], cj), df2_mulf(kc[3], ck)));
-            C = dadd(C, dadd(df2_mulf(kc[7], cj * cj), dadd(df2_mulf(kc[8], cj * ck), df2_mulf(kc[9], ck * ck))));
-            // start value at c_x = -hN, first ratio, line-to-line ratio
-            Ms = df2_exp(dadd(df2_mulf(kc[4], hN * hN), dadd(dmul(B, mhN), C)));
-            rs = df2_exp(dadd(df2_mulf(kc[4], 2.f - N), B));
-            rl = df2_exp(dadd(dadd(kc[2], df2_mulf(kc[5], -hN)), dadd(df2_mulf(kc[7], 2.f * cj + 1.f), df2_mulf(kc[8], ck))));
-        }
-        acc2 S0 = {0.f, 0.f}, S1 = {0.f, 0.f}, S2 = {0.f, 0.f};
-        float T0 = 0.f, T1 = 0.f, T2 = 0.f, T3 = 0.f, T4 = 0.f;
-        df2 M = Ms, r = rs;
-        float ci = ci0;
-// unrolled by 2 (measured: 4.5% faster than by 4, 10% faster than by 8)
-#pragma unroll 2
-        for (int i = 0; i < N; ++i) {
-            // ordered Fast2Sum (S0, S2: non-negative terms; S1: any sign;
-            // measured: Harris fit 11.95 -> 11.63 ms per step, TwoSum's bits)
-            // of the weighted terms as chained products, each split exactly
-            // by an FMA: M ci = p1 + e1, (p1 + e1) ci = p2 + e2 (no ci^2;
-            // the Jacobian's sums of degree 3 and 4 continue the chain)
-            acc2_add_nn(S0, M.hi, M.lo);
-            const float p1 = __fmul_rn(M.hi, ci);
-            float e1 = fmaf(M.hi, ci, -p1);
-            e1 = fmaf(M.lo, ci, e1);
-            acc2_add_mag(S1, p1, e1);
-            const float p2 = __fmul_rn(p1, ci);
-            float e2 = fmaf(p1, ci, -p2);
-            e2 = fmaf(e1, ci, e2);
-            acc2_add_nn(S2, p2, e2);
-            if (GRAM) {
-                const float p3 = __fmul_rn(p2, ci);
-                T0 = __fadd_rn(T0, M.hi);
-                T1 = __fadd_rn(T1, p1);
-                T2 = __fadd_rn(T2, p2);
-                T3 = __fadd_rn(T3, p3);
-                T4 = fmaf(p3, ci, T4);
+        for (int lb = l0; lb < l1; lb += S) {
+            df2 M = Ms, r = rs;
+#pragma unroll 1
+            for (int s = 0; s < S && lb + s < l1; ++s) {
+                const int l = lb + s;
+                const int j = l % N, k = l / N;
+                const float cj = (float)j - hN, ck = (float)k - hN;
+                if (l == l0 || j == 0) {
+                    // B = kx + kxy cj + kxz ck; C = k0 + ky cj + kz ck + kyy cj^2 + kyz cj ck + kzz ck^2
+                    df2 B = dadd(kc[1], dadd(df2_mulf(kc[5], cj), df2_mulf(kc[6], ck)));
+                    df2 C = dadd(kc[0], dadd(df2_mulf(kc[2], cj), df2_mulf(kc[3], ck)));
+                    C = dadd(C, dadd(df2_mulf(kc[7], cj * cj), dadd(df2_mulf(kc[8], cj * ck), df2_mulf(kc[9], ck * ck))));
+                    // start value at c_x = -hN, first ratio, line-to-line ratio
+                    Ms = df2_exp(dadd(df2_mulf(kc[4], hN * hN), dadd(dmul(B, mhN), C)));
+                    rs = df2_exp(dadd(df2_mulf(kc[4], 2.f - N), B));
+                    rl = df2_exp(dadd(dadd(kc[2], df2_mulf(kc[5], -hN)), dadd(df2_mulf(kc[7], 2.f * cj + 1.f), df2_mulf(kc[8], ck))));
+                }
+                if (s == sub) {
+                    M = Ms;
+                    r = rs;
+                }
+                Ms = df2_mul(Ms, rl);
+                rl = df2_mul(rl, e_j);
+                rs = df2_mul(rs, e_xy);
             }
-            // unnormalised products where only the pair's sum is read (the
-            // ratio always, the value without the Jacobian's FP32 sums of
-            // its high part): three operations fewer each (measured: fit
-            // 11.63 -> 11.06 ms per step; iterations unchanged)
-            M = GRAM ? df2_mul(M, r) : df2_mul_raw(M, r);
-            r = df2_mul_raw(r, e_in);
-            ci += 1.f;
+            acc2 S0 = {0.f, 0.f}, S1 = {0.f, 0.f}, S2 = {0.f, 0.f};
+            float T0 = 0.f, T1 = 0.f, T2 = 0.f, T3 = 0.f, T4 = 0.f;
+            float ci = ci0;
+        // as below: unrolled by 2 (measured: 4.5% faster than by 4, 10% faster than by 8)
+#pragma unroll 2
+            for (int i = 0; i < N; ++i) {
+                // ordered Fast2Sum (S0, S2: non-negative terms; S1: any sign;
+                // measured: Harris fit 11.95 -> 11.63 ms per step, TwoSum's bits)
+                // of the weighted terms as chained products, each split exactly
+                // by an FMA: M ci = p1 + e1, (p1 + e1) ci = p2 + e2 (no ci^2;
+                // the Jacobian's sums of degree 3 and 4 continue the chain)
+                acc2_add_nn(S0, M.hi, M.lo);
+                const float p1 = __fmul_rn(M.hi, ci);
+                float e1 = fmaf(M.hi, ci, -p1);
+                e1 = fmaf(M.lo, ci, e1);
+                acc2_add_mag(S1, p1, e1);
+                const float p2 = __fmul_rn(p1, ci);
+                float e2 = fmaf(p1, ci, -p2);
+                e2 = fmaf(e1, ci, e2);
+                acc2_add_nn(S2, p2, e2);
+                if (GRAM) {
+                    const float p3 = __fmul_rn(p2, ci);
+                    T0 = __fadd_rn(T0, M.hi);
+                    T1 = __fadd_rn(T1, p1);
+                    T2 = __fadd_rn(T2, p2);
+                    T3 = __fadd_rn(T3, p3);
+                    T4 = fmaf(p3, ci, T4);
+                }
+                // unnormalised products where only the pair's sum is read (the
+                // ratio always, the value without the Jacobian's FP32 sums of
+                // its high part): three operations fewer each (measured: fit
+                // 11.63 -> 11.06 ms per step; iterations unchanged)
+                M = GRAM ? df2_mul(M, r) : df2_mul_raw(M, r);
+                r = df2_mul_raw(r, e_in);
+                ci += 1.f;
+            }
+#pragma unroll 1
+            for (int s = 0; s < S && lb + s < l1; ++s) {
+                const int l = lb + s, j = l % N, k = l / N;
+                const float cj = (float)j - hN, ck = (float)k - hN;
+                const float T[5] = {GRAM ? from_sub(T0, s) : 0.f, GRAM ? from_sub(T1, s) : 0.f,
+                                    GRAM ? from_sub(T2, s) : 0.f, GRAM ? from_sub(T3, s) : 0.f,
+                                    GRAM ? from_sub(T4, s) : 0.f};
+                plane_add<GRAM>(P, G, from_sub(S0, s), from_sub(S1, s), from_sub(S2, s), T, cj - shy);
+                if (j == N - 1 || l == l1 - 1) plane_flush<GRAM>(m, g, P, G, ck - shz);
+            }
         }
-        const float T[5] = {T0, T1, T2, T3, T4};
-        plane_add<GRAM>(P, G, S0, S1, S2, T, cj - shy);
-        if (j == N - 1 || l == l1 - 1) plane_flush<GRAM>(m, g, P, G, ck - shz);
-        Ms = df2_mul(Ms, rl);
-        rl = df2_mul(rl, e_j);
-        rs = df2_mul(rs, e_xy);
+    } else {
+#pragma unroll 1
+        for (int l = l0; l < l1; ++l) {
+            const int j = l % N, k = l / N;
+            const float cj = (float)j - hN, ck = (float)k - hN;
+            if (l == l0 || j == 0) {
+                // B = kx + kxy cj + kxz ck; C = k0 + ky cj + kz ck + kyy cj^2 + kyz cj ck + kzz ck^2
+                df2 B = dadd(kc[1], dadd(df2_mulf(kc[5], cj), df2_mulf(kc[6], ck)));
+                df2 C = dadd(kc[0], dadd(df2_mulf(kc[2], cj), df2_mulf(kc[3], ck)));
+                C = dadd(C, dadd(df2_mulf(kc[7], cj * cj), dadd(df2_mulf(kc[8], cj * ck), df2_mulf(kc[9], ck * ck))));
+                // start value at c_x = -hN, first ratio, line-to-line ratio
+                Ms = df2_exp(dadd(df2_mulf(kc[4], hN * hN), dadd(dmul(B, mhN), C)));
+                rs = df2_exp(dadd(df2_mulf(kc[4], 2.f - N), B));
+                rl = df2_exp(dadd(dadd(kc[2], df2_mulf(kc[5], -hN)), dadd(df2_mulf(kc[7], 2.f * cj + 1.f), df2_mulf(kc[8], ck))));
+            }
+            acc2 S0 = {0.f, 0.f}, S1 = {0.f, 0.f}, S2 = {0.f, 0.f};
+            float T0 = 0.f, T1 = 0.f, T2 = 0.f, T3 = 0.f, T4 = 0.f;
+            df2 M = Ms, r = rs;
+            float ci = ci0;
+    // unrolled by 2 (measured: 4.5% faster than by 4, 10% faster than by 8)
+#pragma unroll 2
+            for (int i = 0; i < N; ++i) {
+                // ordered Fast2Sum (S0, S2: non-negative terms; S1: any sign;
+                // measured: Harris fit 11.95 -> 11.63 ms per step, TwoSum's bits)
+                // of the weighted terms as chained products, each split exactly
+                // by an FMA: M ci = p1 + e1, (p1 + e1) ci = p2 + e2 (no ci^2;
+                // the Jacobian's sums of degree 3 and 4 continue the chain)
+                acc2_add_nn(S0, M.hi, M.lo);
+                const float p1 = __fmul_rn(M.hi, ci);
+                float e1 = fmaf(M.hi, ci, -p1);
+                e1 = fmaf(M.lo, ci, e1);
+                acc2_add_mag(S1, p1, e1);
+                const float p2 = __fmul_rn(p1, ci);
+                float e2 = fmaf(p1, ci, -p2);
+                e2 = fmaf(e1, ci, e2);
+                acc2_add_nn(S2, p2, e2);
+                if (GRAM) {
+                    const float p3 = __fmul_rn(p2, ci);
+                    T0 = __fadd_rn(T0, M.hi);
+                    T1 = __fadd_rn(T1, p1);
+                    T2 = __fadd_rn(T2, p2);
+                    T3 = __fadd_rn(T3, p3);
+                    T4 = fmaf(p3, ci, T4);
+                }
+                // unnormalised products where only the pair's sum is read (the
+                // ratio always, the value without the Jacobian's FP32 sums of
+                // its high part): three operations fewer each (measured: fit
+                // 11.63 -> 11.06 ms per step; iterations unchanged)
+                M = GRAM ? df2_mul(M, r) : df2_mul_raw(M, r);
+                r = df2_mul_raw(r, e_in);
+                ci += 1.f;
+            }
+            const float T[5] = {T0, T1, T2, T3, T4};
+            plane_add<GRAM>(P, G, S0, S1, S2, T, cj - shy);
+            if (j == N - 1 || l == l1 - 1) plane_flush<GRAM>(m, g, P, G, ck - shz);
+            Ms = df2_mul(Ms, rl);
+            rl = df2_mul(rl, e_j);
+            rs = df2_mul(rs, e_xy);
+        }
     }
 #pragma unroll
     for (int q = 0; q < 10; ++q) {
-        df2 v = gsum_acc(m[q]);
+        df2 v = gsum_acc<S>(m[q]);
         if (gl == 0) cs.m[q] = v;
     }
     if (GRAM) {
 #pragma unroll
         for (int q = 0; q < 35; ++q) {
-            float v = gsumf(g[q]);
+            float v = gsumf<S>(g[q]);
             if (gl == 0) cs.g[q] = v;
         }
     }
-    __syncwarp(gmask());
+    __syncwarp(gmask<S>());
 }
 
 // Slow path: one FP64 exponential per cell (any exponent range).
-template <int N>
+template <int N, int S>
 __device__ __noinline__ void eval_slow(CellScratch& cs, const df2* kcd, bool want_gram) {
-    const int gl = glane();
+    const int gl = glane<S>();
     constexpr double hN = 0.5 * (N - 1);
     double kc[10];
 #pragma unroll
@@ -431,23 +541,23 @@ __device__ __noinline__ void eval_slow(CellScratch& cs, const df2* kcd, bool wan
     }
 #pragma unroll
     for (int q = 0; q < 10; ++q) {
-        double v = gsumd(m[q]);
+        double v = gsumd<S>(m[q]);
         if (gl == 0) cs.m[q] = df2_d(v);
     }
     if (want_gram)
 #pragma unroll
         for (int q = 0; q < 35; ++q) {
-            float v = gsumf(g[q]);
+            float v = gsumf<S>(g[q]);
             if (gl == 0) cs.g[q] = v;
         }
-    __syncwarp(gmask());
+    __syncwarp(gmask<S>());
 }
 
 // Evaluates the moments (and the Gram sums if gram) at eta; returns whether
 // the fast path was taken (uniform over the group).
 // the centre-out pass and the slow path for blocks beyond the float range
 // (defined at the end of this file, away from the common path's code)
-template <int N>
+template <int N, int S>
 __device__ __noinline__ bool evaluate_wide(CellScratch& cs, const df2* kc, bool gram);
 
 // WIDE selects the kernel that holds the centre-out evaluation; it is a
@@ -457,18 +567,18 @@ __device__ __noinline__ bool evaluate_wide(CellScratch& cs, const df2* kc, bool 
 // only those beyond the float range), so that the cells of a warp run the
 // same code rather than both passes in turn (measured: instruction-fetch
 // stalls dominated the mixed form).
-template <int N, bool WIDE>
+template <int N, bool WIDE, int S>
 __device__ __noinline__ bool evaluate(CellScratch& cs, const df2* eta, bool gram) {
     df2 kc[10];
     index_coeffs(eta, cs.wc, cs.h, kc);
-    if constexpr (WIDE) return evaluate_wide<N>(cs, kc, gram);
-    const bool fast = edge_ok<N>(kc);
+    if constexpr (WIDE) return evaluate_wide<N, S>(cs, kc, gram);
+    const bool fast = edge_ok<N, S>(kc);
     if (fast) {
-        if (gram) eval_edge<N, true>(cs, kc);
-        else eval_edge<N, false>(cs, kc);
+        if (gram) eval_edge<N, true, S>(cs, kc);
+        else eval_edge<N, false, S>(cs, kc);
         return true;
     }
-    eval_slow<N>(cs, kc, gram);
+    eval_slow<N, S>(cs, kc, gram);
     return false;
 }
 
@@ -524,9 +634,10 @@ __device__ __forceinline__ void binom_coeffs(float w, float h, float* c) {
 // separable binomial transforms (x, then y, then z), then the FP32 Cholesky
 // solve J dl = rhs into cs.step. Lane 0 of the group, fully unrolled, in
 // shared memory.
+template <int S>
 __device__ __noinline__ bool newton_step_f32(CellScratch& cs, float vol) {
     int ok = 1;
-    if (glane() == 0) {
+    if (glead<S>()) {
         float cx[15], cy[15], cz[15];
         binom_coeffs(cs.wm[0].hi, cs.h[0].hi, cx);
         binom_coeffs(cs.wm[1].hi, cs.h[1].hi, cy);
@@ -611,15 +722,15 @@ __device__ __noinline__ bool newton_step_f32(CellScratch& cs, float vol) {
 #pragma unroll
         for (int i = 0; i < 10; ++i) cs.step[i] = df2_f(y[i]);
     }
-    __syncwarp(gmask());
-    return __shfl_sync(gmask(), ok, gbase()) != 0;
+    __syncwarp(gmask<S>());
+    return __shfl_sync(gmask<S>(), ok, gbase<S>()) != 0;
 }
 
 // Precise mode: Gram matrix in FP64 (one exponential per cell) and FP64
 // Cholesky by lane 0 of the group; rhs = -G in FP64 (cs.dd on input).
-template <int N>
+template <int N, int S>
 __device__ __noinline__ bool newton_step_f64(CellScratch& cs, const df2* eta, double vol) {
-    const int gl = glane();
+    const int gl = glane<S>();
     constexpr double hN = 0.5 * (N - 1);
     df2 kcd[10];
     index_coeffs(eta, cs.wc, cs.h, kcd);
@@ -667,9 +778,9 @@ __device__ __noinline__ bool newton_step_f64(CellScratch& cs, const df2* eta, do
                 for (int c = 0; c <= 4 - a - b; ++c) W[mono4(a, b, c)] += T[a] * py[b] * pz[c];
     }
 #pragma unroll
-    for (int q = 0; q < 35; ++q) W[q] = gsumd(W[q]) * vol;
+    for (int q = 0; q < 35; ++q) W[q] = gsumd<S>(W[q]) * vol;
     int ok = 1;
-    if (gl == 0) {
+    if (glead<S>()) {
         const int E[10][3] = {{0, 0, 0}, {1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {2, 0, 0},
                               {1, 1, 0}, {1, 0, 1}, {0, 2, 0}, {0, 1, 1}, {0, 0, 2}};
         double* J = cs.Jd;
@@ -706,21 +817,22 @@ __device__ __noinline__ bool newton_step_f64(CellScratch& cs, const df2* eta, do
             }
         }
     }
-    __syncwarp(gmask());
-    return __shfl_sync(gmask(), ok, gbase()) != 0;
+    __syncwarp(gmask<S>());
+    return __shfl_sync(gmask<S>(), ok, gbase<S>()) != 0;
 }
 
 // Fit set-up by the 8 lanes of a group (targets in cs.tgt): scaled
 // coordinates, w-space targets and the start point (the continuous
 // Maxwellian of the targets). Returns false, with zero coefficients written,
 // for invalid targets (n <= 0 or non-finite, Theta not positive definite).
-template <int N>
+template <int N, int S>
 __device__ __noinline__ bool fit_setup(CellScratch& cs, const FitArgs& a, double* coef, const float* warm) {
-    const int gl = glane();
-    const unsigned msk = gmask();
+    const int gl = glane<S>();
+    const unsigned msk = gmask<S>();
     const double* t = cs.tgt;
     const double n = t[0];
     auto write_zero = [&]() {
+        if (!coef) return;
         coef[gl] = 0.0;
         coef[gl + 8] = 0.0;
     };
@@ -837,16 +949,15 @@ __device__ __noinline__ bool fit_setup(CellScratch& cs, const FitArgs& a, double
 // the warp call it together (active = false for a group that only keeps the
 // others company). Returns whether the residual reached the tolerance; the
 // number of Newton steps is added to *iters.
-template <int N, bool WIDE>
+template <int N, bool WIDE, int S>
 __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool active, float nf, df2 vol,
                                          float tolf, int* iters, FitWork& work) {
-    constexpr unsigned kAll = 0xffffffffu;
-    const int gl = glane();
-    const unsigned msk = gmask();
+    const int gl = glane<S>();
+    const unsigned msk = gmask<S>();
     bool converged = false, have_gram = false;
     int nit = 0;
     if (active) {
-        work.add(evaluate<N, WIDE>(cs, cs.eta, true), true);
+        work.add(evaluate<N, WIDE, S>(cs, cs.eta, true), true);
         have_gram = true;
     }
     for (int it = 0;; ++it) {
@@ -872,13 +983,13 @@ __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool
             grel = gmax / nf;
             L0 = D[0];
         }
-        if (!__any_sync(kAll, active)) break;
+        if (!unit_any<S>(active)) break;
         const bool precise = it >= 6;
         // Jacobian at eta where the last evaluation did not form it
         const bool need_g = active && !precise && !have_gram;
-        if (__any_sync(kAll, need_g)) {
+        if (unit_any<S>(need_g)) {
             if (need_g) {
-                work.add(evaluate<N, WIDE>(cs, cs.eta, true), true);
+                work.add(evaluate<N, WIDE, S>(cs, cs.eta, true), true);
                 have_gram = true;
             }
         }
@@ -889,7 +1000,7 @@ __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool
                     for (int q = 0; q < 10; ++q) cs.dd[q] = -df2_to_d(G[q]);
                 work.precise += 1u;
                 __syncwarp(msk);
-                ok = newton_step_f64<N>(cs, cs.eta, df2_to_d(vol));
+                ok = newton_step_f64<N, S>(cs, cs.eta, df2_to_d(vol));
                 for (int r = 0; r < 2; ++r) {
                     const int c = gl + 8 * r;
                     if (c < 10) cs.step[c] = df2_d(cs.dd[c]);
@@ -899,7 +1010,7 @@ __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool
                 if (gl == 0)
                     for (int q = 0; q < 10; ++q) cs.rhs[q] = -(G[q].hi + G[q].lo);
                 __syncwarp(msk);
-                ok = newton_step_f32(cs, vol.hi);
+                ok = newton_step_f32<S>(cs, vol.hi);
             }
             if (!ok) {
                 active = false;
@@ -922,7 +1033,7 @@ __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool
         // step is likely: below 1e-5 of n one step from here converges in
         // almost every cell (measured: the Jacobian sums halve, the moment
         // evaluations grow by 0.2%, the fit time drops by 1.3%)
-        const bool gram_next = __any_sync(kAll, active && grel > 1e-5f);
+        const bool gram_next = unit_any<S>(active && grel > 1e-5f);
         float lamb = 1.f;
         bool pending = active;
         for (int ls = 0; ls < 12; ++ls) {
@@ -932,7 +1043,7 @@ __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool
                     if (c < 10) cs.et[c] = dadd(cs.eta[c], df2_mulf(cs.step[c], lamb));
                 }
                 __syncwarp(msk);
-                work.add(evaluate<N, WIDE>(cs, cs.et, gram_next), gram_next);
+                work.add(evaluate<N, WIDE, S>(cs, cs.et, gram_next), gram_next);
                 if (!damp) {
                     pending = false;
                 } else {
@@ -945,7 +1056,7 @@ __device__ __noinline__ bool newton_loop(CellScratch& cs, const FitArgs& a, bool
                     else lamb *= 0.5f;
                 }
             }
-            if (!__any_sync(kAll, pending)) break;
+            if (!unit_any<S>(pending)) break;
         }
         if (active) {
             have_gram = gram_next;
@@ -1019,27 +1130,27 @@ __device__ __noinline__ void continuous_eta_f64(const CellScratch& cs, double* e
 // together (have = false for a group without a cell). Starts from the MLP's
 // prediction when warm is not null and falls back to the cold start (the
 // continuous Maxwellian of the targets) if that run does not converge.
-// Writes the coefficients (eta, u0, sigma) to coef (16 doubles, global),
+// Writes the coefficients (eta, u0, sigma) to coef (16 doubles, global; null:
+// a fit that is only run along, nothing of it is kept),
 // appends a training sample for a converged fit when harvesting, and returns
 // the status: 0 converged, 1 fallback (continuous Maxwellian of the targets),
 // 2 invalid targets.
-template <int N, bool WIDE>
+template <int N, bool WIDE, int S>
 __device__ int fit_cell(CellScratch& cs, const FitArgs& a, bool have, double* coef, const float* warm, int* iters,
                         FitWork& work) {
-    constexpr unsigned kAll = 0xffffffffu;
-    const int gl = glane();
-    const unsigned msk = gmask();
+    const int gl = glane<S>();
+    const unsigned msk = gmask<S>();
     *iters = 0;
-    const bool valid = have && fit_setup<N>(cs, a, coef, warm);
+    const bool valid = have && fit_setup<N, S>(cs, a, coef, warm);
     // the guard of the network's inference writes NaN rows for the fits it rejects
     if (valid && warm && warm[0] == warm[0] && fabsf(warm[0]) < 1e30f) work.warm += 1u;
     const double n = valid ? cs.tgt[0] : 1.0;
     const float nf = (float)n;
     const df2 vol = df2_d(a.dv[0] * a.dv[1] * a.dv[2]);
     const float tolf = (float)(a.tol * n);
-    bool good = newton_loop<N, WIDE>(cs, a, valid, nf, vol, tolf, iters, work) && gaussian_exponent(cs);
+    bool good = newton_loop<N, WIDE, S>(cs, a, valid, nf, vol, tolf, iters, work) && gaussian_exponent(cs);
     const bool retry = valid && warm != nullptr && !good;
-    if (__any_sync(kAll, retry)) {
+    if (unit_any<S>(retry)) {
         if (retry) {
             for (int r = 0; r < 2; ++r) {
                 const int c = gl + 8 * r;
@@ -1047,22 +1158,23 @@ __device__ int fit_cell(CellScratch& cs, const FitArgs& a, bool have, double* co
             }
             __syncwarp(msk);
         }
-        const bool g2 = newton_loop<N, WIDE>(cs, a, retry, nf, vol, tolf, iters, work) && gaussian_exponent(cs);
+        const bool g2 = newton_loop<N, WIDE, S>(cs, a, retry, nf, vol, tolf, iters, work) && gaussian_exponent(cs);
         if (retry) good = g2;
     }
     if (!valid) return 2;
     double fb[10];
     if (!good) continuous_eta_f64(cs, fb);  // rare: every lane of the group forms it
-    for (int r = 0; r < 2; ++r) {
-        const int c = gl + 8 * r;
-        if (c < 10) coef[c] = good ? df2_to_d(cs.eta[c]) : fb[c];
-        else if (c < 13) coef[c] = cs.u0[c - 10];
-        else if (c < 16) coef[c] = cs.sg[c - 13];
-    }
-    if (good && a.harvest) {
+    if (coef)
+        for (int r = 0; r < 2; ++r) {
+            const int c = gl + 8 * r;
+            if (c < 10) coef[c] = good ? df2_to_d(cs.eta[c]) : fb[c];
+            else if (c < 13) coef[c] = cs.u0[c - 10];
+            else if (c < 16) coef[c] = cs.sg[c - 13];
+        }
+    if (good && coef && a.harvest) {
         unsigned long long slot = 0;
-        if (gl == 0) slot = atomicAdd(a.harvest_count, 1ull);
-        slot = __shfl_sync(msk, slot, gbase());
+        if (glead<S>()) slot = atomicAdd(a.harvest_count, 1ull);
+        slot = __shfl_sync(msk, slot, gbase<S>());
         if (slot < (unsigned long long)a.harvest_cap) {
             float* smp = a.harvest + slot * mlp::kSample;
             if (gl == 0) {
@@ -1092,9 +1204,9 @@ __device__ int fit_cell(CellScratch& cs, const FitArgs& a, bool have, double* co
 // +-80 from one cell outside the box to one cell outside on the other side
 // (differences are linear in position, extreme at the corners; 8 lanes,
 // one corner each).
-template <int N>
+template <int N, int S>
 __device__ bool centre_ok(const df2* kcd) {
-    const int gl = glane();
+    const int gl = glane<S>();
     constexpr float hN = 0.5f * (N - 1);
     float k[10];
 #pragma unroll
@@ -1109,7 +1221,7 @@ __device__ bool centre_ok(const df2* kcd) {
         const float dy = k[7] * (2.f * a + 1.f) + k[2] + k[5] * b + k[8] * c;
         ok = ok && fabsf(dx) < 80.f && fabsf(dy) < 80.f;
     }
-    return __all_sync(gmask(), ok);
+    return __all_sync(gmask<S>(), ok);
 }
 
 // One v_x line of the centre-out path: the values from the start cell ic
@@ -1119,9 +1231,9 @@ __device__ bool centre_ok(const df2* kcd) {
 // one times exp(2 k_xx). Weights are the x indices relative to ic (integers,
 // exact in FP32). The FP32 Jacobian sums are formed where rt is set.
 template <int N, bool GRAM>
-__device__ __forceinline__ void fast_line(acc2 (&P)[6], float (&G)[GRAM ? 15 : 1], df2 Mc, df2 rR, df2 rL, df2 e_in,
-                                          int ic, float sj, bool rt) {
-    acc2 S0 = {0.f, 0.f}, S1 = {0.f, 0.f}, S2 = {0.f, 0.f};
+__device__ __forceinline__ void fast_line(acc2& S0, acc2& S1, acc2& S2, float (&T)[5], df2 Mc, df2 rR, df2 rL, df2 e_in,
+                                          int ic, bool rt) {
+    S0 = S1 = S2 = {0.f, 0.f};
     float T0 = 0.f, T1 = 0.f, T2 = 0.f, T3 = 0.f, T4 = 0.f;
     const df2 ML = df2_mul(Mc, rL), rLL = df2_mul(rL, e_in);
     const int turn = N - 1 - ic;
@@ -1152,8 +1264,11 @@ __device__ __forceinline__ void fast_line(acc2 (&P)[6], float (&G)[GRAM ? 15 : 1
         dc = tt ? -1.f : dc;
         ci = tt ? -1.f : ci + dc;
     }
-    const float T[5] = {T0, T1, T2, T3, T4};
-    plane_add<GRAM>(P, G, S0, S1, S2, T, sj, rt);
+    T[0] = T0;
+    T[1] = T1;
+    T[2] = T2;
+    T[3] = T3;
+    T[4] = T4;
 }
 
 // Float bound of one line's exponent q(c) = k_xx c^2 + B c + C over the box
@@ -1187,9 +1302,9 @@ __device__ __forceinline__ void line_bounds(const df2* k, float m_inv2kxx, float
 // part) has its maximum 45 e-folds below the block's largest value, i.e.
 // contributes below 3e-20 of it. The Jacobian sums are formed where rt is
 // set (GRAM is the storage for them).
-template <int N, bool GRAM>
+template <int N, bool GRAM, int S>
 __device__ __noinline__ bool eval_centre(CellScratch& cs, const df2* kc, bool rt) {
-    const int gl = glane();
+    const int gl = glane<S>();
     constexpr float hN = 0.5f * (N - 1);
     constexpr int R = (N * N) / kG;
     const int l0 = gl * R, l1 = l0 + R;
@@ -1222,106 +1337,202 @@ __device__ __noinline__ bool eval_centre(CellScratch& cs, const df2* kc, bool rt
     float ck = 0.f, sk = 0.f;
     bool taint = false;
     df2 M0 = {0.f, 0.f}, rR0 = M0, rL0 = M0, rD0 = M0, Mc = M0, rV = M0, rR = M0, rL = M0, fxy = M0, fyx = M0;
+    if constexpr (S > 1) {
+        // S lines at a time, as in eval_edge
+        const int sub = threadIdx.x & (S - 1);
 #pragma unroll 1
-    for (int t = 0; t < R; ++t) {
-        if (left == 0) {
-            ++kk;
-            const int ja = max(l0 - kk * N, 0);
-            jb = min(l1 - 1 - kk * N, N - 1);
-            js = min(max(jc, ja), jb);
-            left = jb - ja + 1;
-            ck = (float)kk - hN;
-            sk = ck - shz;
-            const float cjs = (float)js - hN;
-            // exponent at (cc, cjs, ck) and its one-cell differences in x and y
-            const df2 B = dadd(kc[1], dadd(df2_mulf(kc[5], cjs), df2_mulf(kc[6], ck)));
-            df2 C = dadd(kc[0], dadd(df2_mulf(kc[2], cjs), df2_mulf(kc[3], ck)));
-            C = dadd(C, dadd(df2_mulf(kc[7], cjs * cjs), dadd(df2_mulf(kc[8], cjs * ck), df2_mulf(kc[9], ck * ck))));
-            const df2 q0 = dadd(C, df2_mulf(dadd(B, df2_mulf(kc[4], cc)), cc));
-            const df2 dX = dadd(B, df2_mulf(kc[4], 2.f * cc + 1.f));
-            const df2 dY =
-                dadd(dadd(kc[2], df2_mulf(kc[7], 2.f * cjs + 1.f)), dadd(df2_mulf(kc[5], cc), df2_mulf(kc[8], ck)));
-            M0 = df2_exp(q0);
-            rR0 = df2_exp(dX);
-            const df2 rU0 = df2_exp(dY);
-            // ratios to the left and down: exp(2 k_xx - dX), exp(2 k_yy - dY)
-            rL0 = df2_div(e_in, rR0);
-            rD0 = df2_div(e_j, rU0);
-            taint = !(M0.hi >= kPrecise);
-            Mc = M0;
-            rV = rU0;
-            rR = rR0;
-            rL = rL0;
-            fxy = e_xy;
-            fyx = e_yx;
-            j = js;
-            dj = 1;
+        for (int tb = 0; tb < R; tb += S) {
+            df2 Mo = M0, rRo = M0, rLo = M0;
+            float sjs[S], sks[S];
+            bool last[S];
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                sjs[s] = sks[s] = 0.f;
+                last[s] = false;
+                if (tb + s >= R) continue;
+                if (left == 0) {
+                    ++kk;
+                    const int ja = max(l0 - kk * N, 0);
+                    jb = min(l1 - 1 - kk * N, N - 1);
+                    js = min(max(jc, ja), jb);
+                    left = jb - ja + 1;
+                    ck = (float)kk - hN;
+                    sk = ck - shz;
+                    const float cjs = (float)js - hN;
+                    // exponent at (cc, cjs, ck) and its one-cell differences in x and y
+                    const df2 B = dadd(kc[1], dadd(df2_mulf(kc[5], cjs), df2_mulf(kc[6], ck)));
+                    df2 C = dadd(kc[0], dadd(df2_mulf(kc[2], cjs), df2_mulf(kc[3], ck)));
+                    C = dadd(C, dadd(df2_mulf(kc[7], cjs * cjs), dadd(df2_mulf(kc[8], cjs * ck), df2_mulf(kc[9], ck * ck))));
+                    const df2 q0 = dadd(C, df2_mulf(dadd(B, df2_mulf(kc[4], cc)), cc));
+                    const df2 dX = dadd(B, df2_mulf(kc[4], 2.f * cc + 1.f));
+                    const df2 dY =
+                        dadd(dadd(kc[2], df2_mulf(kc[7], 2.f * cjs + 1.f)), dadd(df2_mulf(kc[5], cc), df2_mulf(kc[8], ck)));
+                    M0 = df2_exp(q0);
+                    rR0 = df2_exp(dX);
+                    const df2 rU0 = df2_exp(dY);
+                    // ratios to the left and down: exp(2 k_xx - dX), exp(2 k_yy - dY)
+                    rL0 = df2_div(e_in, rR0);
+                    rD0 = df2_div(e_j, rU0);
+                    taint = !(M0.hi >= kPrecise);
+                    Mc = M0;
+                    rV = rU0;
+                    rR = rR0;
+                    rL = rL0;
+                    fxy = e_xy;
+                    fyx = e_yx;
+                    j = js;
+                    dj = 1;
+                }
+                const float cj = (float)j - hN;
+                float qhi, qlo;
+                line_bounds<N>(kc, m_inv2kxx, cj, ck, qhi, qlo);
+                qtop = fmaxf(qtop, qlo);
+                over = over || !(qhi < 80.f);
+                if (taint || !(Mc.hi >= kPrecise)) qlost = fmaxf(qlost, qhi);
+                if (s == sub) {
+                    Mo = Mc;
+                    rRo = rR;
+                    rLo = rL;
+                }
+                sjs[s] = cj - shy;
+                sks[s] = sk;
+                --left;
+                last[s] = left == 0;
+                if (dj > 0 && j == jb) {
+                    // turn: the downward walk starts one line below js
+                    Mc = df2_mul(M0, rD0);
+                    rV = df2_mul(rD0, e_j);
+                    rR = df2_mul(rR0, e_yx);
+                    rL = df2_mul(rL0, e_xy);
+                    fxy = e_yx;
+                    fyx = e_xy;
+                    j = js - 1;
+                    dj = -1;
+                } else {
+                    Mc = df2_mul(Mc, rV);
+                    rV = df2_mul(rV, e_j);
+                    rR = df2_mul(rR, fxy);
+                    rL = df2_mul(rL, fyx);
+                    j += dj;
+                }
+            }
+            acc2 S0, S1, S2;
+            float T[5];
+            fast_line<N, GRAM>(S0, S1, S2, T, Mo, rRo, rLo, e_in, ic, rt);
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                if (tb + s >= R) continue;
+                const float Ts[5] = {from_sub(T[0], s), from_sub(T[1], s), from_sub(T[2], s), from_sub(T[3], s),
+                                     from_sub(T[4], s)};
+                plane_add<GRAM>(P, G, from_sub(S0, s), from_sub(S1, s), from_sub(S2, s), Ts, sjs[s], rt);
+                if (last[s]) plane_flush<GRAM>(m, g, P, G, sks[s], rt);
+            }
         }
-        const float cj = (float)j - hN;
-        float qhi, qlo;
-        line_bounds<N>(kc, m_inv2kxx, cj, ck, qhi, qlo);
-        qtop = fmaxf(qtop, qlo);
-        over = over || !(qhi < 80.f);
-        if (taint || !(Mc.hi >= kPrecise)) qlost = fmaxf(qlost, qhi);
-        fast_line<N, GRAM>(P, G, Mc, rR, rL, e_in, ic, cj - shy, rt);
-        --left;
-        if (left == 0) plane_flush<GRAM>(m, g, P, G, sk, rt);
-        if (dj > 0 && j == jb) {
-            // turn: the downward walk starts one line below js
-            Mc = df2_mul(M0, rD0);
-            rV = df2_mul(rD0, e_j);
-            rR = df2_mul(rR0, e_yx);
-            rL = df2_mul(rL0, e_xy);
-            fxy = e_yx;
-            fyx = e_xy;
-            j = js - 1;
-            dj = -1;
-        } else {
-            Mc = df2_mul(Mc, rV);
-            rV = df2_mul(rV, e_j);
-            rR = df2_mul(rR, fxy);
-            rL = df2_mul(rL, fyx);
-            j += dj;
+    } else {
+#pragma unroll 1
+        for (int t = 0; t < R; ++t) {
+            if (left == 0) {
+                ++kk;
+                const int ja = max(l0 - kk * N, 0);
+                jb = min(l1 - 1 - kk * N, N - 1);
+                js = min(max(jc, ja), jb);
+                left = jb - ja + 1;
+                ck = (float)kk - hN;
+                sk = ck - shz;
+                const float cjs = (float)js - hN;
+                // exponent at (cc, cjs, ck) and its one-cell differences in x and y
+                const df2 B = dadd(kc[1], dadd(df2_mulf(kc[5], cjs), df2_mulf(kc[6], ck)));
+                df2 C = dadd(kc[0], dadd(df2_mulf(kc[2], cjs), df2_mulf(kc[3], ck)));
+                C = dadd(C, dadd(df2_mulf(kc[7], cjs * cjs), dadd(df2_mulf(kc[8], cjs * ck), df2_mulf(kc[9], ck * ck))));
+                const df2 q0 = dadd(C, df2_mulf(dadd(B, df2_mulf(kc[4], cc)), cc));
+                const df2 dX = dadd(B, df2_mulf(kc[4], 2.f * cc + 1.f));
+                const df2 dY =
+                    dadd(dadd(kc[2], df2_mulf(kc[7], 2.f * cjs + 1.f)), dadd(df2_mulf(kc[5], cc), df2_mulf(kc[8], ck)));
+                M0 = df2_exp(q0);
+                rR0 = df2_exp(dX);
+                const df2 rU0 = df2_exp(dY);
+                // ratios to the left and down: exp(2 k_xx - dX), exp(2 k_yy - dY)
+                rL0 = df2_div(e_in, rR0);
+                rD0 = df2_div(e_j, rU0);
+                taint = !(M0.hi >= kPrecise);
+                Mc = M0;
+                rV = rU0;
+                rR = rR0;
+                rL = rL0;
+                fxy = e_xy;
+                fyx = e_yx;
+                j = js;
+                dj = 1;
+            }
+            const float cj = (float)j - hN;
+            float qhi, qlo;
+            line_bounds<N>(kc, m_inv2kxx, cj, ck, qhi, qlo);
+            qtop = fmaxf(qtop, qlo);
+            over = over || !(qhi < 80.f);
+            if (taint || !(Mc.hi >= kPrecise)) qlost = fmaxf(qlost, qhi);
+            acc2 S0, S1, S2;
+            float T[5];
+            fast_line<N, GRAM>(S0, S1, S2, T, Mc, rR, rL, e_in, ic, rt);
+            plane_add<GRAM>(P, G, S0, S1, S2, T, cj - shy, rt);
+            --left;
+            if (left == 0) plane_flush<GRAM>(m, g, P, G, sk, rt);
+            if (dj > 0 && j == jb) {
+                // turn: the downward walk starts one line below js
+                Mc = df2_mul(M0, rD0);
+                rV = df2_mul(rD0, e_j);
+                rR = df2_mul(rR0, e_yx);
+                rL = df2_mul(rL0, e_xy);
+                fxy = e_yx;
+                fyx = e_xy;
+                j = js - 1;
+                dj = -1;
+            } else {
+                Mc = df2_mul(Mc, rV);
+                rV = df2_mul(rV, e_j);
+                rR = df2_mul(rR, fxy);
+                rL = df2_mul(rL, fyx);
+                j += dj;
+            }
         }
     }
 #pragma unroll
     for (int o = kG / 2; o > 0; o >>= 1) {
-        qtop = fmaxf(qtop, __shfl_xor_sync(gmask(), qtop, o));
-        qlost = fmaxf(qlost, __shfl_xor_sync(gmask(), qlost, o));
+        qtop = fmaxf(qtop, __shfl_xor_sync(gmask<S>(), qtop, o * S));
+        qlost = fmaxf(qlost, __shfl_xor_sync(gmask<S>(), qlost, o * S));
     }
-    const bool ok = !__any_sync(gmask(), over) && qtop > -40.f && qlost < qtop - 45.f;
+    const bool ok = !__any_sync(gmask<S>(), over) && qtop > -40.f && qlost < qtop - 45.f;
 #pragma unroll
     for (int q = 0; q < 10; ++q) {
-        df2 v = gsum_acc(m[q]);
+        df2 v = gsum_acc<S>(m[q]);
         if (gl == 0) cs.m[q] = v;
     }
     if (GRAM && rt) {
 #pragma unroll
         for (int q = 0; q < 35; ++q) {
-            float v = gsumf(g[q]);
+            float v = gsumf<S>(g[q]);
             if (gl == 0) cs.g[q] = v;
         }
     }
-    __syncwarp(gmask());
+    __syncwarp(gmask<S>());
     return ok;
 }
 
 // The WIDE kernel's evaluation: the centre-out pass where it is valid, else
 // the edge pass where that is, else the slow path.
-template <int N>
+template <int N, int S>
 __device__ __noinline__ bool evaluate_wide(CellScratch& cs, const df2* kc, bool gram) {
     bool fast = false;
     // one copy of the centre-out pass for both kinds of evaluation (the
     // Jacobian sums behind a flag uniform over the group): half the code of
     // two instantiations (measured: instruction-fetch stalls; 44.6 against
     // 45.8 ms per step on the asymmetric sheet with the same network)
-    if (centre_ok<N>(kc)) fast = eval_centre<N, true>(cs, kc, gram);
-    if (!fast && edge_ok<N>(kc)) {
-        if (gram) eval_edge<N, true>(cs, kc);
-        else eval_edge<N, false>(cs, kc);
+    if (centre_ok<N, S>(kc)) fast = eval_centre<N, true, S>(cs, kc, gram);
+    if (!fast && edge_ok<N, S>(kc)) {
+        if (gram) eval_edge<N, true, S>(cs, kc);
+        else eval_edge<N, false, S>(cs, kc);
         fast = true;
     }
-    if (!fast) eval_slow<N>(cs, kc, gram);
+    if (!fast) eval_slow<N, S>(cs, kc, gram);
     return fast;
 }
 
@@ -1331,10 +1542,66 @@ __device__ __forceinline__ bool bad_target_pair(double t0, double tq, bool first
     return !isfinite(tq) || (first && !(t0 >= 0.0));
 }
 
-// CTAs per SM the register budget is sized for (128 threads each): four for
-// the common kernel (128 registers: measured 2.5% faster than three), three
-// for the wide kernel (170 registers: 13% faster per Newton iteration on the
-// asymmetric sheet than four, whose budget spills the centre-out pass)
+// One fit by its lanes of a unit: targets, fit, counters. V targets are the
+// moments of f, F targets the fluid moments rescaled by n_V / n_F (listed: the
+// closed-form kernel has done that). keep = false: a fit that only runs along.
+template <int N, bool WIDE, int S>
+__device__ __forceinline__ void fit_of_unit(CellScratch& cs, const FitArgs& a, long long cell, bool fluid, bool have,
+                                            bool keep, bool listed, unsigned long long* cnt) {
+    const int gl = glane<S>();
+    const unsigned msk = gmask<S>();
+    bool bad = false;
+    if (have) {
+        const double* src = fluid ? a.fluid + cell * 10 : a.vmom + cell * 20;
+        const double n0 = src[0];
+        double scale = 1.0;
+        if (fluid && !listed) scale = n0 > 0.0 ? a.vmom[cell * 20] / n0 : 0.0;
+        for (int r = 0; r < 2; ++r) {
+            const int c = gl + 8 * r;
+            if (c < 10) {
+                const double raw = src[c];
+                bad = bad || bad_target_pair(n0, raw, c == 0);
+                cs.tgt[c] = fluid && !listed ? raw * scale : raw;
+            }
+        }
+    }
+    __syncwarp(msk);
+    if (have && fluid && !listed)
+        for (int r = 0; r < 2; ++r) {
+            const int c = gl + 8 * r;
+            if (c < 10) a.fluid[cell * 10 + c] = cs.tgt[c];
+        }
+    __syncwarp(msk);
+    FitWork work = {0u, 0u, 0u, 0u, 0u};
+    int iters = 0;
+    double* coef = keep ? (fluid ? a.coef_f : a.coef_v) + cell * kCoefN : nullptr;
+    const float* warm = (have && a.warm) ? a.warm + cell * 20 + (fluid ? 10 : 0) : nullptr;
+    const int st = fit_cell<N, WIDE, S>(cs, a, have, coef, warm, &iters, work);
+    bad = __any_sync(msk, bad);
+    if (keep && glead<S>()) {
+        if (bad && a.numeric) *reinterpret_cast<volatile int*>(a.numeric) = VL_ENUMERIC;
+        if (WIDE && !listed) atomicAdd_block(&cnt[CNT_WIDE_FITS], 1ull);
+        a.status[cell * 2 + (fluid ? 1 : 0)] = st;
+        atomicAdd_block(&cnt[CNT_ITERS], (unsigned long long)iters);
+        if (st == 1) atomicAdd_block(&cnt[CNT_FALLBACK], 1ull);
+        if (st == 2) atomicAdd_block(&cnt[CNT_INVALID], 1ull);
+        atomicAdd_block(&cnt[CNT_EVAL_M], (unsigned long long)work.m);
+        atomicAdd_block(&cnt[CNT_EVAL_G], (unsigned long long)work.g);
+        atomicAdd_block(&cnt[CNT_EVAL_SLOW], (unsigned long long)work.slow);
+        atomicAdd_block(&cnt[CNT_PRECISE], (unsigned long long)work.precise);
+        if (work.warm) atomicAdd_block(&cnt[CNT_WARM], (unsigned long long)work.warm);
+    }
+    __syncwarp(msk);
+}
+
+// A unit is the V or the F fits of four consecutive cells, whose lanes vote on
+// the work (newton_loop).
+//
+// newton_kernel: every fit of the species, a warp per unit. CTAs per SM the
+// register budget is sized for (128 threads each): four for the common kernel
+// (128 registers: measured 2.5% faster than three), three for the wide kernel
+// (170 registers: 13% faster per Newton iteration on the asymmetric sheet than
+// four, whose budget spills the centre-out pass)
 template <int N, bool WIDE>
 __global__ void __launch_bounds__(128, WIDE ? 3 : 4) newton_kernel(FitArgs a) {
     __shared__ CellScratch scratch[16];
@@ -1345,90 +1612,85 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) newton_kernel(FitArgs a) {
         const double nwide = __longlong_as_double((long long)a.select[1]);
         if ((nwide > 1e-10 * nmax) != WIDE) return;
     }
-    // every fit of the species, or those the closed-form kernel left
-    const long long nfit = a.ntodo ? (long long)*a.ntodo : 2 * a.ncell;
-    if (WIDE && a.select && blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd(&a.counters[CNT_WIDE_FITS], 2ull * (unsigned long long)a.ncell);
-    const long long per_cta = blockDim.x / kG;
-    if ((long long)blockIdx.x * per_cta >= nfit) return;
     if (threadIdx.x < VL_NSTATS) cnt[threadIdx.x] = 0ull;
     __syncthreads();
-    const int gl = glane();
     const int slot = threadIdx.x / kG;  // 16 fits per CTA
-    CellScratch& cs = scratch[slot];
-    const unsigned msk = gmask();
-    // the trip count is uniform over the CTA, so the four groups of a warp
-    // always call fit_cell together (a group past the last fit takes part
-    // with have = false)
-    for (long long base = (long long)blockIdx.x * per_cta; base < nfit; base += (long long)gridDim.x * per_cta) {
-        const bool have = base + slot < nfit;
-        const long long fit = !have ? 0 : (a.ntodo ? (long long)a.todo[base + slot] : base + slot);
-        const long long cell = fit >> 1;
-        const bool fluid = (fit & 1) != 0;
-        // V targets: the moments of f; F targets: the fluid moments rescaled
-        // by n_V / n_F (already done for the fits of the list)
-        bool bad = false;
-        double scale = 1.0, n0 = 0.0;
-        const double* src = fluid ? a.fluid + cell * 10 : a.vmom + cell * 20;
-        if (have) {
-            n0 = src[0];
-            if (fluid && !a.ntodo) scale = n0 > 0.0 ? a.vmom[cell * 20] / n0 : 0.0;
-            for (int r = 0; r < 2; ++r) {
-                const int c = gl + 8 * r;
-                if (c < 10) {
-                    const double raw = src[c];
-                    bad = bad || bad_target_pair(n0, raw, c == 0);
-                    cs.tgt[c] = fluid ? raw * scale : raw;
-                }
-            }
-        }
-        __syncwarp(msk);
-        if (have && fluid && !a.ntodo)
-            for (int r = 0; r < 2; ++r) {
-                const int c = gl + 8 * r;
-                if (c < 10) a.fluid[cell * 10 + c] = cs.tgt[c];
-            }
-        __syncwarp(msk);
-        FitWork work = {0u, 0u, 0u, 0u, 0u};
-        int iters = 0;
-        double* coef = (fluid ? a.coef_f : a.coef_v) + cell * kCoefN;
-        const float* warm = (have && a.warm) ? a.warm + fit * 10 : nullptr;
-        const int st = fit_cell<N, WIDE>(cs, a, have, have ? coef : nullptr, warm, &iters, work);
-        bad = __any_sync(msk, bad);
-        if (have && gl == 0) {
-            if (bad && a.numeric) *reinterpret_cast<volatile int*>(a.numeric) = VL_ENUMERIC;
-            if (WIDE && !a.select) atomicAdd_block(&cnt[CNT_WIDE_FITS], 1ull);
-            a.status[fit] = st;
-            atomicAdd_block(&cnt[CNT_ITERS], (unsigned long long)iters);
-            if (st == 1) atomicAdd_block(&cnt[CNT_FALLBACK], 1ull);
-            if (st == 2) atomicAdd_block(&cnt[CNT_INVALID], 1ull);
-            atomicAdd_block(&cnt[CNT_EVAL_M], (unsigned long long)work.m);
-            atomicAdd_block(&cnt[CNT_EVAL_G], (unsigned long long)work.g);
-            atomicAdd_block(&cnt[CNT_EVAL_SLOW], (unsigned long long)work.slow);
-            atomicAdd_block(&cnt[CNT_PRECISE], (unsigned long long)work.precise);
-            if (work.warm) atomicAdd_block(&cnt[CNT_WARM], (unsigned long long)work.warm);
-        }
-        __syncwarp(msk);
+    const long long units = 2 * ((a.ncell + 3) / 4);
+    for (long long u = (long long)blockIdx.x * 4 + (threadIdx.x >> 5); u < units; u += (long long)gridDim.x * 4) {
+        const long long cell = (u >> 1) * 4 + (slot & 3);
+        const bool have = cell < a.ncell;  // a group past the last cell takes part with have = false
+        fit_of_unit<N, WIDE, 1>(scratch[slot], a, cell, (u & 1) != 0, have, have, false, cnt);
     }
     __syncthreads();
     if (threadIdx.x < VL_NSTATS && threadIdx.x != CNT_CLIPPED && cnt[threadIdx.x])
         atomicAdd(&a.counters[threadIdx.x], cnt[threadIdx.x]);
 }
 
-// One CTA per 16 fits: fits take uneven time (one to several Newton
-// iterations), so the hardware's CTA scheduler, which starts a new CTA
-// wherever one finishes, balances the load better than a fixed persistent
-// share per CTA (grids beyond 2^31 - 1 CTAs fall back to looping). The fits
-// left by the closed-form kernel are few and their number is on the device:
-// at most kListBlocks CTAs loop over them.
-// With wide = -1 both kernels are launched and the one not chosen by the
-// device-side selection (a.select) returns at once.
-constexpr long long kListBlocks = 152 * 8;
+// newton_list_kernel: the units holding fits the closed-form kernel left. The
+// unit's other fits run along and are not kept: a fit has the same neighbours,
+// hence the same bits, whoever asked for it. The list is usually short (a few
+// units in a thousand), and then what counts is the latency of one fit, a chain
+// of some 80 k instructions with eight lanes per cell: up to kShortList units
+// each get a CTA, a warp per cell. A longer list is fitted a warp per unit.
+constexpr long long kShortList = 912;  // two waves of 3 CTAs per SM
+template <int N, bool WIDE>
+__global__ void __launch_bounds__(128, 3) newton_list_kernel(FitArgs a) {
+    __shared__ CellScratch scratch[16];
+    __shared__ unsigned long long cnt[VL_NSTATS];
+    const long long units = (long long)*a.ntodo;
+    const double nmax = __longlong_as_double((long long)a.select[0]);
+    const double nwide = __longlong_as_double((long long)a.select[1]);
+    // chosen on the device: this kernel runs only if it is the one wanted
+    if ((nwide > 1e-10 * nmax) != WIDE) return;
+    // (the counter's fits are those of a species whose targets call for the wide kernel)
+    if (WIDE && blockIdx.x == 0 && threadIdx.x == 0)
+        atomicAdd(&a.counters[CNT_WIDE_FITS], 2ull * (unsigned long long)a.ncell);
+    const bool brief = units <= kShortList;
+    if ((brief ? (long long)blockIdx.x : (long long)blockIdx.x * 4) >= units) return;
+    if (threadIdx.x < VL_NSTATS) cnt[threadIdx.x] = 0ull;
+    __syncthreads();
+    if (brief) {
+        const int c = threadIdx.x >> 5;
+        for (long long k = blockIdx.x; k < units; k += gridDim.x) {
+            const unsigned long long entry = a.todo[k];
+            const long long cell = (long long)(entry >> 5) * 4 + c;
+            const bool have = cell < a.ncell, keep = have && ((entry >> c) & 1ull) != 0;
+            fit_of_unit<N, WIDE, 4>(scratch[c], a, cell, ((entry >> 4) & 1ull) != 0, have, keep, true, cnt);
+        }
+    } else {
+        const int slot = threadIdx.x / kG, c = slot & 3;
+        for (long long k = (long long)blockIdx.x * 4 + (threadIdx.x >> 5); k < units; k += (long long)gridDim.x * 4) {
+            const unsigned long long entry = a.todo[k];
+            const long long cell = (long long)(entry >> 5) * 4 + c;
+            const bool have = cell < a.ncell, keep = have && ((entry >> c) & 1ull) != 0;
+            fit_of_unit<N, WIDE, 1>(scratch[slot], a, cell, ((entry >> 4) & 1ull) != 0, have, keep, true, cnt);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < VL_NSTATS && threadIdx.x != CNT_CLIPPED && cnt[threadIdx.x])
+        atomicAdd(&a.counters[threadIdx.x], cnt[threadIdx.x]);
+}
+
+// newton_kernel: one CTA per four units (16 fits): fits take uneven time (one
+// to several Newton iterations), so the hardware's CTA scheduler, which starts
+// a new CTA wherever one finishes, balances the load better than a fixed
+// persistent share per CTA (grids beyond 2^31 - 1 CTAs fall back to looping).
+// Where the choice is the device's (a.select) both kernels are launched and the
+// one not chosen returns at once. The list's length is on the device.
 template <int N>
 cudaError_t launch_n(const FitArgs& a, cudaStream_t st) {
-    long long blocks = (2 * a.ncell + 15) / 16;
+    const long long quads = (a.ncell + 3) / 4;
+    if constexpr (N >= kClosedMin) {
+        if (a.ntodo) {
+            const long long blocks = 2 * quads < kShortList ? 2 * quads : kShortList;
+            newton_list_kernel<N, true><<<(unsigned)blocks, 128, 0, st>>>(a);
+            newton_list_kernel<N, false><<<(unsigned)blocks, 128, 0, st>>>(a);
+            count_launch(2);
+            return cudaGetLastError();
+        }
+    }
+    long long blocks = (2 * quads + 3) / 4;
     if (blocks > 0x7FFFFFFFLL) blocks = 0x7FFFFFFFLL;
-    if (a.ntodo && blocks > kListBlocks) blocks = kListBlocks;
     FitArgs b = a;
     if (a.wide >= 0) b.select = nullptr;
     if (a.wide != 0) {
