@@ -134,8 +134,8 @@ vl_status pfc_advect_x(vl_ctx* ctx, int species, int axis, double dt, vl_stream_
  * the context (the caller may pass it as f_out of the next call). The result
  * is element for element that of pfc_advect_x(x) then pfc_advect_x(y); the
  * same limits apply (VL_EINVAL). Grids whose nx or ny is not a multiple of 8,
- * or whose y shift exceeds 6 cells, take the two single-axis sweeps in place
- * followed by a device copy into f_out, with the same result. */
+ * or whose y shift exceeds 6 cells, take the two single-axis sweeps, the first
+ * in place and the second into f_out, with the same result. */
 vl_status pfc_advect_xy(vl_ctx* ctx, int species, double dt, void* f_out, vl_stream_t stream);
 
 /* Velocity-space PFC advection of species s under (q/m)(E + v x B) over dt

@@ -296,7 +296,8 @@ vl_status vl_sync_status(vl_ctx* ctx, vl_stream_t stream) {
 
 const char* vl_last_error(const vl_ctx* ctx) { return ctx ? ctx->err : g_err; }
 
-vl_status pfc_advect_x(vl_ctx* ctx, int s, int axis, double dt, vl_stream_t stream) {
+// one directional sweep of a species' f into f_out (f itself: in place)
+static vl_status sweep_axis(vl_ctx* ctx, int s, int axis, double dt, void* f_out, vl_stream_t stream) {
     Range nvtx_("pfc_advect_x");
     vl_status st = check_species(ctx, s);
     if (st != VL_OK) return st;
@@ -308,6 +309,7 @@ vl_status pfc_advect_x(vl_ctx* ctx, int s, int axis, double dt, vl_stream_t stre
     const int es = d.precision == 64 ? 8 : 4;
     vl::SpaceSweepArgs a;
     a.f = ctx->f[s];
+    a.f_out = f_out ? f_out : ctx->f[s];
     a.V = V;
     a.nvx = d.nv[s][0];
     a.nvy = d.nvdim == 3 ? d.nv[s][1] : 1;
@@ -372,6 +374,10 @@ vl_status pfc_advect_x(vl_ctx* ctx, int s, int axis, double dt, vl_stream_t stre
     return cuda_check(ctx, vl::launch_pfc_space(a, d.precision, (cudaStream_t)stream), "pfc_advect_x");
 }
 
+vl_status pfc_advect_x(vl_ctx* ctx, int s, int axis, double dt, vl_stream_t stream) {
+    return sweep_axis(ctx, s, axis, dt, nullptr, stream);
+}
+
 vl_status pfc_advect_xy(vl_ctx* ctx, int s, double dt, void* f_out, vl_stream_t stream) {
     Range nvtx_("pfc_advect_xy");
     vl_status st = check_species(ctx, s);
@@ -434,15 +440,24 @@ vl_status pfc_advect_xy(vl_ctx* ctx, int s, double dt, void* f_out, vl_stream_t 
     const long long ntiles = a.tx && a.ty ? (long long)a.nchunks * (d.nx / a.tx) * (d.ny / a.ty) : 0;
     const bool fused = a.tx && a.ty && a.hy <= 8 && a.hy <= d.ny && ntiles < (1LL << 31);
     cudaStream_t cs = (cudaStream_t)stream;
-    if (fused) {
+    cudaError_t e = cudaErrorNotSupported;
+    if (d.precision == 32 && fused && vl::march_fits(a)) {
+        // Whole 16 x 16 tiles with shifts up to 2 cells add an update's two
+        // products in physical order, other grids in the order of the sweep's
+        // direction: the roundings pfc_advect_xy has had on either kind of
+        // grid, so that a run keeps its bits
+        const bool frame = !(a.hx <= 4 && a.hy <= 4 && d.nx % 16 == 0 && d.ny % 16 == 0);
+        e = vl::launch_pfc_space_march(a, frame, cs);
+    }
+    if (e != cudaErrorNotSupported) {
+        st = cuda_check(ctx, e, "pfc_advect_xy");
+    } else if (fused) {
         st = cuda_check(ctx, vl::launch_pfc_space_xy(a, d.precision, cs), "pfc_advect_xy");
     } else {
-        // grids without 8-cell tiles or with long y shifts: the two in-place
-        // sweeps, then the result moves to f_out
-        st = pfc_advect_x(ctx, s, 0, dt, stream);
-        if (st == VL_OK) st = pfc_advect_x(ctx, s, 1, dt, stream);
-        if (st == VL_OK)
-            st = cuda_check(ctx, cudaMemcpyAsync(f_out, ctx->f[s], bytes, cudaMemcpyDeviceToDevice, cs), "pfc_advect_xy copy");
+        // grids without 8-cell tiles or with long y shifts: the two sweeps,
+        // the second out of place
+        st = sweep_axis(ctx, s, 0, dt, nullptr, stream);
+        if (st == VL_OK) st = sweep_axis(ctx, s, 1, dt, f_out, stream);
     }
     if (st == VL_OK) ctx->f[s] = f_out;
     return st;

@@ -8,6 +8,7 @@ namespace vl {
 // ---- spatial PFC sweep ----------------------------------------------------
 struct SpaceSweepArgs {
     void* f;
+    void* f_out;            // f itself (in place) or a buffer apart from it
     int n;                  // cells along the sweep axis
     long long row_stride;   // elements between neighbouring cells along the line
     long long line_stride;  // elements between neighbouring lines
@@ -67,6 +68,10 @@ struct SpaceXYArgs {
 };
 size_t pfc_space_xy_smem(const SpaceXYArgs& a, int precision);
 cudaError_t launch_pfc_space_xy(const SpaceXYArgs& a, int precision, cudaStream_t st);
+// the streamed form in FP32 (pfc_space_march.cu), any grid; frame: products
+// added in the single-axis sweeps' order. cudaErrorNotSupported: not taken
+bool march_fits(const SpaceXYArgs& a);
+cudaError_t launch_pfc_space_march(const SpaceXYArgs& a, bool frame, cudaStream_t st);
 
 // ---- velocity-space PFC pass (+ fused moments) -----------------------------
 // Centred-index moments -> physical raw moments: out[o] = sum_t coef[o][t] *

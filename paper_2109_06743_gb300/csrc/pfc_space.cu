@@ -113,6 +113,7 @@ template <typename T>
 __global__ void __launch_bounds__(1024) pfc_space_kernel(SpaceSweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* f = reinterpret_cast<T*>(a.f);
+    T* g = reinterpret_cast<T*>(a.f_out);
     const int ncol = a.ncol, n = a.n;
     T* const buf0 = reinterpret_cast<T*>(smem_raw);
     T* const buf1 = buf0 + (size_t)n * ncol;
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(1024) pfc_space_kernel(SpaceSweepArgs a) {
                 T fm1 = fetch(j - 1), f0 = fetch(j), fp1 = fetch(j + 1);
                 T phim = pfc_phi<T>(alpha, A, B, fetch(j - 2), fm1, f0);
                 // output walks the line in the frame's direction
-                T* out = f + base + vi + (long long)(fwd ? k0 : n - 1 - k0) * a.row_stride;
+                T* out = g + base + vi + (long long)(fwd ? k0 : n - 1 - k0) * a.row_stride;
                 const long long os = fwd ? a.row_stride : -a.row_stride;
                 // at step k the window needs the value at frame index k - s + 2:
                 // inside the line for s - 2 <= k <= n - 3 + s, where it is read

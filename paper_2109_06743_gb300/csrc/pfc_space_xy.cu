@@ -20,13 +20,17 @@
 // q - s - 2 and every index below is a compile-time constant; a negative
 // displacement walks the line backwards.
 //
-// Two kernels: pfc_space_xy_tma_kernel (persistent; the input box of a tile,
-// halos included, is one TMA tensor copy into shared memory, issued two tiles
-// ahead into a double buffer and completed on an mbarrier; only the cells a
-// tensor copy cannot express -- periodic images in x and y, mirror rows at a
+// Two kernels: pfc_space_xy_tma_kernel (FP64; persistent; the input box of a
+// tile, halos included, is one TMA tensor copy into shared memory, issued two
+// tiles ahead into a double buffer and completed on an mbarrier; only the cells
+// a tensor copy cannot express -- periodic images in x and y, mirror rows at a
 // wall -- are patched in with plain loads) for x and y shifts up to 2 cells;
 // pfc_space_xy_kernel (one CTA per tile, inputs read straight from global
-// memory) for any shift.
+// memory) for any shift. FP32 calls come here only with an f that is not
+// 16-byte aligned or with x shifts above 6 cells: pfc_space_march.cu takes the
+// rest. In FP64 its march has only one FP64 chain per thread to offer where the
+// FP64 pipe is the bound (128 x 64 x 16^3 1545 us against 1535 here, 100 x 50 x
+// 12^3 538 against 402, 16^2 x 16^3 150 against 63).
 #include <cuda.h>
 
 #include "common.cuh"
@@ -271,15 +275,7 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
 // real copy time; each poll is a bounded hardware wait)
 constexpr uint32_t kCopyWaitPolls = 1u << 20;
 
-#ifndef VL_XY_TX
-#define VL_XY_TX 16
-#endif
-#ifndef VL_XY_TY
-#define VL_XY_TY 16
-#endif
-#ifndef VL_XY_NT
-#define VL_XY_NT 1024
-#endif
+constexpr int kTileX = 16, kTileY = 16;
 
 // Shared memory: [2 mbarriers | pad to 128][S0][S1][xs][x steps][y steps];
 // S = the input box [TY + 2 hy][TX + 2 hx][NCOL] of one tile. The tile
@@ -554,12 +550,12 @@ static cudaError_t launch_xy(const SpaceXYArgs& a, size_t smem, long long ntiles
 }
 
 cudaError_t launch_pfc_space_xy(const SpaceXYArgs& args, int precision, cudaStream_t st) {
-    // TMA path: 32 x 8 tiles, shifts of at most 2 cells, a 16-byte aligned
-    // f_in whose rows are whole multiples of 16 bytes
-    {
+    // FP64 TMA path: shifts of at most 2 cells, a 16-byte aligned f_in whose
+    // rows are whole multiples of 16 bytes
+    if (precision == 64) {
         SpaceXYArgs a = args;
-        a.tx = VL_XY_TX;
-        a.ty = VL_XY_TY;
+        a.tx = kTileX;
+        a.ty = kTileY;
         a.div_nvx = make_fastdiv(a.nvx);
         a.div_nvy = make_fastdiv(a.nvy);
         a.div_ntx = make_fastdiv(a.nx / a.tx > 0 ? a.nx / a.tx : 1);
@@ -574,9 +570,7 @@ cudaError_t launch_pfc_space_xy(const SpaceXYArgs& args, int precision, cudaStre
             const size_t smem = tma_smem(a, precision);
             const long long ntiles = (long long)a.nchunks * (a.nx / a.tx) * (a.ny / a.ty);
             if (smem <= 227 * 1024 && ntiles < (1LL << 31) - (1LL << 20) && a.V < (1LL << 31)) {
-                constexpr int SX = VL_XY_TX < 16 ? VL_XY_TX : 16, SY = VL_XY_TY < 8 ? VL_XY_TY : 8;
-                if (precision == 64) return launch_tma<double, VL_XY_TX, VL_XY_TY, SX, SY, 512>(m, a, smem, ntiles, st);
-                return launch_tma<float, VL_XY_TX, VL_XY_TY, SX, SY, VL_XY_NT>(m, a, smem, ntiles, st);
+                return launch_tma<double, kTileX, kTileY, 16, 8, 512>(m, a, smem, ntiles, st);
             }
         }
     }
