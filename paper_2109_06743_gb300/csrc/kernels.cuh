@@ -93,6 +93,7 @@ struct VelocityArgs {
     int nshear;
     int nbuf;               // block buffers in shared memory (set by the launcher)
     int vec;                // f is 16-byte aligned: write blocks back with 16-byte stores (set by the launcher)
+    unsigned long long* counters;  // null: cells by a fixed stride
     double qm, dt;
     double vmin[3], dv[3];
     MomConv conv;

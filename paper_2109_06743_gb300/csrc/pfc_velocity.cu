@@ -20,10 +20,13 @@
 // FP32 blocks run velocity_pair_kernel (two lines per thread, packed FP32x2
 // arithmetic, every line walked upwards); FP64 blocks run velocity_kernel
 // (one line per thread, walked in the direction of its displacement).
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "block_moments.cuh"
 #include "f32x2.cuh"
+#include "work_queue.cuh"
 
 namespace vl {
 
@@ -362,6 +365,39 @@ __device__ __forceinline__ void store_block_groups(float* dst, const float* blk)
     }
 }
 
+// The same by planes of v_z: warp w copies the planes its lines w 64 .. w 64 + 63
+// lie in, 64 N contiguous values
+template <int N>
+__device__ __forceinline__ void prefetch_planes(float* blk, const float* src) {
+    const int t = threadIdx.x & 31, row = (threadIdx.x >> 5) * 64;
+    const unsigned d = (unsigned)__cvta_generic_to_shared(blk + (row + t / N) * (N + 1) + t % N);
+    const float* g = src + row * N + t;
+#pragma unroll
+    for (int u = 0; u < 2 * N; ++u)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d + 4u * (unsigned)(u * (32 / N) * (N + 1))),
+                     "l"(g + u * 32)
+                     : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void store_planes(float* dst, const float* blk, bool vec) {
+    const int t = threadIdx.x & 31, row = (threadIdx.x >> 5) * 64;
+    if (!vec) {
+        const float* r = blk + (row + t / N) * (N + 1) + t % N;
+        float* g = dst + row * N + t;
+#pragma unroll
+        for (int u = 0; u < 2 * N; ++u) g[u * 32] = r[u * (32 / N) * (N + 1)];
+        return;
+    }
+    const float* r = blk + (row + 4 * t / N) * (N + 1) + (4 * t) % N;
+    float* g = dst + row * N + 4 * t;
+#pragma unroll
+    for (int u = 0; u < N / 2; ++u) {
+        const float* q = r + u * (128 / N) * (N + 1);
+        *reinterpret_cast<float4*>(g + u * 128) = make_float4(q[0], q[1], q[2], q[3]);
+    }
+}
+
 // write the block back; with vec (16-byte aligned f) in 16-byte stores: a
 // row holds N values (N a multiple of 4), so each group of 16 bytes comes
 // from one padded row
@@ -477,7 +513,10 @@ using x2::sub;
 constexpr int threads(int n) { return ((n * n / 2 + 31) / 32) * 32; }
 constexpr int warps(int n) { return threads(n) / 32; }
 // CTAs per SM the register cap is sized for
-constexpr int min_blocks(int n) { return n <= 8 ? 16 : (n <= 12 ? 6 : (n <= 16 ? 5 : 2)); }
+// blocks staged in shared memory, or the first and last sweep straight from and
+// to global memory
+constexpr bool staged(int n) { return n <= 16; }
+constexpr int min_blocks(int n) { return n <= 8 ? 24 : (n <= 12 ? 7 : (n <= 16 ? 5 : (n <= 20 ? 3 : 2))); }
 
 // physical exponents (x, y, z) of moment o, packed x + 4 y + 16 z
 __host__ __device__ constexpr int mono_exp(int o) {
@@ -521,40 +560,24 @@ __device__ __forceinline__ PairCoef pair_coef(float2 c) {
     return k;
 }
 
-// integer part of the displacement of one line: g (the fractional update,
-// both box faces closed) moves s cells in the direction of the displacement,
-// what would leave the box piles up in the last cell, the cells it leaves
-// become zero (the one-dimensional sweep at any displacement, Sec. 2.1)
-template <int N, int ST, int C>
-__device__ __forceinline__ void shift_store(float* line, const float2 (&g)[N], int s, bool fwd) {
-    auto at = [&](int q) -> float { return C == 0 ? g[q].x : g[q].y; };
-    if (s == 0) {
-#pragma unroll
-        for (int q = 0; q < N; ++q) line[q * ST] = at(q);
-        return;
-    }
+// integer part of the displacement of one line, whose values g (the fractional
+// update, both box faces closed) are in place: they move s cells in the direction
+// of the displacement, what would leave the box piles up in the last cell, the
+// cells they leave become zero (the one-dimensional sweep at any displacement,
+// Sec. 2.1). Rare (drifts of a whole velocity cell per step), so it is kept
+// small: the sweeps' code has to stay in the instruction caches.
+template <int N, int ST>
+__device__ __forceinline__ void shift_line(float* line, int s, bool fwd) {
+    if (s == 0) return;
+    // walked from the end the displacement points to: p = 0 is the last cell
+    float* const end = fwd ? line + (N - 1) * ST : line;
+    const int st = fwd ? -ST : ST;
     float acc = 0.0f;
-    if (fwd) {
-#pragma unroll
-        for (int q = 0; q < N; ++q) {
-            if (q + s < N - 1) line[(q + s) * ST] = at(q);
-            else acc += at(q);
-        }
-        line[(N - 1) * ST] = acc;
-#pragma unroll
-        for (int p = 0; p < N - 1; ++p)
-            if (p < s) line[p * ST] = 0.0f;
-    } else {
-#pragma unroll
-        for (int q = N - 1; q >= 0; --q) {
-            if (q - s > 0) line[(q - s) * ST] = at(q);
-            else acc += at(q);
-        }
-        line[0] = acc;
-#pragma unroll
-        for (int p = 1; p < N; ++p)
-            if (p > N - 1 - s) line[p * ST] = 0.0f;
-    }
+#pragma unroll 1
+    for (int p = min(s, N - 1); p >= 0; --p) acc += end[p * st];
+    *end = acc;
+#pragma unroll 1
+    for (int p = 1; p < N; ++p) end[p * st] = p + s < N ? end[(p + s) * st] : 0.0f;
 }
 
 // the 20 raw-moment products of one line along axis AX with centred sums
@@ -576,32 +599,62 @@ __device__ __forceinline__ void line_moments(float (&m)[20], const float (&S)[4]
     }
 }
 
-// One sweep along velocity axis AX over the pair of lines (lo1, hi1),
-// (lo2, hi2) of this thread. RAGGED: some threads hold fewer than two lines
-// (v1, v2 false), their loads give zero and their stores are skipped. MOM:
-// this is the block's last sweep: the 20 moment products of the result are
-// formed from the registers and reduced over the CTA into out.
-template <int N, int AX, bool RAGGED, bool MOM>
-__device__ __forceinline__ void sweep(float* blk, const float* sh, const float* vc, const float* inv_dv, int lo1,
-                                      int hi1, int lo2, int hi2, bool v1, bool v2, float (&m)[20]) {
-    constexpr int ST = AX == 0 ? 1 : (AX == 1 ? N + 1 : N * (N + 1));
-    constexpr int alo = AX == 0 ? 1 : 0, ahi = AX == 2 ? 1 : 2;
-    auto start = [](int lo, int hi) {
-        return AX == 0 ? padded<N>(0, lo, hi) : (AX == 1 ? padded<N>(lo, 0, hi) : padded<N>(lo, hi, 0));
-    };
-    float* const L1 = blk + start(lo1, hi1);
-    float* const L2 = blk + start(lo2, hi2);
-    const float idv = inv_dv[AX];
-    const PairCoef k = pair_coef<N>(make_float2((sh[1] * vc[alo * N + lo1] + sh[2] * vc[ahi * N + hi1] + sh[3]) * idv,
-                                                (sh[1] * vc[alo * N + lo2] + sh[2] * vc[ahi * N + hi2] + sh[3]) * idv));
-    const float2 a0 = k.a0, P = k.P, Q = k.Q, c0 = k.c0, cm = k.cm, cp = k.cp;
-    const bool whole = __ballot_sync(0xffffffffu, (v1 && k.s1 != 0) || (v2 && k.s2 != 0)) != 0u;
-    float2 r[N];
+// where a sweep reads its lines from and writes them to
+enum { SHARED = 0, GLOBAL = 1 };
+// when it forms moments
+enum { NEVER = 0, ALWAYS = 1, ASKED = 2 };
+
+// a line of N values at compile-time stride in global memory; along v_x it is
+// a contiguous row, moved 16 bytes at a time where f allows it
+template <int N, int AX>
+__device__ __forceinline__ int global_start(int lo, int hi) {
+    return AX == 0 ? (hi * N + lo) * N : (AX == 1 ? hi * N * N + lo : hi * N + lo);
+}
+template <int N, int AX, int C>
+__device__ __forceinline__ void load_line(float2 (&r)[N], const float* g, bool vec) {
+    constexpr int ST = AX == 0 ? 1 : (AX == 1 ? N : N * N);
+    auto put = [&](int q, float v) { C == 0 ? r[q].x = v : r[q].y = v; };
+    if (AX == 0 && vec) {
 #pragma unroll
-    for (int q = 0; q < N; ++q) {
-        r[q].x = (!RAGGED || v1) ? L1[q * ST] : 0.0f;
-        r[q].y = (!RAGGED || v2) ? L2[q * ST] : 0.0f;
+        for (int q = 0; q < N / 4; ++q) {
+            const float4 v = reinterpret_cast<const float4*>(g)[q];
+            put(4 * q, v.x);
+            put(4 * q + 1, v.y);
+            put(4 * q + 2, v.z);
+            put(4 * q + 3, v.w);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) put(q, g[q * ST]);
     }
+}
+template <int N, int AX, int C>
+__device__ __forceinline__ void store_line(float* g, const float2 (&r)[N], bool vec) {
+    constexpr int ST = AX == 0 ? 1 : (AX == 1 ? N : N * N);
+    auto at = [&](int q) -> float { return C == 0 ? r[q].x : r[q].y; };
+    if (AX == 0 && vec) {
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q)
+            reinterpret_cast<float4*>(g)[q] = make_float4(at(4 * q), at(4 * q + 1), at(4 * q + 2), at(4 * q + 3));
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) g[q * ST] = at(q);
+    }
+}
+
+// the two lines of a thread and its constant inputs
+struct Lines {
+    int lo1, hi1, lo2, hi2;
+    bool v1, v2;       // which of them exist (RAGGED)
+    bool vec;          // f is 16-byte aligned
+    const float* vc;   // [3][N] cell-centre velocities
+    const float* inv_dv;
+};
+
+// the fractional update of both lines in registers
+template <int N>
+__device__ __forceinline__ void advance(float2 (&r)[N], const PairCoef& k) {
+    const float2 a0 = k.a0, P = k.P, Q = k.Q, c0 = k.c0, cm = k.cm, cp = k.cp;
     float2 a_prev = r[0];  // a_{-1} = f_0 - 0
     float2 ph1 = make_float2(0.0f, 0.0f), ph2 = ph1;  // phi_{q-1}, phi_{q-2}
 #pragma unroll
@@ -619,126 +672,277 @@ __device__ __forceinline__ void sweep(float* blk, const float* sh, const float* 
         a_prev = a;
     }
     r[N - 1] = fma(cm, ph2, fma(neg(cp), ph1, r[N - 1]));
-    if (!whole) {
-#pragma unroll
-        for (int q = 0; q < N; ++q) {
-            if (!RAGGED || v1) L1[q * ST] = r[q].x;
-            if (!RAGGED || v2) L2[q * ST] = r[q].y;
-        }
-    } else {
-        if (!RAGGED || v1) shift_store<N, ST, 0>(L1, r, k.s1, k.f1);
-        if (!RAGGED || v2) shift_store<N, ST, 1>(L2, r, k.s2, k.f2);
-        if (MOM) {
-            // the thread's own stores: read back the shifted lines
-#pragma unroll
-            for (int q = 0; q < N; ++q) {
-                r[q].x = (!RAGGED || v1) ? L1[q * ST] : 0.0f;
-                r[q].y = (!RAGGED || v2) ? L2[q * ST] : 0.0f;
-            }
-        }
-    }
-    if (MOM) {
-        // centred sums S_p = sum_q xi_q^p f_q, xi_q = q - (N-1)/2, folded over
-        // the mirror pairs q, N-1-q (xi_{N-1-q} = -xi_q)
-        float2 s0 = make_float2(0.0f, 0.0f);
-        float S1x = 0.0f, S1y = 0.0f, S2x = 0.0f, S2y = 0.0f, S3x = 0.0f, S3y = 0.0f;
-#pragma unroll
-        for (int q = 0; q < N / 2; ++q) {
-            const float xi = (float)q - 0.5f * (float)(N - 1);
-            const float2 u = add(r[q], r[N - 1 - q]);
-            const float2 d = sub(r[q], r[N - 1 - q]);
-            s0 = add(s0, u);
-            S1x = fmaf(d.x, xi, S1x);
-            S1y = fmaf(d.y, xi, S1y);
-            S2x = fmaf(u.x, xi * xi, S2x);
-            S2y = fmaf(u.y, xi * xi, S2y);
-            S3x = fmaf(d.x, xi * xi * xi, S3x);
-            S3y = fmaf(d.y, xi * xi * xi, S3y);
-        }
-        const float cc = 0.5f * (float)(N - 1);
-        const float Sa[4] = {s0.x, S1x, S2x, S3x}, Sb[4] = {s0.y, S1y, S2y, S3y};
-        line_moments<AX>(m, Sa, (float)lo1 - cc, (float)hi1 - cc);
-        line_moments<AX>(m, Sb, (float)lo2 - cc, (float)hi2 - cc);
-    }
 }
 
-template <int N, bool RAGGED, bool MOM>
-__device__ __forceinline__ void sweep_axis(int axis, float* blk, const float* sh, const float* vc,
-                                           const float* inv_dv, int lo1, int hi1, int lo2, int hi2, bool v1, bool v2,
+// adds the 20 moment products of both lines, from centred sums S_p = sum_q xi_q^p f_q,
+// xi_q = q - (N-1)/2, folded over the mirror pairs q, N-1-q (xi_{N-1-q} = -xi_q)
+template <int N, int AX>
+__device__ __forceinline__ void products(float (&m)[20], const float2 (&r)[N], const Lines& t) {
+    float2 s0 = make_float2(0.0f, 0.0f);
+    float S1x = 0.0f, S1y = 0.0f, S2x = 0.0f, S2y = 0.0f, S3x = 0.0f, S3y = 0.0f;
+#pragma unroll
+    for (int q = 0; q < N / 2; ++q) {
+        const float xi = (float)q - 0.5f * (float)(N - 1);
+        const float2 u = add(r[q], r[N - 1 - q]);
+        const float2 d = sub(r[q], r[N - 1 - q]);
+        s0 = add(s0, u);
+        S1x = fmaf(d.x, xi, S1x);
+        S1y = fmaf(d.y, xi, S1y);
+        S2x = fmaf(u.x, xi * xi, S2x);
+        S2y = fmaf(u.y, xi * xi, S2y);
+        S3x = fmaf(d.x, xi * xi * xi, S3x);
+        S3y = fmaf(d.y, xi * xi * xi, S3y);
+    }
+    const float cc = 0.5f * (float)(N - 1);
+    const float Sa[4] = {s0.x, S1x, S2x, S3x}, Sb[4] = {s0.y, S1y, S2y, S3y};
+    line_moments<AX>(m, Sa, (float)t.lo1 - cc, (float)t.hi1 - cc);
+    line_moments<AX>(m, Sb, (float)t.lo2 - cc, (float)t.hi2 - cc);
+}
+
+// One sweep along velocity axis AX over the pair of lines (lo1, hi1),
+// (lo2, hi2) of this thread, from SRC to DST (blk: the block in shared memory,
+// g: in global memory). RAGGED: some threads hold fewer than two lines (v1, v2
+// false), their loads give zero and their stores are skipped. The 20 moment
+// products of the result are added to m from the registers: MOM NEVER, ALWAYS,
+// or ASKED (if mom).
+template <int N, int AX, bool RAGGED, int SRC, int DST, int MOM>
+__device__ __forceinline__ void sweep(bool mom, float* blk, float* g, const float* sh, const Lines& t, float (&m)[20]) {
+    constexpr int ST = AX == 0 ? 1 : (AX == 1 ? N + 1 : N * (N + 1));
+    constexpr int alo = AX == 0 ? 1 : 0, ahi = AX == 2 ? 1 : 2;
+    auto start = [](int lo, int hi) {
+        return AX == 0 ? padded<N>(0, lo, hi) : (AX == 1 ? padded<N>(lo, 0, hi) : padded<N>(lo, hi, 0));
+    };
+    float* const L1 = blk + start(t.lo1, t.hi1);
+    float* const L2 = blk + start(t.lo2, t.hi2);
+    auto load = [&](float2 (&r)[N]) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            r[q].x = (!RAGGED || t.v1) ? L1[q * ST] : 0.0f;
+            r[q].y = (!RAGGED || t.v2) ? L2[q * ST] : 0.0f;
+        }
+    };
+    auto store = [&](const float2 (&r)[N]) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            if (!RAGGED || t.v1) L1[q * ST] = r[q].x;
+            if (!RAGGED || t.v2) L2[q * ST] = r[q].y;
+        }
+    };
+    float2 r[N];
+    if (SRC == GLOBAL) {
+        if (RAGGED) {
+#pragma unroll
+            for (int q = 0; q < N; ++q) r[q] = make_float2(0.0f, 0.0f);
+        }
+        if (!RAGGED || t.v1) load_line<N, AX, 0>(r, g + global_start<N, AX>(t.lo1, t.hi1), t.vec);
+        if (!RAGGED || t.v2) load_line<N, AX, 1>(r, g + global_start<N, AX>(t.lo2, t.hi2), t.vec);
+    }
+    const float idv = t.inv_dv[AX];
+    const float* vc = t.vc;
+    const PairCoef k =
+        pair_coef<N>(make_float2((sh[1] * vc[alo * N + t.lo1] + sh[2] * vc[ahi * N + t.hi1] + sh[3]) * idv,
+                                 (sh[1] * vc[alo * N + t.lo2] + sh[2] * vc[ahi * N + t.hi2] + sh[3]) * idv));
+    const bool whole = __ballot_sync(0xffffffffu, (t.v1 && k.s1 != 0) || (t.v2 && k.s2 != 0)) != 0u;
+    if (SRC == SHARED) load(r);
+    advance<N>(r, k);
+    auto shift = [&]() {
+        if (!RAGGED || t.v1) shift_line<N, ST>(L1, k.s1, k.f1);
+        if (!RAGGED || t.v2) shift_line<N, ST>(L2, k.s2, k.f2);
+    };
+    if (MOM == ASKED) {
+        if (__builtin_expect(!whole, 1)) {
+            store(r);
+            if (mom) products<N, AX>(m, r, t);
+        } else {
+            store(r);
+            shift();
+            if (mom) {
+                float2 z[N];  // r itself would cost the common path a move per value
+                load(z);
+                products<N, AX>(m, z, t);
+            }
+        }
+        return;
+    }
+    if (__builtin_expect(!whole, 1)) {
+        if (DST == SHARED) store(r);
+    } else {
+        store(r);
+        shift();
+        if (MOM == ALWAYS || DST == GLOBAL) load(r);  // the thread's own stores
+    }
+    if (DST == GLOBAL) {
+        if (!RAGGED || t.v1) store_line<N, AX, 0>(g + global_start<N, AX>(t.lo1, t.hi1), r, t.vec);
+        if (!RAGGED || t.v2) store_line<N, AX, 1>(g + global_start<N, AX>(t.lo2, t.hi2), r, t.vec);
+    }
+    if (MOM == ALWAYS) products<N, AX>(m, r, t);
+}
+
+template <int N, bool RAGGED, int SRC, int DST, int MOM>
+__device__ __forceinline__ void sweep_axis(int axis, bool mom, float* blk, float* g, const float* sh, const Lines& t,
                                            float (&m)[20]) {
-    if (axis == 0) sweep<N, 0, RAGGED, MOM>(blk, sh, vc, inv_dv, lo1, hi1, lo2, hi2, v1, v2, m);
-    else if (axis == 1) sweep<N, 1, RAGGED, MOM>(blk, sh, vc, inv_dv, lo1, hi1, lo2, hi2, v1, v2, m);
-    else sweep<N, 2, RAGGED, MOM>(blk, sh, vc, inv_dv, lo1, hi1, lo2, hi2, v1, v2, m);
+    if (axis == 0) sweep<N, 0, RAGGED, SRC, DST, MOM>(mom, blk, g, sh, t, m);
+    else if (axis == 1) sweep<N, 1, RAGGED, SRC, DST, MOM>(mom, blk, g, sh, t, m);
+    else sweep<N, 2, RAGGED, SRC, DST, MOM>(mom, blk, g, sh, t, m);
 }
 
 }  // namespace pair
 
-// One CTA per velocity block at a time (persistent over cells), as
-// velocity_kernel, with the FP32 two-lines-per-thread sweeps. Thread t of
-// warp w holds lines w 64 + lane and w 64 + 32 + lane (line = hi N + lo), so
-// each shared-memory instruction of a warp touches 32 consecutive lines.
+// One CTA per velocity block at a time, with the FP32 two-lines-per-thread
+// sweeps. Thread t of warp w holds lines w 64 + lane and w 64 + 32 + lane (line
+// = hi N + lo), so each shared-memory instruction of a warp touches 32
+// consecutive lines. A pass reads and writes f once, but what bounds it is the
+// issue of the sweeps: 64 instructions per value for N = 16, 41 of them the
+// arithmetic and the shared-memory accesses of five sweeps.
+//
+// The next cell comes from the block scheduler (work_queue.cuh), known one cell
+// ahead so that its block is on its way while this one is swept. With a fixed
+// stride the CTAs of an SM drift apart and the last ones run alone (16.4 of 20
+// warps active on average): 256 x 128 x 16^3 475 us against 428.
+//
+// STAGED (N <= 16): two buffers; the next block is copied asynchronously. One
+// copy of each sweep's code, the moments' part behind a flag: with a second one
+// for the sweep that forms moments the code outgrows the instruction caches
+// (462 us).
+// OWN (N = 16): a warp's 64 lines are four whole planes of v_z, along v_x and
+// along v_y alike, so a warp that copies, sweeps along v_x and v_y and stores its
+// own planes meets the others only around a sweep along v_z (two block barriers
+// per cell instead of seven; 442 -> 431 us).
+//
+// Direct (N >= 20): the first sweep reads its lines straight from global memory
+// and the last one writes them there from registers, so a block passes through
+// shared memory once per pair of sweeps and not once more on either side (8
+// instead of 12 accesses per value). 128 x 64 x 20^3 353 -> 294 us, 24^3 615 ->
+// 481. For N = 16 that is slower (507 us against 477 staged, then): along v_x
+// the rows of a warp's lines are 32 different 128-byte lines per instruction.
 template <int N>
 __global__ void __launch_bounds__(pair::threads(N), pair::min_blocks(N)) velocity_pair_kernel(VelocityArgs a) {
     constexpr int NTH = pair::threads(N);
-    constexpr bool RAGGED = (N * N) % 64 != 0;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr bool RAGGED = (N * N) % 64 != 0, STAGED = pair::staged(N), OWN = N == 16;
+    constexpr long long V = (long long)N * N * N;
     constexpr int BLK = N * N * (N + 1);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ WorkQueue queue;
+    __shared__ int item;  // the cell after the next one
     float* const buf0 = reinterpret_cast<float*>(smem_raw);
-    float* const buf1 = buf0 + BLK;
     double* red = reinterpret_cast<double*>(smem_raw + sizeof(float) * BLK * a.nbuf);
-    float* sh = reinterpret_cast<float*>(red + 20 * pair::warps(N) + 20);  // [20] shears of the cell
-    float* vc = sh + 20;                                                   // [3][N] cell-centre velocities
+    float* sh = reinterpret_cast<float*>(red + 20 * pair::warps(N) + 20);  // [2][20] shears of this and the next cell
+    float* vc = sh + 40;                                                   // [3][N] cell-centre velocities
     float* inv_dv = vc + 3 * N;                                            // [3]
     float* f = reinterpret_cast<float*>(a.f);
-    constexpr long long V = (long long)N * N * N;
-    const bool two = a.nbuf == 2;
-    for (int q = threadIdx.x; q < 3 * N; q += NTH) {
+    const int tid = threadIdx.x;
+    const bool dyn = a.counters != nullptr;
+    if (dyn && tid == 0) {
+        queue.init();
+        queue.request();
+    }
+    for (int q = tid; q < 3 * N; q += NTH) {
         const int ax = q / N, i = q % N;
         vc[q] = (float)(a.vmin[ax] + (i + 0.5) * a.dv[ax]);
     }
-    if (threadIdx.x < 3) inv_dv[threadIdx.x] = (float)(1.0 / a.dv[threadIdx.x]);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m1 = warp * 64 + lane, m2 = m1 + 32;
-    const bool v1 = m1 < N * N, v2 = m2 < N * N;
-    const int lo1 = v1 ? m1 % N : 0, hi1 = v1 ? m1 / N : 0;
-    const int lo2 = v2 ? m2 % N : 0, hi2 = v2 ? m2 / N : 0;
-    long long cell = blockIdx.x;
-    auto prefetch = [](float* blk, const float* src) {
-        if constexpr (rows_tile<N, NTH>()) prefetch_block_rows<N, NTH>(blk, src);
+    if (tid < 3) inv_dv[tid] = (float)(1.0 / a.dv[tid]);
+    const int m1 = (tid >> 5) * 64 + (tid & 31), m2 = m1 + 32;
+    pair::Lines t;
+    t.v1 = m1 < N * N;
+    t.v2 = m2 < N * N;
+    t.lo1 = t.v1 ? m1 % N : 0;
+    t.hi1 = t.v1 ? m1 / N : 0;
+    t.lo2 = t.v2 ? m2 % N : 0;
+    t.hi2 = t.v2 ? m2 / N : 0;
+    t.vec = a.vec != 0;
+    t.vc = vc;
+    t.inv_dv = inv_dv;
+    auto fetch = [&](float* blk, const float* src) {  // start the copies of a block
+        if constexpr (OWN) prefetch_planes<N>(blk, src);
+        else if constexpr (rows_tile<N, NTH>()) prefetch_block_rows<N, NTH>(blk, src);
         else prefetch_block<float, N, NTH>(blk, src);
     };
-    if (two && cell < a.ncell) prefetch(buf0, f + cell * V);
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    for (int it = 0; cell < a.ncell; cell += gridDim.x, ++it) {
-        float* blk = (two && (it & 1)) ? buf1 : buf0;
-        if (two) {
-            const long long nx = cell + gridDim.x;
-            if (nx < a.ncell) prefetch((it & 1) ? buf0 : buf1, f + nx * V);
+    long long cell = blockIdx.x, next = -1;
+    if (STAGED) {
+        if (cell < a.ncell) fetch(buf0, f + cell * V);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    if (tid < 20 && cell < a.ncell) sh[tid] = (float)a.shears[cell * 20 + tid];
+    if (dyn && tid == 0) item = queue.take(0, a.counters);
+    __syncthreads();
+    if (dyn) next = item;
+    else next = cell + gridDim.x < a.ncell ? cell + gridDim.x : -1;
+    for (int it = 0; cell >= 0 && cell < a.ncell; ++it) {
+        float* blk = (a.nbuf == 2 && (it & 1)) ? buf0 + BLK : buf0;
+        float* g = f + cell * V;
+        const float* s = sh + (it & 1) * 20;
+        double* const out = a.mom_out ? a.mom_out + cell * 20 : nullptr;
+        const int last = a.nshear - 1;
+        double shn = 0.0;
+        bool first = true;  // the cell's first barrier is still to come
+        // After it every warp has left the previous cell: that one's shears make
+        // room for the next cell's, and the cell after it becomes known. A second
+        // barrier always follows before the cell's end.
+        auto barrier = [&]() {
+            __syncthreads();
+            if (first && next >= 0) {
+                if (tid < 20) sh[((it + 1) & 1) * 20 + tid] = (float)shn;
+                if (dyn && tid == 0) item = queue.take(it + 1, a.counters);
+            }
+            first = false;
+        };
+        float m[20];
+        if constexpr (STAGED) {
+            if (next >= 0) fetch((it & 1) ? buf0 : buf0 + BLK, f + next * V);
             asm volatile("cp.async.commit_group;\n" ::: "memory");
+            if (dyn && tid == 0 && next >= 0) queue.request();
+            if (tid < 20 && next >= 0) shn = a.shears[next * 20 + tid];
             asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        } else {
-            load_block<float, N, NTH>(blk, f + cell * V);
-        }
-        if (threadIdx.x < 20) sh[threadIdx.x] = (float)a.shears[cell * 20 + threadIdx.x];
-        __syncthreads();
-        double* out = a.mom_out ? a.mom_out + cell * 20 : nullptr;
-        for (int k = 0; k < a.nshear; ++k) {
-            const float* s = sh + 4 * k;
-            const int axis = (int)s[0];
-            float m[20];
+            // axis of the sweep before (v_z: barrier needed; the copy counts as v_x)
+            int prev = 0;
+            for (int k = 0; k <= last; ++k) {
+                const int axis = (int)s[4 * k];
+                if (!OWN || prev == 2 || axis == 2) barrier();
+                else __syncwarp();
+                prev = axis;
+                const bool mom = out && k == last;
 #pragma unroll
-            for (int o = 0; o < 20; ++o) m[o] = 0.0f;
-            if (out && k == a.nshear - 1) {
-                pair::sweep_axis<N, RAGGED, true>(axis, blk, s, vc, inv_dv, lo1, hi1, lo2, hi2, v1, v2, m);
+                for (int o = 0; o < 20; ++o) m[o] = 0.0f;
+                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::SHARED, pair::ASKED>(axis, mom, blk, g, s + 4 * k, t, m);
+                if (mom) reduce_moments<float, pair::warps(N)>(m, red, out, a.conv);
+            }
+            if (!OWN || prev == 2) barrier();
+            else __syncwarp();
+            if constexpr (OWN) {
+                store_planes<N>(g, blk, t.vec);
+            } else {
+                if (groups_tile<N, NTH>() && t.vec) store_block_groups<N, NTH>(g, blk);
+                else store_block<float, N, NTH>(g, blk, t.vec);
+                __syncthreads();
+            }
+        } else {
+            if (next >= 0) {
+                for (int o = tid * 32; o < V; o += NTH * 32)
+                    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(f + next * V + o));
+            }
+            if (dyn && tid == 0 && next >= 0) queue.request();
+            if (tid < 20 && next >= 0) shn = a.shears[next * 20 + tid];
+            pair::sweep_axis<N, RAGGED, pair::GLOBAL, pair::SHARED, pair::NEVER>((int)s[0], false, blk, g, s, t, m);
+            barrier();
+            for (int k = 1; k < last; ++k) {
+                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::SHARED, pair::NEVER>((int)s[4 * k], false, blk, g, s + 4 * k, t, m);
+                barrier();
+            }
+            const float* sl = s + 4 * last;
+            if (out) {
+#pragma unroll
+                for (int o = 0; o < 20; ++o) m[o] = 0.0f;
+                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::GLOBAL, pair::ALWAYS>((int)sl[0], true, blk, g, sl, t, m);
                 reduce_moments<float, pair::warps(N)>(m, red, out, a.conv);
             } else {
-                pair::sweep_axis<N, RAGGED, false>(axis, blk, s, vc, inv_dv, lo1, hi1, lo2, hi2, v1, v2, m);
+                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::GLOBAL, pair::NEVER>((int)sl[0], false, blk, g, sl, t, m);
             }
-            __syncthreads();
+            // one buffer: the next cell's first sweep overwrites lines others still read
+            if (a.nbuf == 1) __syncthreads();
         }
-        if (groups_tile<N, NTH>() && a.vec) store_block_groups<N, NTH>(f + cell * V, blk);
-        else store_block<float, N, NTH>(f + cell * V, blk, a.vec != 0);
-        __syncthreads();
+        cell = next;
+        if (dyn) next = next >= 0 ? item : -1;
+        else next = cell >= 0 && cell + gridDim.x < a.ncell ? cell + gridDim.x : -1;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
@@ -855,15 +1059,23 @@ static cudaError_t launch_velocity_pair(const VelocityArgs& a, cudaStream_t st) 
     const int threads = pair::threads(N);
     const size_t blk = sizeof(float) * N * N * (N + 1);
     VelocityArgs b = a;
-    b.nbuf = 2 * blk <= 100 * 1024 ? 2 : 1;
+    // staged: double buffering while two buffers leave room for two CTAs per SM;
+    // direct: where the register cap's CTAs still fit with both
+    b.nbuf = pair::staged(N) || 2 * blk * pair::min_blocks(N) <= 210 * 1024 ? 2 : 1;
     b.vec = reinterpret_cast<uintptr_t>(a.f) % 16 == 0;
-    size_t smem = blk * b.nbuf + sizeof(double) * (20 * pair::warps(N) + 20) + sizeof(float) * (20 + 3 * N + 3);
+    size_t smem = blk * b.nbuf + sizeof(double) * (20 * pair::warps(N) + 20) + sizeof(float) * (40 + 3 * N + 3);
     cudaFuncSetAttribute(velocity_pair_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, velocity_pair_kernel<N>, threads, smem);
-    if (per_sm < 1) per_sm = 1;
-    long long grid = (long long)num_sms() * per_sm;
-    if (grid > a.ncell) grid = a.ncell;
+    const long long slots = (long long)num_sms() * std::max(per_sm, 1);
+    // The queue pays from about six cells a slot on: below, the blocks that
+    // start first take cells that free slots were about to start (40 x 25 cells
+    // of 16^3 33.2 us against 28.8 by the stride; 128 x 64 121.7 against 132.5)
+    long long grid = a.ncell;
+    if (!b.counters || a.ncell < 6 * slots || a.ncell >= (1LL << 31)) {
+        b.counters = nullptr;
+        grid = std::min(a.ncell, slots);
+    }
     velocity_pair_kernel<N><<<(unsigned)grid, threads, smem, st>>>(b);
     count_launch();
     return cudaGetLastError();
