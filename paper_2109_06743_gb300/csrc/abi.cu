@@ -473,7 +473,6 @@ vl_status pfc_advect_v(vl_ctx* ctx, int s, double dt, double* mom_out, vl_stream
     a.f = ctx->f[s];
     a.eb = ctx->eb;
     a.shears = ctx->ws.cellwork;
-    a.counters = ctx->ws.counters;
     a.mom_out = mom_out;
     a.ncell = ncell_of(d);
     a.nv = d.nv[s][0];
@@ -522,7 +521,6 @@ vl_status pfc_advect_v_static(const vl_desc* desc, int s, void* f_dev, const dou
     a.f = f_dev;
     a.eb = eb_dev;
     a.shears = static_cast<double*>(scratch);
-    a.counters = nullptr;
     a.mom_out = mom_out;
     a.ncell = ncell;
     a.nv = d.nv[s][0];

@@ -93,7 +93,7 @@ struct VelocityArgs {
     int nshear;
     int nbuf;               // block buffers in shared memory (set by the launcher)
     int vec;                // f is 16-byte aligned: write blocks back with 16-byte stores (set by the launcher)
-    unsigned long long* counters;  // null: cells by a fixed stride
+    float inv_dv[3];        // 1 / dv (set by the launcher of the FP32 pass)
     double qm, dt;
     double vmin[3], dv[3];
     MomConv conv;

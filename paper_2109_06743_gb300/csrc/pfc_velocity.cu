@@ -20,13 +20,10 @@
 // FP32 blocks run velocity_pair_kernel (two lines per thread, packed FP32x2
 // arithmetic, every line walked upwards); FP64 blocks run velocity_kernel
 // (one line per thread, walked in the direction of its displacement).
-#include <algorithm>
-
 #include "common.cuh"
 #include "kernels.cuh"
 #include "block_moments.cuh"
 #include "f32x2.cuh"
-#include "work_queue.cuh"
 
 namespace vl {
 
@@ -512,11 +509,13 @@ using x2::sub;
 
 constexpr int threads(int n) { return ((n * n / 2 + 31) / 32) * 32; }
 constexpr int warps(int n) { return threads(n) / 32; }
-// CTAs per SM the register cap is sized for
 // blocks staged in shared memory, or the first and last sweep straight from and
 // to global memory
 constexpr bool staged(int n) { return n <= 16; }
-constexpr int min_blocks(int n) { return n <= 8 ? 24 : (n <= 12 ? 7 : (n <= 16 ? 5 : (n <= 20 ? 3 : 2))); }
+// CTAs per SM the register cap is sized for (24^3 three: 430 us at 128 x 64 cells,
+// two: 434; 20^3 four: 256, three: 281, five: 289; 16^3 seven: 412 at 256 x 128,
+// five: 426; 12^3 eight: 278, ten: 285)
+constexpr int min_blocks(int n) { return n <= 8 ? 24 : (n <= 12 ? 8 : (n <= 16 ? 7 : (n <= 20 ? 4 : 3))); }
 
 // physical exponents (x, y, z) of moment o, packed x + 4 y + 16 z
 __host__ __device__ constexpr int mono_exp(int o) {
@@ -788,33 +787,34 @@ __device__ __forceinline__ void sweep_axis(int axis, bool mom, float* blk, float
 
 }  // namespace pair
 
-// One CTA per velocity block at a time, with the FP32 two-lines-per-thread
-// sweeps. Thread t of warp w holds lines w 64 + lane and w 64 + 32 + lane (line
-// = hi N + lo), so each shared-memory instruction of a warp touches 32
-// consecutive lines. A pass reads and writes f once, but what bounds it is the
-// issue of the sweeps: 64 instructions per value for N = 16, 41 of them the
-// arithmetic and the shared-memory accesses of five sweeps.
+// One CTA per cell, with the FP32 two-lines-per-thread sweeps. Thread t of warp w
+// holds lines w 64 + lane and w 64 + 32 + lane (line = hi N + lo), so each
+// shared-memory instruction of a warp touches 32 consecutive lines. A pass reads
+// and writes f once, but what bounds it is the issue of the sweeps: about 64
+// instructions per value for N = 16, 41 of them the arithmetic and the
+// shared-memory accesses of five sweeps.
 //
-// The next cell comes from the block scheduler (work_queue.cuh), known one cell
-// ahead so that its block is on its way while this one is swept. With a fixed
-// stride the CTAs of an SM drift apart and the last ones run alone (16.4 of 20
-// warps active on average): 256 x 128 x 16^3 475 us against 428.
+// Why a CTA per cell: CTAs that stay and walk the cells by a fixed stride drift
+// apart (16.4 of 20 warps active on average for N = 16, 475 us at 256 x 128
+// cells); taking the next cell from the block scheduler and prefetching it mends
+// that (428 us), but the loop, the second buffer and the look-ahead cost
+// instructions, registers and shared memory, and the CTAs that follow each other
+// overlap their copies just as well. 256 x 128 cells, before -> now: 16^3 477 ->
+// 412 us, 12^3 334 -> 278, 8^3 84 -> 78; 128 x 64 cells of 20^3 355 -> 256, 24^3
+// 615 -> 430.
 //
-// STAGED (N <= 16): two buffers; the next block is copied asynchronously. One
-// copy of each sweep's code, the moments' part behind a flag: with a second one
-// for the sweep that forms moments the code outgrows the instruction caches
-// (462 us).
+// STAGED (N <= 16): the block is copied to shared memory and back. One copy of
+// each sweep's code, the moments' part behind a flag: with a second one for the
+// sweep that forms moments the code outgrows the instruction caches.
 // OWN (N = 16): a warp's 64 lines are four whole planes of v_z, along v_x and
 // along v_y alike, so a warp that copies, sweeps along v_x and v_y and stores its
-// own planes meets the others only around a sweep along v_z (two block barriers
-// per cell instead of seven; 442 -> 431 us).
+// own planes meets the others only around a sweep along v_z.
 //
 // Direct (N >= 20): the first sweep reads its lines straight from global memory
 // and the last one writes them there from registers, so a block passes through
 // shared memory once per pair of sweeps and not once more on either side (8
-// instead of 12 accesses per value). 128 x 64 x 20^3 353 -> 294 us, 24^3 615 ->
-// 481. For N = 16 that is slower (507 us against 477 staged, then): along v_x
-// the rows of a warp's lines are 32 different 128-byte lines per instruction.
+// instead of 12 accesses per value). For N = 16 that is slower: along v_x the
+// rows of a warp's lines are 32 different 128-byte lines per instruction.
 template <int N>
 __global__ void __launch_bounds__(pair::threads(N), pair::min_blocks(N)) velocity_pair_kernel(VelocityArgs a) {
     constexpr int NTH = pair::threads(N);
@@ -822,25 +822,26 @@ __global__ void __launch_bounds__(pair::threads(N), pair::min_blocks(N)) velocit
     constexpr long long V = (long long)N * N * N;
     constexpr int BLK = N * N * (N + 1);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ WorkQueue queue;
-    __shared__ int item;  // the cell after the next one
-    float* const buf0 = reinterpret_cast<float*>(smem_raw);
-    double* red = reinterpret_cast<double*>(smem_raw + sizeof(float) * BLK * a.nbuf);
-    float* sh = reinterpret_cast<float*>(red + 20 * pair::warps(N) + 20);  // [2][20] shears of this and the next cell
-    float* vc = sh + 40;                                                   // [3][N] cell-centre velocities
-    float* inv_dv = vc + 3 * N;                                            // [3]
-    float* f = reinterpret_cast<float*>(a.f);
+    float* const blk = reinterpret_cast<float*>(smem_raw);
+    double* const red = reinterpret_cast<double*>(smem_raw + sizeof(float) * BLK);
+    float* const s = reinterpret_cast<float*>(red + 20 * pair::warps(N) + 20);  // [20] shears of the cell
+    float* const vc = s + 20;                                                  // [3][N] cell-centre velocities
+    float* const inv_dv = vc + 3 * N;                                          // [3]
+    const long long cell = blockIdx.x;
+    float* const g = reinterpret_cast<float*>(a.f) + cell * V;
     const int tid = threadIdx.x;
-    const bool dyn = a.counters != nullptr;
-    if (dyn && tid == 0) {
-        queue.init();
-        queue.request();
+    if constexpr (STAGED) {
+        if constexpr (OWN) prefetch_planes<N>(blk, g);
+        else if constexpr (rows_tile<N, NTH>()) prefetch_block_rows<N, NTH>(blk, g);
+        else prefetch_block<float, N, NTH>(blk, g);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
+    if (tid < 20) s[tid] = (float)a.shears[cell * 20 + tid];
     for (int q = tid; q < 3 * N; q += NTH) {
         const int ax = q / N, i = q % N;
         vc[q] = (float)(a.vmin[ax] + (i + 0.5) * a.dv[ax]);
     }
-    if (tid < 3) inv_dv[tid] = (float)(1.0 / a.dv[tid]);
+    if (tid < 3) inv_dv[tid] = a.inv_dv[tid];
     const int m1 = (tid >> 5) * 64 + (tid & 31), m2 = m1 + 32;
     pair::Lines t;
     t.v1 = m1 < N * N;
@@ -852,99 +853,52 @@ __global__ void __launch_bounds__(pair::threads(N), pair::min_blocks(N)) velocit
     t.vec = a.vec != 0;
     t.vc = vc;
     t.inv_dv = inv_dv;
-    auto fetch = [&](float* blk, const float* src) {  // start the copies of a block
-        if constexpr (OWN) prefetch_planes<N>(blk, src);
-        else if constexpr (rows_tile<N, NTH>()) prefetch_block_rows<N, NTH>(blk, src);
-        else prefetch_block<float, N, NTH>(blk, src);
-    };
-    long long cell = blockIdx.x, next = -1;
-    if (STAGED) {
-        if (cell < a.ncell) fetch(buf0, f + cell * V);
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    if (tid < 20 && cell < a.ncell) sh[tid] = (float)a.shears[cell * 20 + tid];
-    if (dyn && tid == 0) item = queue.take(0, a.counters);
-    __syncthreads();
-    if (dyn) next = item;
-    else next = cell + gridDim.x < a.ncell ? cell + gridDim.x : -1;
-    for (int it = 0; cell >= 0 && cell < a.ncell; ++it) {
-        float* blk = (a.nbuf == 2 && (it & 1)) ? buf0 + BLK : buf0;
-        float* g = f + cell * V;
-        const float* s = sh + (it & 1) * 20;
-        double* const out = a.mom_out ? a.mom_out + cell * 20 : nullptr;
-        const int last = a.nshear - 1;
-        double shn = 0.0;
-        bool first = true;  // the cell's first barrier is still to come
-        // After it every warp has left the previous cell: that one's shears make
-        // room for the next cell's, and the cell after it becomes known. A second
-        // barrier always follows before the cell's end.
-        auto barrier = [&]() {
-            __syncthreads();
-            if (first && next >= 0) {
-                if (tid < 20) sh[((it + 1) & 1) * 20 + tid] = (float)shn;
-                if (dyn && tid == 0) item = queue.take(it + 1, a.counters);
-            }
-            first = false;
-        };
-        float m[20];
-        if constexpr (STAGED) {
-            if (next >= 0) fetch((it & 1) ? buf0 : buf0 + BLK, f + next * V);
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
-            if (dyn && tid == 0 && next >= 0) queue.request();
-            if (tid < 20 && next >= 0) shn = a.shears[next * 20 + tid];
-            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-            // axis of the sweep before (v_z: barrier needed; the copy counts as v_x)
-            int prev = 0;
-            for (int k = 0; k <= last; ++k) {
-                const int axis = (int)s[4 * k];
-                if (!OWN || prev == 2 || axis == 2) barrier();
+    double* const out = a.mom_out ? a.mom_out + cell * 20 : nullptr;
+    const int last = a.nshear - 1;
+    float m[20];
+    if constexpr (STAGED) {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        int prev = 2;  // axis of the sweep before (at first: the shears and vc are everyone's)
+        for (int k = 0; k <= last; ++k) {
+            const bool mom = out && k == last;
+            if (k == 0) __syncthreads();
+            const int axis = (int)s[4 * k];
+            if (k > 0) {
+                if (!OWN || prev == 2 || axis == 2) __syncthreads();
                 else __syncwarp();
-                prev = axis;
-                const bool mom = out && k == last;
+            }
+            prev = axis;
 #pragma unroll
-                for (int o = 0; o < 20; ++o) m[o] = 0.0f;
-                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::SHARED, pair::ASKED>(axis, mom, blk, g, s + 4 * k, t, m);
-                if (mom) reduce_moments<float, pair::warps(N)>(m, red, out, a.conv);
-            }
-            if (!OWN || prev == 2) barrier();
-            else __syncwarp();
-            if constexpr (OWN) {
-                store_planes<N>(g, blk, t.vec);
-            } else {
-                if (groups_tile<N, NTH>() && t.vec) store_block_groups<N, NTH>(g, blk);
-                else store_block<float, N, NTH>(g, blk, t.vec);
-                __syncthreads();
-            }
-        } else {
-            if (next >= 0) {
-                for (int o = tid * 32; o < V; o += NTH * 32)
-                    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(f + next * V + o));
-            }
-            if (dyn && tid == 0 && next >= 0) queue.request();
-            if (tid < 20 && next >= 0) shn = a.shears[next * 20 + tid];
-            pair::sweep_axis<N, RAGGED, pair::GLOBAL, pair::SHARED, pair::NEVER>((int)s[0], false, blk, g, s, t, m);
-            barrier();
-            for (int k = 1; k < last; ++k) {
-                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::SHARED, pair::NEVER>((int)s[4 * k], false, blk, g, s + 4 * k, t, m);
-                barrier();
-            }
-            const float* sl = s + 4 * last;
-            if (out) {
-#pragma unroll
-                for (int o = 0; o < 20; ++o) m[o] = 0.0f;
-                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::GLOBAL, pair::ALWAYS>((int)sl[0], true, blk, g, sl, t, m);
-                reduce_moments<float, pair::warps(N)>(m, red, out, a.conv);
-            } else {
-                pair::sweep_axis<N, RAGGED, pair::SHARED, pair::GLOBAL, pair::NEVER>((int)sl[0], false, blk, g, sl, t, m);
-            }
-            // one buffer: the next cell's first sweep overwrites lines others still read
-            if (a.nbuf == 1) __syncthreads();
+            for (int o = 0; o < 20; ++o) m[o] = 0.0f;
+            pair::sweep_axis<N, RAGGED, pair::SHARED, pair::SHARED, pair::ASKED>(axis, mom, blk, g, s + 4 * k, t, m);
+            if (mom) reduce_moments<float, pair::warps(N)>(m, red, out, a.conv);
         }
-        cell = next;
-        if (dyn) next = next >= 0 ? item : -1;
-        else next = cell >= 0 && cell + gridDim.x < a.ncell ? cell + gridDim.x : -1;
+        if (!OWN || prev == 2) __syncthreads();
+        else __syncwarp();
+        if constexpr (OWN) {
+            store_planes<N>(g, blk, t.vec);
+        } else {
+            if (groups_tile<N, NTH>() && t.vec) store_block_groups<N, NTH>(g, blk);
+            else store_block<float, N, NTH>(g, blk, t.vec);
+        }
+    } else {
+        __syncthreads();
+        pair::sweep_axis<N, RAGGED, pair::GLOBAL, pair::SHARED, pair::NEVER>((int)s[0], false, blk, g, s, t, m);
+        __syncthreads();
+        for (int k = 1; k < last; ++k) {
+            pair::sweep_axis<N, RAGGED, pair::SHARED, pair::SHARED, pair::NEVER>((int)s[4 * k], false, blk, g, s + 4 * k, t, m);
+            __syncthreads();
+        }
+        const float* sl = s + 4 * last;
+        if (out) {
+#pragma unroll
+            for (int o = 0; o < 20; ++o) m[o] = 0.0f;
+            pair::sweep_axis<N, RAGGED, pair::SHARED, pair::GLOBAL, pair::ALWAYS>((int)sl[0], true, blk, g, sl, t, m);
+            reduce_moments<float, pair::warps(N)>(m, red, out, a.conv);
+        } else {
+            pair::sweep_axis<N, RAGGED, pair::SHARED, pair::GLOBAL, pair::NEVER>((int)sl[0], false, blk, g, sl, t, m);
+        }
     }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
 template <typename T, int N>
@@ -1056,27 +1010,14 @@ static cudaError_t launch_velocity_n(const VelocityArgs& a, cudaStream_t st) {
 
 template <int N>
 static cudaError_t launch_velocity_pair(const VelocityArgs& a, cudaStream_t st) {
-    const int threads = pair::threads(N);
-    const size_t blk = sizeof(float) * N * N * (N + 1);
     VelocityArgs b = a;
-    // staged: double buffering while two buffers leave room for two CTAs per SM;
-    // direct: where the register cap's CTAs still fit with both
-    b.nbuf = pair::staged(N) || 2 * blk * pair::min_blocks(N) <= 210 * 1024 ? 2 : 1;
+    b.nbuf = 1;
     b.vec = reinterpret_cast<uintptr_t>(a.f) % 16 == 0;
-    size_t smem = blk * b.nbuf + sizeof(double) * (20 * pair::warps(N) + 20) + sizeof(float) * (40 + 3 * N + 3);
+    for (int q = 0; q < 3; ++q) b.inv_dv[q] = (float)(1.0 / a.dv[q]);
+    const size_t smem = sizeof(float) * N * N * (N + 1) + sizeof(double) * (20 * pair::warps(N) + 20) +
+                        sizeof(float) * (20 + 3 * N + 3);
     cudaFuncSetAttribute(velocity_pair_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, velocity_pair_kernel<N>, threads, smem);
-    const long long slots = (long long)num_sms() * std::max(per_sm, 1);
-    // The queue pays from about six cells a slot on: below, the blocks that
-    // start first take cells that free slots were about to start (40 x 25 cells
-    // of 16^3 33.2 us against 28.8 by the stride; 128 x 64 121.7 against 132.5)
-    long long grid = a.ncell;
-    if (!b.counters || a.ncell < 6 * slots || a.ncell >= (1LL << 31)) {
-        b.counters = nullptr;
-        grid = std::min(a.ncell, slots);
-    }
-    velocity_pair_kernel<N><<<(unsigned)grid, threads, smem, st>>>(b);
+    velocity_pair_kernel<N><<<(unsigned)a.ncell, pair::threads(N), smem, st>>>(b);
     count_launch();
     return cudaGetLastError();
 }

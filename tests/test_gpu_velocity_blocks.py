@@ -1,8 +1,8 @@
-"""The FP32 velocity pass on more cells than the chip holds blocks: cells taken
-from the block scheduler (pfc_advect_v) against cells by a fixed stride on an f
-that is not 16-byte aligned (pfc_advect_v_static). A cell's arithmetic does not
-depend on who sweeps it or where from, so both give the same bits; that the
-values themselves are right is checked against the oracle elsewhere.
+"""The FP32 velocity pass on more cells than the chip holds blocks, on an f that is
+16-byte aligned (pfc_advect_v: 16-byte copies and stores) and on one that is not
+(pfc_advect_v_static: scalar ones). A cell's arithmetic depends on neither, so
+both give the same bits; that the values themselves are right is checked
+against the oracle elsewhere.
 """
 import numpy as np
 import pytest
@@ -24,7 +24,7 @@ def gpu():
 
 @pytest.mark.parametrize("nv,nx,ny", [(8, 160, 150), (12, 96, 72), (16, 80, 60), (16, 3, 3), (20, 64, 48), (24, 48, 40)])
 @pytest.mark.parametrize("e_scale,nshear", [(0.3, 5), (6.0, 5), (0.3, 3)])
-def test_queue_equals_stride(gpu, nv, nx, ny, e_scale, nshear):
+def test_aligned_equals_unaligned(gpu, nv, nx, ny, e_scale, nshear):
     from gpu_util import AbiRunner
     from paper_2109_06743_gb300 import abi
     cfg = W.harris(nx=nx, ny=ny, nv=nv, lx=25.6 * nx / 128, ly=12.8 * ny / 64, precision=32)
@@ -46,5 +46,4 @@ def test_queue_equals_stride(gpu, nv, nx, ny, e_scale, nshear):
         gpu.cuda.synchronize()
         assert gpu.equal(moved, r.f[k])
         assert gpu.equal(mom, mom2)
-    assert abi.vl_read_stats(r.ctx)[8] == 0  # no request ran out of time
     r.close()
