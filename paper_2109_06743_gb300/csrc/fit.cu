@@ -225,14 +225,34 @@ __device__ __noinline__ void add_maxwellian(double (&r)[N], const double* pd, in
 
 constexpr int ex_threads(int n) { return ((n * n + 31) / 32) * 32; }
 
-// One CTA per cell at a time (persistent): thread t < N^2 owns the v_z line
-// (i, j) = (t mod N, t / N), so each load and store of the block is a
-// contiguous run of N^2 values. f <- f - M_V + M_F; if any value is negative
-// all are clipped at zero and the cell rescaled to n_V (the limiter of
-// Algorithm 1); cells whose fits are invalid are left alone. Fused with the
-// moments of the new f.
+// CTAs per SM the register cap leaves room for. FP32: as many as pay (24^3 two:
+// 196 us at 128 x 64 cells, three: 227; 20^3 three: 123, two: 160; 16^3 seven: 217
+// at 256 x 128, five: 224); FP64: the compiler's own choice, made explicit.
 template <typename T, int N>
-__global__ void __launch_bounds__(ex_threads(N)) exchange_kernel(ExchangeArgs a) {
+constexpr int ex_blocks() {
+    if (sizeof(T) == 8) return N == 8 ? 14 : (N == 12 ? 4 : (N == 16 ? 3 : 1));
+    return N == 8 ? 28 : (N == 12 ? 10 : (N == 16 ? 7 : (N == 20 ? 3 : 2)));
+}
+
+// FP64 blocks of 20^3 and 24^3 leave room for one CTA per SM: it stays and walks the
+// cells (24^3 685 us at 32 x 32 cells, by a CTA per cell 694)
+template <typename T, int N>
+constexpr bool ex_stays() { return sizeof(T) == 8 && N >= 20; }
+
+// One CTA per cell: thread t < N^2 owns the v_z line (i, j) = (t mod N, t / N),
+// so each load and store of the block is a contiguous run of N^2 values.
+// f <- f - M_V + M_F; if any value is negative all are clipped at zero and the
+// cell rescaled to n_V (the limiter of Algorithm 1); cells whose fits are
+// invalid are left alone. Fused with the moments of the new f.
+//
+// A cell is short (a few barriers around one pass over its block), so a CTA
+// that ends and makes room for the next one overlaps cells better than one that
+// stays: the loop over cells of a resident CTA also cost 8 to 24 registers, and
+// with them warps. With the parameters' kernel, 256 x 128 cells: 16^3 247 -> 217
+// us (5.7 TB/s in this kernel), 12^3 171 -> 137, 8^3 68 -> 66; 128 x 64 cells of
+// 20^3 155 -> 123, 24^3 212 -> 196.
+template <typename T, int N>
+__global__ void __launch_bounds__(ex_threads(N), ex_blocks<T, N>()) exchange_kernel(ExchangeArgs a) {
     __shared__ double red[20 * 32 + 20];
     __shared__ T ssum[32];
     __shared__ T sscale;
@@ -246,7 +266,8 @@ __global__ void __launch_bounds__(ex_threads(N)) exchange_kernel(ExchangeArgs a)
     const bool active = t < NN;
     const int i = active ? t % N : 0, j = active ? t / N : 0;
     const T* par = reinterpret_cast<const T*>(a.par);
-    for (long long cell = blockIdx.x; cell < a.ncell; cell += gridDim.x) {
+    long long cell = blockIdx.x;
+    do {
         T r[N];
         const T* src = f + cell * V + t;
         if (active) {
@@ -319,8 +340,8 @@ __global__ void __launch_bounds__(ex_threads(N)) exchange_kernel(ExchangeArgs a)
             if (a.mom_out) line_products_z<T, N>(m, S0, S1, S2, S3, i, j);
         }
         if (a.mom_out) reduce_moments<T>(m, red, a.mom_out + cell * 20, a.conv);
-        __syncthreads();
-    }
+        if (ex_stays<T, N>()) __syncthreads();  // the shared arrays are the next cell's
+    } while (ex_stays<T, N>() && (cell += gridDim.x) < a.ncell);
 }
 
 // ------------------------------------------------------------------- 1D1V
@@ -493,17 +514,6 @@ __global__ void exchange1d_kernel(ExchangeArgs a) {
 
 // ---------------------------------------------------------------- launchers
 
-static int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
-}
-
 // 1D1V: theta is stored directly in the coefficient slots
 __global__ void theta1d_kernel(const double* coef, const int* status, int which, double* theta, long long ncell) {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -540,12 +550,14 @@ static cudaError_t launch_exchange_n(const ExchangeArgs& a, cudaStream_t st) {
         if (e != cudaSuccess) return e;
     }
     const int threads = ex_threads(N);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, exchange_kernel<T, N>, threads, 0);
-    if (per_sm < 1) per_sm = 1;
-    long long grid = (long long)sm_count() * per_sm;
-    if (grid > a.ncell) grid = a.ncell;
-    exchange_kernel<T, N><<<(unsigned)grid, threads, 0, st>>>(a);
+    unsigned grid = (unsigned)a.ncell;
+    if (ex_stays<T, N>()) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (sms > 0 && (unsigned)sms < grid) grid = (unsigned)sms;
+    }
+    exchange_kernel<T, N><<<grid, threads, 0, st>>>(a);
     count_launch();
     return cudaGetLastError();
 }
