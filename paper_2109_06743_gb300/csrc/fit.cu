@@ -78,7 +78,7 @@ __global__ void coef_to_theta_kernel(const double* coef, const int* status, int 
     }
     const double* u0 = k + 10;
     const double* sg = k + 13;
-    th[0] = exp(k[0] + 0.5 * quad) * pow(2.0 * M_PI, 1.5) * sqrt(det3(Thw)) * sg[0] * sg[1] * sg[2];
+    th[0] = exp(k[0] + 0.5 * quad) * 15.749609945722419 /* (2 pi)^(3/2) */ * sqrt(det3(Thw)) * sg[0] * sg[1] * sg[2];
     for (int p = 0; p < 3; ++p) th[1 + p] = u0[p] + sg[p] * uw[p];
     int q = 4;
     for (int p = 0; p < 3; ++p)
