@@ -130,8 +130,9 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# Work of the Newton fits per velocity cell and evaluation of a discrete
-# Maxwellian, in operations (add, multiply or fused multiply-add: one each).
+# Work of the Newton fits by direct sums (8^3 blocks, the fits the closed form
+# leaves over, and the method's own count, which the closed form does not perform)
+# per velocity cell and evaluation of a discrete Maxwellian, in operations (add, multiply or fused multiply-add: one each).
 # The method's own work (Sec. 2.2's discrete fit): the ten moment sums of
 # degree <= 2 per evaluation, and 25 more sums (degree 3 and 4, the entries
 # of the Gram matrix beyond the moments) when the Jacobian is formed.
@@ -232,6 +233,27 @@ def newton_roofline(cfg, stats, fit_ms, launches, alu, fp64=False):
         out["method_vs_fp64_peak"] = achieved / alu["fp64_tops"]
         out["issued_alu_ops_per_launch"] = issued_alu / max(1, launches)
     return out
+
+
+def fit_roofline(cfg, stats, fit_ms, launches, alu, hbm_peak, fp64=False):
+    """Roofline of the fits as they run. Blocks of 12^3 and more are fitted from
+    the closed form of the discrete moments (one thread per fit, some ten
+    thousand dependent operations, no sum over the velocity cells): neither
+    HBM nor an ALU pipe is near its rate, the slowest fits' chains bound the
+    launch. achieved and frac are the bytes a launch must move over its time
+    against the copy bandwidth; direct_sum_equivalent is the rate at which
+    direct sums would have to work to be as fast (above 1: faster than any
+    direct sum could be on that pipe)."""
+    direct = newton_roofline(cfg, stats, fit_ms, launches, alu, fp64=fp64)
+    if direct is None or cfg.species[0].nv[0] < 12:
+        return direct
+    gbps = direct["algorithmic_bytes_per_launch"] * max(1, launches) / (fit_ms / 1e3) / 1e9
+    return {"kernel": "fit_solve (closed_fit_kernel, newton_list_kernel)" if not fp64 else
+            "fit_solve (closed_fit_kernel, newton64_kernel)", "bound": "latency", "achieved": gbps, "peak": hbm_peak,
+            "unit": "GB/s", "frac": gbps / hbm_peak, "traffic": None,
+            "algorithmic_bytes_per_launch": direct["algorithmic_bytes_per_launch"], "evaluations": direct["evaluations"],
+            "direct_sum_equivalent": {"achieved": direct["achieved"], "peak": direct["peak"], "unit": direct["unit"],
+                                      "frac": direct["frac"]}}
 
 
 def slowest(seconds, dist=None, device="cpu"):
@@ -711,7 +733,7 @@ def measure_2d3v(name, device, alu, steps, warmup, e2e_steps, cold_steps, fp64_s
     per_launch_cells = cells // nsp  # one species per launch
     rows = hbm_rows(phase_ms, count, per_launch_cells)
     dom = max(phase_ms, key=lambda k: phase_ms[k])
-    newton = newton_roofline(cfg, stats, phase_ms.get("fit_solve"), count.get("fit_solve", 1), alu)
+    newton = fit_roofline(cfg, stats, phase_ms.get("fit_solve"), count.get("fit_solve", 1), alu, peak)
     if dom in rows:
         roof = {"kernel": dom, "bound": "hbm", "achieved": rows[dom]["GBps"], "peak": peak, "unit": "GB/s",
                 "frac": rows[dom]["GBps"] / peak, "traffic": None, "peak_kind": peak_kind,
@@ -818,7 +840,7 @@ def measure_2d3v(name, device, alu, steps, warmup, e2e_steps, cold_steps, fp64_s
                 "steps": fp64_steps, "phases_ms_per_step": {k: v / fp64_steps for k, v in sorted(ph64.items())},
                 "hbm_phases": hbm_rows(ph64, cnt64, per_launch_cells, 16),
                 "newton_iterations_per_fit": st64[0] / nf64, "newton_fallbacks_per_fit": st64[1] / nf64,
-                "fit_roofline": newton_roofline(cfg64, st64, ph64.get("fit_solve"), cnt64.get("fit_solve", 1), alu,
+                "fit_roofline": fit_roofline(cfg64, st64, ph64.get("fit_solve"), cnt64.get("fit_solve", 1), alu, peak,
                                                 fp64=True),
                 "note": "same workload, FP64 f, sweeps, fluid and plain FP64 Newton fit, cold-started"}
         s64.close()
