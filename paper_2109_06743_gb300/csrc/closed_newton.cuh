@@ -332,9 +332,14 @@ CF_FN double wide_of(double a) { return a; }
 // tolerance, by one step more or less (measured against the direct kernels
 // over 1.6e5 fits: 5e-13, 1.8e-6 of the step, the residual or the step). A fit
 // with a parameter that close to a rounding boundary is decided by the direct
-// kernel, so that f does not depend on which kernel made a fit (about two
-// fits in ten thousand; small off-diagonal parameters, whose last place moves
-// nothing by 1e-8, do not count).
+// kernel, so that f does not depend on which kernel made a fit. Off-diagonal
+// parameters below 1/64 have a finer last place: it moves the Maxwellian by less
+// than 1e-8, but a value that falls below zero makes the exchange rescale its cell,
+// and that moves it by a rounding of f. They count down to 1/512, with the
+// typical difference of two fits (1.5e-13) instead of the largest; below, the last
+// place is lost in the exchange's own roundings. (Cells of 512 x 256 x 16^3 that
+// differ from the direct kernels' after an exchange, of 1.6 million: 5 without
+// them, one by 9e-8; 1 with them, by 6e-9. Fits of 256 x 128 ions 429 -> 447 us.)
 template <typename T>
 CF_FN bool rounds_alike(const Maxw<T>& g, const FitBox<T>& b, const double (&u0)[3], const double (&sg)[3], double tol,
                         const FitArgs& a, const FitCount& fc) {
@@ -343,8 +348,10 @@ CF_FN bool rounds_alike(const Maxw<T>& g, const FitBox<T>& b, const double (&u0)
     if (res > 0.9 * tol) eps += res;
     if ((double)fc.prev < 1.1 * tol) eps += 2.2 * last;
     auto alike = [](double p, double d) { return (float)(p - d) == (float)(p + d); };
-    auto small = [&](double p, double d) { return fabs(p) < 0.015625 || alike(p, d); };
-    const double e2 = 1.5 * eps, e4 = 3.0 * eps;
+    const double e2 = 1.5 * eps, e4 = 3.0 * eps, es = (eps - 6.5e-13) / e4;
+    auto small = [&](double p, double d) {
+        return fabs(p) < 0.001953125 || alike(p, fabs(p) < 0.015625 ? d * es : d);
+    };
     double h[3], P[6];
     bool ok = alike(wide_of(g.L), e2);
     CF_UNROLL
