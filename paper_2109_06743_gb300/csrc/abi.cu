@@ -357,6 +357,8 @@ static vl_status sweep_axis(vl_ctx* ctx, int s, int axis, double dt, void* f_out
         a.mode = 0;
         a.ncol = 32;
         while (a.ncol > 8 && (size_t)a.n * a.ncol * es > 64 * 1024) a.ncol /= 2;
+        // FP64 in 1D1V: narrow tiles, on more SMs (see launch_pfc_space)
+        if (d.nvdim == 1 && es == 8) a.ncol = 8;
         a.nchunks = (int)((V + a.ncol - 1) / a.ncol);
     }
     // cp.async staging needs every column run (V, nvx and the tile width in

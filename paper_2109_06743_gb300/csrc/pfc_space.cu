@@ -240,8 +240,13 @@ cudaError_t launch_pfc_space(const SpaceSweepArgs& a, int precision, cudaStream_
     const long long ntiles = (long long)a.nchunks * a.nlines;
     // one thread per (column, segment of about 16 cells), up to 1024 threads:
     // short segments give each SM enough independent sliding windows to hide
-    // the shared-memory latency of the window updates
-    int nseg = (a.n + 15) / 16;
+    // the shared-memory latency of the window updates; in FP64 with fewer tiles
+    // than SMs (1D1V, smallest grids) segments of 4: there the FP64 pipe of the few
+    // SMs at work and the depth of a segment bound the sweep (64 cells of 32
+    // velocities: one tile of 32 columns in segments of 16 13.5 us, four tiles in
+    // segments of 16 15.5, in segments of 4 9.5)
+    const int cells = precision == 64 && ntiles < 152 ? 4 : 16;
+    int nseg = (a.n + cells - 1) / cells;
     if (nseg > 1024 / a.ncol) nseg = 1024 / a.ncol;
     if (nseg < 1) nseg = 1;
     const int threads = a.ncol * nseg;
