@@ -20,7 +20,7 @@
 //   * the doubly and triply outside cells weigh the product of the tails
 //     (1e-12 and less for a box of five standard deviations): FP32 sums over
 //     the corners' first few cells.
-// About 5 thousand operations instead of 37 N^3. closed_eval refuses (returns
+// About 10 thousand operations instead of 37 N^3. closed_eval refuses (returns
 // false) whatever it cannot give to rounding: means near or beyond a face,
 // strongly correlated or very narrow covariances, heavy corners; such fits
 // take the direct sums (newton.cuh, newton64.cuh).

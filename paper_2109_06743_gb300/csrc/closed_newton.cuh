@@ -15,13 +15,15 @@
 // differently (rounds_alike) go on a list; the direct kernels then fit those
 // from their start as before. Results agree to the fit tolerance either way.
 //
-// Why one thread per fit: an evaluation is about 5 k operations with little
+// Why one thread per fit: an evaluation is some 10 k operations with little
 // parallelism inside (three axes, two sides), against 152 k for the direct
 // sums by eight lanes; 65536 fits fill the chip 14 warps deep per SM.
 // Measured (GB300), closed form and list: 65536 cold fits of 16^3 Harris ions
-// 2.23 -> 0.43 ms (0.29 + 0.14), 65536 network-started fits of 12^3
-// asymmetric-sheet electrons 2.14 -> 0.78 ms, 16384 fits in FP64 mode 5.08 ->
-// 0.44 ms.
+// 2.23 -> 0.44 ms (0.25 + 0.15, and theta), 65536 network-started fits of 12^3
+// asymmetric-sheet electrons 2.11 -> 0.76 ms, 16384 fits in FP64 mode 5.08 -> 0.42
+// ms. What bounds it: the slowest warps' chains of dependent operations (5.6
+// cycles per instruction and warp, 10 warps per SM); blocks of 32 to 128 threads
+// at 96 to 168 registers are all within 3%.
 #pragma once
 
 #include "closed_form.cuh"
