@@ -20,7 +20,7 @@
 // sums by eight lanes; 65536 fits fill the chip 14 warps deep per SM.
 // Measured (GB300), closed form and list: 65536 cold fits of 16^3 Harris ions
 // 2.23 -> 0.44 ms (0.25 + 0.15, and theta), 65536 network-started fits of 12^3
-// asymmetric-sheet electrons 2.11 -> 0.76 ms, 16384 fits in FP64 mode 5.08 -> 0.42
+// asymmetric-sheet electrons 2.11 -> 0.73-0.86 ms, 16384 fits in FP64 mode 5.08 -> 0.42
 // ms. What bounds it: the slowest warps' chains of dependent operations (5.6
 // cycles per instruction and warp, 10 warps per SM); blocks of 32 to 128 threads
 // at 96 to 168 registers are all within 3%.
