@@ -33,6 +33,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "df64.cuh"
 #include "fit_index.cuh"
 
@@ -124,6 +126,14 @@ CF_FN df2 from(float x, df2) { return {x, 0.f}; }
 CF_FN double from(double x, double) { return x; }
 CF_FN double from(float x, double) { return (double)x; }
 
+CF_FN double wide_of(df2 a) { return (double)a.hi + (double)a.lo; }
+CF_FN double wide_of(double a) { return a; }
+// a value in V: FP64, or FP32 without the rest
+template <typename V, typename T>
+CF_FN V plain(T a) {
+    return sizeof(V) == 8 ? (V)wide_of(a) : (V)hi(a);
+}
+
 CF_FN float expj(float x) { return expf(x); }
 CF_FN double expj(double x) { return exp(x); }
 
@@ -203,6 +213,16 @@ CF_FN void add_low(Eval<T>& e, T t0, T t1, T t2, const T (&r)[3], const T (&S)[6
         for (int b = a; b < 3; ++b)
             e.A2[sym(a, b)] = add(e.A2[sym(a, b)], add(mul(rt, r[b]), mul(S[sym(a, b)], t0)));
     }
+}
+
+// adds moments 1, d, d d in a plain type
+template <typename T, typename V>
+CF_FN void add_moments(Eval<T>& e, const V (&m)[10]) {
+    e.A0 = add(e.A0, num<T>(m[0]));
+    CF_UNROLL
+    for (int q = 0; q < 3; ++q) e.A1[q] = add(e.A1[q], num<T>(m[1 + q]));
+    CF_UNROLL
+    for (int q = 0; q < 6; ++q) e.A2[q] = add(e.A2[q], num<T>(m[4 + q]));
 }
 
 template <typename J>
@@ -450,73 +470,90 @@ CF_FN void far_mode(int q, int& x, int& y, int& z) {
     }
 }
 
-// The Poisson modes along the two other axes of the cells outside along axis
-// a (FP32: they are the product of two small parts): at signed distance t the
-// cross section is a Gaussian with mean r t and covariance Sc, so mode k adds
-// 2 amp Re exp(-i (phi + omega t)) times the moments of r t + N(-i s, Sc),
-// s = 2 pi Sc k / h. f is minus the lattice integral; out collects 1, d, d d.
-CF_FN void tail_modes(int a, float f, float ca, float iv, float tp, float tm, float h, const float (&ih)[3],
-                      const float (&xf)[3], const float (&r)[3], const float (&Sc)[6], float cut, float (&out)[10]) {
+// The Poisson modes along the two other axes of the cells outside along axis a:
+// at signed distance t the cross section is a Gaussian with mean r t and
+// covariance Sc, so mode k adds 2 amp Re exp(-i (phi + omega t)) times the
+// moments of r t + N(-i s, Sc), s = 2 pi Sc k / h. f is minus the lattice
+// integral, x the mean's offset from its cell, out gets 1, d, d d.
+//
+// They are the product of two small parts, so FP32 gives them where that
+// product is small enough (Limits::tail). A narrow Maxwellian next to a face
+// makes both parts large (0.7 cells per standard deviation, a face at 2: 1e-4 of
+// the density, of which FP32 loses 1e-10): those are summed in FP64, by the
+// evaluation's FINE form, whichever the arithmetic.
+template <typename V>
+struct Tail {
+    V f, ca, iv, tp, tm, h, ih[3], x[3], r[3], S[6];
+};
+
+CF_FN void turn(float y, float& c, float& s) {
+    y -= rintf(y);
+    c = cosf(6.2831853f * y);
+    s = sinf(6.2831853f * y);
+}
+CF_FN void turn(double y, double& c, double& s) { cossin(y, c, s); }
+
+template <typename V>
+CF_FN void tail_modes(int a, const Tail<V>& q, V cut, V (&out)[10]) {
+    constexpr V two_pi = V(6.283185307179586476925);
+    CF_UNROLL
+    for (int d = 0; d < 10; ++d) out[d] = V(0);
     CF_LOOP
-    for (int q = 0; q < 4; ++q) {
-        const float kb = q == 1 ? 0.f : 1.f, kc = q == 0 ? 0.f : (q == 3 ? -1.f : 1.f);
-        const float k[3] = {a == 0 ? 0.f : kb, a == 1 ? 0.f : (a == 0 ? kb : kc), a == 2 ? 0.f : kc};
-        float u[3], y[3], ex = 0.f, om = 0.f, ph = 0.f;
+    for (int m = 0; m < 4; ++m) {
+        const V kb = m == 1 ? V(0) : V(1), kc = m == 0 ? V(0) : (m == 3 ? V(-1) : V(1));
+        const V k[3] = {a == 0 ? V(0) : kb, a == 1 ? V(0) : (a == 0 ? kb : kc), a == 2 ? V(0) : kc};
+        V u[3], y[3], ex = V(0), om = V(0), ph = V(0);
         CF_UNROLL
-        for (int d = 0; d < 3; ++d) u[d] = k[d] * ih[d];
+        for (int d = 0; d < 3; ++d) u[d] = k[d] * q.ih[d];
         CF_UNROLL
         for (int d = 0; d < 3; ++d) {
-            y[d] = Sc[sym(d, 0)] * u[0] + Sc[sym(d, 1)] * u[1] + Sc[sym(d, 2)] * u[2];
+            y[d] = q.S[sym(d, 0)] * u[0] + q.S[sym(d, 1)] * u[1] + q.S[sym(d, 2)] * u[2];
             ex += u[d] * y[d];
-            om += u[d] * r[d];
-            ph += k[d] * xf[d];
+            om += u[d] * q.r[d];
+            ph += k[d] * q.x[d];
         }
-        ex *= 19.7392088f;  // 2 pi^2
-        if (ex > 40.f) continue;
-        const float am = 2.f * f * expf(-ex);
-        const float cr = cosf(6.2831853f * om * h), sr = sinf(6.2831853f * om * h);
-        float c0 = 0.f, s0 = 0.f, c1 = 0.f, s1 = 0.f, c2 = 0.f;
+        ex *= V(19.739208802178717238);  // 2 pi^2
+        if (ex > V(40)) continue;
+        const V am = V(2) * q.f * expj(-ex);
+        V cr, sr, c0 = V(0), s0 = V(0), c1 = V(0), s1 = V(0), c2 = V(0);
+        turn(om * q.h, cr, sr);
         CF_LOOP
         for (int side = 0; side < 2; ++side) {
-            float t = side ? tm : tp;
-            float w = ca * expf(-0.5f * t * t * iv), rt = expf(-(t + 0.5f * h) * h * iv);
-            const float rr = expf(-h * h * iv), sg = side ? -1.f : 1.f;
-            float turn = ph + om * sg * t;
-            turn -= rintf(turn);
-            float c = cosf(6.2831853f * turn), s = sinf(6.2831853f * turn);
+            V t = side ? q.tm : q.tp;
+            V w = q.ca * expj(V(-0.5) * t * t * q.iv), rt = expj(-(t + V(0.5) * q.h) * q.h * q.iv);
+            const V rr = expj(-q.h * q.h * q.iv), sg = side ? V(-1) : V(1);
+            V c, s;
+            turn(ph + om * sg * t, c, s);
             CF_LOOP
             for (int j = 0; j < 64 && w > cut; ++j) {
-                const float wt = w * sg * t;
-                c0 = fmaf(w, c, c0);
-                s0 = fmaf(w, s, s0);
-                c1 = fmaf(wt, c, c1);
-                s1 = fmaf(wt, s, s1);
-                c2 = fmaf(wt * sg * t, c, c2);
-                const float cn = c * cr - sg * s * sr;
-                s = fmaf(sg * c, sr, s * cr);
+                const V wt = w * sg * t;
+                c0 += w * c;
+                s0 += w * s;
+                c1 += wt * c;
+                s1 += wt * s;
+                c2 += wt * sg * t * c;
+                const V cn = c * cr - sg * s * sr;
+                s = s * cr + sg * c * sr;
                 c = cn;
                 w *= rt;
                 rt *= rr;
-                t += h;
+                t += q.h;
             }
         }
-        out[0] = fmaf(am, c0, out[0]);
+        out[0] += am * c0;
         CF_UNROLL
         for (int d = 0; d < 3; ++d) {
-            const float sd = 6.2831853f * y[d];
-            out[1 + d] = fmaf(am, r[d] * c1 - sd * s0, out[1 + d]);
+            const V sd = two_pi * y[d];
+            out[1 + d] += am * (q.r[d] * c1 - sd * s0);
             CF_UNROLL
             for (int e = d; e < 3; ++e) {
-                const float se = 6.2831853f * y[e];
-                out[4 + sym(d, e)] = fmaf(am,
-                                          r[d] * r[e] * c2 - (r[d] * se + sd * r[e]) * s1 +
-                                              (Sc[sym(d, e)] - sd * se) * c0,
-                                          out[4 + sym(d, e)]);
+                const V se = two_pi * y[e];
+                out[4 + sym(d, e)] +=
+                    am * (q.r[d] * q.r[e] * c2 - (q.r[d] * se + sd * q.r[e]) * s1 + (q.S[sym(d, e)] - sd * se) * c0);
             }
         }
     }
 }
-
 // limits of a closed-form evaluation, relative to the density: what may be
 // left out, and what may be summed in FP32
 template <typename T>
@@ -526,18 +563,22 @@ struct Limits<df2> {
     static constexpr float drop = 2e-15f;   // a neglected part
     static constexpr float cut = 1e-19f;    // smallest cell weight of a sum
     static constexpr float fp32 = 3e-7f;    // doubly outside cells (times t^2) summed in FP32
+    static constexpr float tail = 2e-8f;    // tails' Poisson modes (times t^2) summed in FP32
 };
 template <>
 struct Limits<double> {
     static constexpr float drop = 1e-16f;
     static constexpr float cut = 1e-21f;
     static constexpr float fp32 = 1e-10f;
+    static constexpr float tail = 2e-11f;
 };
 
 // Discrete moments (and with gram the Gram sums) of g over the N^3 cells of
-// the box, about its own mean. False where the closed form does not apply.
-template <typename T>
-CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, Eval<T>& e) {
+// the box, about its own mean. False where the closed form does not apply, or
+// (coarse) where it takes the FINE form, which sums small parts in FP64 that are
+// too large for FP32.
+template <typename T, bool FINE>
+CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, Eval<T>& e, bool& coarse) {
     typedef typename Jac<T>::type J;
     typedef Limits<T> Lim;
     const T* P = g.P;
@@ -628,7 +669,7 @@ CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
     }
 
     // singly outside cells, axis by axis
-    float out2 = 0.f, cross[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float out2 = 0.f;
     CF_LOOP
     for (int a = 0; a < 3; ++a) {
         const T va = pick(a, S[0], S[3], S[5]);
@@ -681,14 +722,31 @@ CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
             CF_UNROLL
             for (int d = c; d < 3; ++d) Sc[sym(c, d)] = sub(S[sym(c, d)], mul(r[c], row[d]));
         const T nn = neg(np);
-        if (modes1 * fmaxf(f0, f2) > Lim::drop) {
-            float rf[3], scf[6];
+        const float weight = modes1 * fmaxf(f0, f2);
+        if (!FINE && weight > Lim::tail) {
+            coarse = true;
+            return false;
+        }
+        if (weight > Lim::drop) {
+            typedef typename std::conditional<FINE, double, float>::type V;
+            Tail<V> q;
+            q.f = plain<V>(nn);
+            q.ca = plain<V>(ca);
+            q.iv = plain<V>(iv);
+            q.tp = plain<V>(sub(edge, off));
+            q.tm = plain<V>(add(edge, off));
+            q.h = plain<V>(h);
             CF_UNROLL
-            for (int c = 0; c < 3; ++c) rf[c] = hi(r[c]);
+            for (int c = 0; c < 3; ++c) {
+                q.ih[c] = plain<V>(ihT[c]);
+                q.x[c] = plain<V>(x[c]);
+                q.r[c] = plain<V>(r[c]);
+            }
             CF_UNROLL
-            for (int q = 0; q < 6; ++q) scf[q] = hi(Sc[q]);
-            tail_modes(a, hi(nn), hi(ca), hi(iv), pick(a, tp[0], tp[1], tp[2]), pick(a, tm[0], tm[1], tm[2]), hi(h), ih, xf,
-                       rf, scf, Lim::cut, cross);
+            for (int c = 0; c < 6; ++c) q.S[c] = plain<V>(Sc[c]);
+            V part[10];
+            tail_modes<V>(a, q, V(Lim::cut), part);
+            add_moments(e, part);
         }
         add_low(e, mul(nn, t0), mul(nn, t1), mul(nn, t2), r, Sc);
         if (gram) {
@@ -705,11 +763,6 @@ CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
     // remaining axis, are left out
     if (modes) {
         if (24.f * (1.f + 160.f * top) * expf(-4.f * kTwoPi2 * lam) * out2 > 5.f * Lim::drop) return false;
-        e.A0 = add(e.A0, from(cross[0], zero));
-        CF_UNROLL
-        for (int q = 0; q < 3; ++q) e.A1[q] = add(e.A1[q], from(cross[1 + q], zero));
-        CF_UNROLL
-        for (int q = 0; q < 6; ++q) e.A2[q] = add(e.A2[q], from(cross[4 + q], zero));
     }
 
     // doubly outside cells
@@ -929,6 +982,13 @@ CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
         }
     }
     return true;
+}
+
+// either form
+template <typename T>
+CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, Eval<T>& e) {
+    bool coarse = false;
+    return closed_sums<T, false>(g, b, N, gram, e, coarse) || (coarse && closed_sums<T, true>(g, b, N, gram, e, coarse));
 }
 
 }  // namespace cf

@@ -34,6 +34,12 @@
 namespace vl {
 namespace cf {
 
+#ifdef __CUDACC__
+#define CF_CALL __device__ __noinline__
+#else
+#define CF_CALL inline
+#endif
+
 constexpr int kCoefC = 16;
 
 // dl = -J^-1 G, J the Gram matrix packed from the central sums C, by LDL^T
@@ -106,6 +112,7 @@ struct FitCount {
     int iters;
     unsigned evals, grams;
     float last, res, prev;  // size of the last Newton step, residuals after and before it (relative to n)
+    bool coarse;            // an evaluation asked for the FINE form
 };
 
 // thresholds of the direct kernels: damping test above kDamp n, Gram sums with
@@ -116,8 +123,8 @@ CF_FN bool more_steps(float rel, float, float) { return rel > 1e-5f; }
 CF_FN bool more_steps(double rel, double tol, double) { return 100.0 * rel * rel > tol; }
 
 // Newton iteration from g to max |D - Tt| <= tol n. Returns false when the
-// fit is left to the direct kernels.
-template <typename T>
+// fit is left to the FINE form (cnt.coarse) or to the direct kernels.
+template <typename T, bool FINE>
 CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10], double n, double tol,
                          int max_iter, FitCount& cnt) {
     typedef typename Jac<T>::type J;
@@ -128,7 +135,7 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
     CF_LOOP
     for (int it = 0;; ++it) {
         Eval<T> e;
-        if (!closed_eval<T>(g, b, N, gram, e)) return false;
+        if (!closed_sums<T, FINE>(g, b, N, gram, e, cnt.coarse)) return false;
         ++cnt.evals;
         cnt.grams += gram ? 1u : 0u;
         // moments about w = 0, residual G
@@ -324,8 +331,70 @@ CF_FN bool from_eta(const typename Jac<T>::type (&eta)[10], Maxw<T>& g) {
     return true;
 }
 
-CF_FN double wide_of(df2 a) { return (double)a.hi + (double)a.lo; }
-CF_FN double wide_of(double a) { return a; }
+// The fit from the start eta0, or first from eta0 and the network's prediction dw
+// if there is one (the guard of its inference writes NaN rows for the fits it
+// rejects). One way out of the loop: with a return from inside it the lanes of a
+// warp did not come together again (network-started fits 840 -> 1310 us).
+CF_FN bool predicted(const float* dw) { return dw && fabsf(dw[0]) < 1e30f; }
+
+template <typename T, bool FINE>
+CF_FN bool closed_solve(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const typename Jac<T>::type (&eta0)[10],
+                        const float* dw, double n, const FitArgs& a, FitCount& fc) {
+    typedef typename Jac<T>::type J;
+    bool good = false;
+    CF_LOOP
+    for (int pass = predicted(dw) ? 0 : 1; pass < 2 && !good && !fc.coarse; ++pass) {
+        J eta[10];
+        CF_UNROLL
+        for (int q = 0; q < 10; ++q) {
+            const float d = pass == 0 ? dw[q] : 0.f;
+            eta[q] = eta0[q] + (fabsf(d) < 1e30f ? (J)d : J(0));
+        }
+        good = from_eta<T>(eta, g) && closed_newton<T, FINE>(g, b, a.nv, Tt, n, a.tol, a.max_iter, fc);
+    }
+    return good;
+}
+
+// The same in the FINE form, out of line and on copies: few fits take it, and its
+// code and registers stay out of the common path (called from within the
+// evaluation it cost the other fits 4.5%, so less than 1%).
+template <typename T>
+struct FineFit {
+    Maxw<T> g;
+    FitBox<T> b;
+    T Tt[10];
+    typename Jac<T>::type eta0[10];
+    const float* dw;
+    double n;
+    FitCount fc;
+};
+template <typename T>
+CF_CALL bool closed_solve_fine(FineFit<T>& f, const FitArgs& a) {
+    return closed_solve<T, true>(f.g, f.b, f.Tt, f.eta0, f.dw, f.n, a, f.fc);
+}
+
+// the fit in the form it needs
+template <typename T>
+CF_FN bool closed_fit(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const typename Jac<T>::type (&eta0)[10],
+                      const float* dw, double n, const FitArgs& a, FitCount& fc) {
+    if (closed_solve<T, false>(g, b, Tt, eta0, dw, n, a, fc)) return true;
+    if (!fc.coarse) return false;
+    FineFit<T> f;
+    f.b = b;
+    CF_UNROLL
+    for (int q = 0; q < 10; ++q) {
+        f.Tt[q] = Tt[q];
+        f.eta0[q] = eta0[q];
+    }
+    f.dw = dw;
+    f.n = n;
+    f.fc = fc;
+    f.fc.coarse = false;
+    const bool good = closed_solve_fine<T>(f, a);
+    g = f.g;
+    fc = f.fc;
+    return good;
+}
 
 // FP32 mode: the exchange rounds a fit's line parameters (fit.cu) to float,
 // and one unit in the last place of L moves the whole Maxwellian by 5e-7. Two
@@ -378,7 +447,7 @@ CF_FN bool rounds_alike(const Maxw<T>& g, const FitBox<T>& b, const double (&u0)
 // direct kernels are appended to a.todo. With a.sel the kernel also reduces
 // what chooses the direct kernel (see kernels.cuh).
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 2) closed_fit_kernel(FitArgs a) {
+__global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 2) closed_fit_kernel(const __grid_constant__ FitArgs a) {
     typedef typename Jac<T>::type J;
     constexpr bool kF64 = sizeof(J) == 8;
     __shared__ unsigned long long cnt[VL_NSTATS];
@@ -386,7 +455,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
     __syncthreads();
     const long long fit = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool have = fit < 2 * a.ncell;
-    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 1.f};
+    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 1.f, false};
     bool left = false;
     unsigned warm = 0u;
     unsigned long long top = 0ull, wide = 0ull;
@@ -424,21 +493,9 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
                 if (spread > 60.f) wide = top;
             }
             Maxw<T> g;
-            // from the network's prediction, if there is one (the guard of
-            // its inference writes NaN rows for the fits it rejects), then
-            // from the continuous Maxwellian
-            const float* wp = a.warm ? a.warm + fit * 10 : nullptr;
-            const bool started = wp && fabsf(wp[0]) < 1e30f;
-            CF_LOOP
-            for (int pass = started ? 0 : 1; pass < 2 && !good; ++pass) {
-                J eta[10];
-#pragma unroll
-                for (int q = 0; q < 10; ++q) {
-                    const float dw = pass == 0 ? wp[q] : 0.f;
-                    eta[q] = eta0[q] + (fabsf(dw) < 1e30f ? (J)dw : J(0));
-                }
-                good = from_eta<T>(eta, g) && closed_newton<T>(g, b, a.nv, Tt, t[0], a.tol, a.max_iter, fc);
-            }
+            const float* dw = a.warm ? a.warm + fit * 10 : nullptr;
+            const bool started = predicted(dw);
+            good = closed_fit<T>(g, b, Tt, eta0, dw, t[0], a, fc);
             if (!kF64 && good) good = rounds_alike<T>(g, b, u0, sg, a.tol, a, fc);
             if (good) {
                 warm = started ? 1u : 0u;
@@ -480,7 +537,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
             }
         }
         left = !good;
-        if (left) fc = {0, 0u, 0u, 0.f, 0.f, 1.f};
+        if (left) fc = {0, 0u, 0u, 0.f, 0.f, 1.f, false};
     }
     if (kF64) {
         if (left) a.todo[atomicAdd(a.ntodo, 1u)] = (unsigned long long)fit;
