@@ -554,6 +554,42 @@ CF_FN void tail_modes(int a, const Tail<V>& q, V cut, V (&out)[10]) {
         }
     }
 }
+// one far mode's moments 1, d, d d; false where it is below every rounding
+template <typename V>
+struct Far {
+    V n, ih[3], x[3], S[6];
+};
+template <typename V>
+CF_FN bool far_part(int q, const Far<V>& f, V (&out)[10]) {
+    int k[3];
+    far_mode(q, k[0], k[1], k[2]);
+    V u[3], y[3], ex = V(0), ph = V(0);
+    CF_UNROLL
+    for (int a = 0; a < 3; ++a) {
+        u[a] = V(k[a]) * f.ih[a];
+        ph += V(k[a]) * f.x[a];
+    }
+    CF_UNROLL
+    for (int a = 0; a < 3; ++a) {
+        y[a] = f.S[sym(a, 0)] * u[0] + f.S[sym(a, 1)] * u[1] + f.S[sym(a, 2)] * u[2];
+        ex += u[a] * y[a];
+    }
+    ex *= V(19.739208802178717238);  // 2 pi^2
+    if (ex > V(48)) return false;
+    V c, s;
+    turn(ph, c, s);
+    const V am = V(2) * f.n * expj(-ex);
+    out[0] = am * c;
+    CF_UNROLL
+    for (int a = 0; a < 3; ++a) {
+        y[a] *= V(6.283185307179586476925);
+        out[1 + a] = -am * s * y[a];
+        CF_UNROLL
+        for (int b = 0; b <= a; ++b) out[4 + sym(a, b)] = am * c * (f.S[sym(a, b)] - y[a] * y[b]);
+    }
+    return true;
+}
+
 // limits of a closed-form evaluation, relative to the density: what may be
 // left out, and what may be summed in FP32
 template <typename T>
@@ -563,7 +599,7 @@ struct Limits<df2> {
     static constexpr float drop = 2e-15f;   // a neglected part
     static constexpr float cut = 1e-19f;    // smallest cell weight of a sum
     static constexpr float fp32 = 3e-7f;    // doubly outside cells (times t^2) summed in FP32
-    static constexpr float tail = 2e-8f;    // tails' Poisson modes (times t^2) summed in FP32
+    static constexpr float tail = 2e-8f;    // tails' and far Poisson modes (times t^2) summed in FP32
 };
 template <>
 struct Limits<double> {
@@ -637,6 +673,10 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
     const float modes1 = 6.f * (1.f + 39.5f * top) * expf(-kTwoPi2 * kap);
     const bool modes = modes1 > Lim::drop;
     if (modes && !(24.f * (1.f + 240.f * top) * expf(-6.f * kTwoPi2 * lam) <= 4.f * Lim::drop)) return false;
+    if (!FINE && modes && 8.f * (1.f + 120.f * top) * expf(-3.f * kTwoPi2 * lam) > Lim::tail) {
+        coarse = true;
+        return false;
+    }
 
     // lattice integral
     const T zero = num<T>(0.0);
@@ -657,14 +697,12 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
 
     // index of the mean, (m - wc)/h + (N - 1)/2, to the nearest cell
     T ihT[3], x[3];
-    float xf[3];
     if (modes) {
         CF_UNROLL
         for (int a = 0; a < 3; ++a) {
             ihT[a] = inv(b.h[a]);
             x[a] = add(mul(sub(g.m[a], b.wc[a]), ihT[a]), from(0.5f * (float)(N - 1), zero));
             x[a] = add(x[a], from(-rintf(hi(x[a])), zero));
-            xf[a] = hi(x[a]);
         }
     }
 
@@ -957,28 +995,22 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
                 add_gram<J>(e.C, cj, -sj, -cj, sj, cj, rj, Sj);
             }
         }
-        const float nf = hi(np);
+    }
+    if (modes && 3.f * kTwoPi2 * lam < 48.f) {  // far_part leaves out what is below e^-48
+        typedef typename std::conditional<FINE, double, float>::type V;
+        Far<V> f;
+        f.n = plain<V>(np);
+        CF_UNROLL
+        for (int a = 0; a < 3; ++a) {
+            f.ih[a] = plain<V>(ihT[a]);
+            f.x[a] = plain<V>(x[a]);
+        }
+        CF_UNROLL
+        for (int q = 0; q < 6; ++q) f.S[q] = plain<V>(S[q]);
         CF_LOOP
         for (int q = 0; q < kFarModes; ++q) {
-            int kx, ky, kz;
-            far_mode(q, kx, ky, kz);
-            const float u0 = kx * ih[0], u1 = ky * ih[1], u2 = kz * ih[2];
-            const float y0 = sf[0] * u0 + sf[1] * u1 + sf[2] * u2, y1 = sf[1] * u0 + sf[3] * u1 + sf[4] * u2,
-                        y2 = sf[2] * u0 + sf[4] * u1 + sf[5] * u2;
-            const float ex = kTwoPi2 * (u0 * y0 + u1 * y1 + u2 * y2);
-            if (ex > 48.f) continue;
-            float ph = kx * xf[0] + ky * xf[1] + kz * xf[2];
-            ph -= rintf(ph);
-            const float c = cosf(6.2831853f * ph), s = sinf(6.2831853f * ph), am = 2.f * nf * expf(-ex);
-            const float r[3] = {6.2831853f * y0, 6.2831853f * y1, 6.2831853f * y2};
-            e.A0 = add(e.A0, from(am * c, zero));
-            CF_UNROLL
-            for (int a = 0; a < 3; ++a) {
-                e.A1[a] = add(e.A1[a], from(-am * s * r[a], zero));
-                CF_UNROLL
-                for (int d = a; d < 3; ++d)
-                    e.A2[sym(a, d)] = add(e.A2[sym(a, d)], from(am * c * (sf[sym(a, d)] - r[a] * r[d]), zero));
-            }
+            V part[10];
+            if (far_part(q, f, part)) add_moments(e, part);
         }
     }
     return true;

@@ -98,3 +98,18 @@ def test_kept_fits_meet_their_tolerance(fits, arith, N):
     assert taken.sum() > len(tg) // 8
     over = out[taken, 2] - TOL[arith] - EVAL[arith] * out[taken, 4]
     assert np.all(over <= 0.0), out[taken][over > 0.0]
+
+
+@pytest.mark.parametrize("N", [12, 16, 20, 24])
+def test_barely_resolved_in_fp64(host, fits, N):  # noqa: F811
+    """0.6 to 0.78 cells per standard deviation in FP64 mode: the lattice's modes
+    beyond |k|^2 = 2 weigh up to 1e-7 of the density, too much for FP32."""
+    rows, tg = near_faces(np.random.default_rng(43 * N), 480 if N <= 16 else 160, N, 0.6, 0.78)
+    out = np.zeros((len(rows), 3))
+    host.closed_form_f64(N, 5.0, len(rows), rows, out)
+    taken = out[:, 0] == 1.0
+    assert taken.sum() > len(rows) // 16
+    assert np.all(out[taken, 1] <= EVAL["f64"]), out[taken, 1].max()
+    fit = fits("f64", N, tg)
+    kept = fit[:, 0] == 1.0
+    assert np.all(fit[kept, 2] <= TOL["f64"] + EVAL["f64"] * fit[kept, 4]), fit[kept, 2].max()
