@@ -191,11 +191,14 @@ struct FitBox {
 };
 
 // what an evaluation gives: A = moments 1, d, d d (d = w - m) times dv^3,
-// the covariance S = P^-1, and the Gram sums C of degree <= 4 in d (mono4)
+// the covariance S = P^-1, and the Gram sums C of degree <= 4 in d (mono4). C
+// leaves out the doubly and triply outside cells, the tails' modes and the far
+// modes; omitted is the largest weight (of degree <= 2) among them.
 template <typename T>
 struct Eval {
     T A0, A1[3], A2[6], S[6];
     typename Jac<T>::type C[35];
+    float omitted;
 };
 
 // Adds a source: the moments of r t + z with z ~ N(0, S) and given power sums
@@ -673,7 +676,8 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
     const float modes1 = 6.f * (1.f + 39.5f * top) * expf(-kTwoPi2 * kap);
     const bool modes = modes1 > Lim::drop;
     if (modes && !(24.f * (1.f + 240.f * top) * expf(-6.f * kTwoPi2 * lam) <= 4.f * Lim::drop)) return false;
-    if (!FINE && modes && 8.f * (1.f + 120.f * top) * expf(-3.f * kTwoPi2 * lam) > Lim::tail) {
+    e.omitted = modes ? 8.f * (1.f + 120.f * top) * expf(-3.f * kTwoPi2 * lam) : 0.f;
+    if (!FINE && e.omitted > Lim::tail) {
         coarse = true;
         return false;
     }
@@ -761,6 +765,7 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
             for (int d = c; d < 3; ++d) Sc[sym(c, d)] = sub(S[sym(c, d)], mul(r[c], row[d]));
         const T nn = neg(np);
         const float weight = modes1 * fmaxf(f0, f2);
+        e.omitted = fmaxf(e.omitted, weight);
         if (!FINE && weight > Lim::tail) {
             coarse = true;
             return false;
@@ -843,6 +848,7 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
         }
         if (!corner_sums<float>(ap, am, bp, bm, ha, hb, Qaa, Qab, Qbb, w4, Lim::cut, tf)) return false;
         const float weight = fmaxf(tf[0], fmaxf(tf[3] / saa, tf[5] / sbb));
+        e.omitted = fmaxf(e.omitted, weight);
         if (modes1 * weight > 5.f * Lim::drop) return false;
         if (!(tf[0] > 0.f)) continue;
         J t[6];

@@ -111,7 +111,9 @@ CF_FN double log_of(double x) { return log(x); }
 struct FitCount {
     int iters;
     unsigned evals, grams;
-    float last, res, prev;  // size of the last Newton step, residuals after and before it (relative to n)
+    float last, before;     // size of the last Newton step and of the one before it
+    float res, prev;        // residuals after and before the last step (relative to n)
+    float omitted;          // largest Eval::omitted of the pass
     bool coarse;            // an evaluation asked for the FINE form
 };
 
@@ -138,6 +140,7 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
         if (!closed_sums<T, FINE>(g, b, N, gram, e, cnt.coarse)) return false;
         ++cnt.evals;
         cnt.grams += gram ? 1u : 0u;
+        cnt.omitted = it == 0 ? e.omitted : fmaxf(cnt.omitted, e.omitted);
         // moments about w = 0, residual G
         T D[10], G[10];
         D[0] = e.A0;
@@ -211,6 +214,7 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
             const J v = fabs(dl[q]);
             big = v > big ? v : big;
         }
+        cnt.before = it == 0 ? 0.f : cnt.last;
         cnt.last = (float)big;
         cnt.prev = (float)rel;
         check = far;
@@ -397,27 +401,38 @@ CF_FN bool closed_fit(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const t
 }
 
 // FP32 mode: the exchange rounds a fit's line parameters (fit.cu) to float,
-// and one unit in the last place of L moves the whole Maxwellian by 5e-7. Two
-// fits of the same targets differ by the rounding of their sums, by a few 1e-6
-// of the last Newton step (FP32 Jacobian) and, where a residual lies at the
-// tolerance, by one step more or less (measured against the direct kernels
-// over 1.6e5 fits: 5e-13, 1.8e-6 of the step, the residual or the step). A fit
+// and one unit in the last place of L moves the whole Maxwellian by 5e-7. A fit
 // with a parameter that close to a rounding boundary is decided by the direct
-// kernel, so that f does not depend on which kernel made a fit. Off-diagonal
-// parameters below 1/64 have a finer last place: it moves the Maxwellian by less
-// than 1e-8, but a value that falls below zero makes the exchange rescale its cell,
-// and that moves it by a rounding of f. They count down to 1/512, with the
-// typical difference of two fits (1.5e-13) instead of the largest; below, the last
-// place is lost in the exchange's own roundings. (Cells of 512 x 256 x 16^3 that
-// differ from the direct kernels' after an exchange, of 1.6 million: 5 without
-// them, one by 9e-8; 1 with them, by 6e-9. Fits of 256 x 128 ions 429 -> 447 us.)
+// kernel, so that f does not depend on which kernel made a fit.
+//
+// fit_slack: how far two fits of the same targets may lie apart, by the rounding
+// of their sums, by a few 1e-6 of the last Newton step (FP32 Jacobian) and, where
+// a residual lies at the tolerance, by one step more or less (measured against the
+// direct kernels over 1.6e5 fits of the workloads: 5e-13, 1.8e-6 of the step, the
+// residual or the step). Where the Gram sums leave out more than FP32 resolves
+// (Eval::omitted; narrow Maxwellians near a face, two faces at once), the last step
+// leaves a remainder of the size of the residual rather than 2e-6 of the step, and
+// the direct kernel may need a step less: what is left out, times the step before.
+CF_FN double fit_slack(const FitCount& fc, double tol) {
+    const double last = fc.last, res = fc.res;
+    double eps = 8e-13 + 2e-6 * last;
+    if (fc.omitted > 1e-7f || res > 0.9 * tol) eps += res;
+    if ((double)fc.prev < 1.1 * tol + 10.0 * fc.omitted * fc.before) eps += 2.2 * last;
+    return eps;
+}
+
+// Off-diagonal parameters below 1/64 have a finer last place: it moves the
+// Maxwellian by less than 1e-8, but a value that falls below zero makes the
+// exchange rescale its cell, and that moves it by a rounding of f. They count down
+// to 1/512, with the typical difference of two fits (1.5e-13) instead of the
+// largest; below, the last place is lost in the exchange's own roundings. (Cells of
+// 512 x 256 x 16^3 that differ from the direct kernels' after an exchange, of 1.6
+// million: 5 without them, one by 9e-8; 1 with them, by 6e-9. Fits of 256 x 128 ions
+// 429 -> 447 us.)
 template <typename T>
 CF_FN bool rounds_alike(const Maxw<T>& g, const FitBox<T>& b, const double (&u0)[3], const double (&sg)[3], double tol,
                         const FitArgs& a, const FitCount& fc) {
-    const double last = fc.last, res = fc.res;
-    double eps = 8e-13 + 2e-6 * last;
-    if (res > 0.9 * tol) eps += res;
-    if ((double)fc.prev < 1.1 * tol) eps += 2.2 * last;
+    const double eps = fit_slack(fc, tol);
     auto alike = [](double p, double d) { return (float)(p - d) == (float)(p + d); };
     const double e2 = 1.5 * eps, e4 = 3.0 * eps, es = (eps - 6.5e-13) / e4;
     auto small = [&](double p, double d) {
@@ -455,7 +470,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
     __syncthreads();
     const long long fit = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool have = fit < 2 * a.ncell;
-    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 1.f, false};
+    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f, false};
     bool left = false;
     unsigned warm = 0u;
     unsigned long long top = 0ull, wide = 0ull;
@@ -537,7 +552,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
             }
         }
         left = !good;
-        if (left) fc = {0, 0u, 0u, 0.f, 0.f, 1.f, false};
+        if (left) fc = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f, false};
     }
     if (kF64) {
         if (left) a.todo[atomicAdd(a.ntodo, 1u)] = (unsigned long long)fit;

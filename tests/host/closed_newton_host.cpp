@@ -1,6 +1,6 @@
 // Whole closed-form fits (closed_newton.cuh: set-up, Newton iteration, and in FP32
 // mode the rounding screen) on the host, and the residual of what they return from
-// sums over the cells in long double, through two extern "C" functions (one per
+// sums over the cells in long double, through extern "C" functions (one per
 // arithmetic). In: rows of 10 raw moments. Out per row: 0 refused / 1 taken, the
 // reported residual, the true one (both relative to n), 1 if the FP32 mode keeps
 // the fit (rounds_alike), the square of 1 + the largest |mean| in thermal speeds
@@ -15,9 +15,9 @@ using namespace vl;
 using namespace vl::cf;
 typedef long double LD;
 
-template <class T>
-static void run(int N, double half, double tol, int max_iter, int cases, const double* in, double* out) {
-    FitArgs a;
+static const FitCount kNoCount = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f, false};
+
+static void box_of(int N, double half, double tol, int max_iter, FitArgs& a) {
     std::memset(&a, 0, sizeof a);
     a.nv = N;
     a.tol = tol;
@@ -28,6 +28,12 @@ static void run(int N, double half, double tol, int max_iter, int cases, const d
         a.dv[q] = 2.0 * half / N;
         a.inv_dv[q] = 1.0 / a.dv[q];
     }
+}
+
+template <class T>
+static void run(int N, double half, double tol, int max_iter, int cases, const double* in, double* out) {
+    FitArgs a;
+    box_of(N, half, tol, max_iter, a);
     const LD dv = 2.0L * half / N;
     for (int c = 0; c < cases; ++c) {
         double t[10], u0[3], sg[3], *o = out + 8 * c;
@@ -38,7 +44,7 @@ static void run(int N, double half, double tol, int max_iter, int cases, const d
         typename Jac<T>::type eta0[10];
         float spread;
         Maxw<T> g;
-        FitCount fc = {0, 0u, 0u, 0.f, 0.f, 1.f, false};
+        FitCount fc = kNoCount;
         if (!closed_setup<T>(t, a, u0, sg, b, Tt, eta0, spread)) continue;
         o[0] = closed_fit<T>(g, b, Tt, eta0, nullptr, t[0], a, fc) ? 1.0 : 0.0;
         o[5] = fc.iters;
@@ -80,6 +86,42 @@ static void run(int N, double half, double tol, int max_iter, int cases, const d
         double big = 0.0;
         for (int q = 0; q < 3; ++q) big = std::fmax(big, (double)fabsl(m[q]));
         o[4] = (1.0 + big) * (1.0 + big);
+    }
+}
+
+// FP32 mode: the double-float fits against FP64 fits of the same targets to 4e-15 n.
+// Out per row: 0 refused / 1 taken by both, the largest difference of L and of the
+// means (in standard deviations), that of P (relative), and fit_slack.
+extern "C" void closed_fit_apart(int N, double half, double tol, int max_iter, int cases, const double* in, double* out) {
+    FitArgs a;
+    box_of(N, half, tol, max_iter, a);
+    FitArgs fine = a;
+    fine.tol = 4e-15;
+    for (int c = 0; c < cases; ++c) {
+        double t[10], u0[3], sg[3], v0[3], s0[3], Td[10], ed[10], *o = out + 4 * c;
+        for (int q = 0; q < 10; ++q) t[q] = in[10 * c + q];
+        for (int q = 0; q < 4; ++q) o[q] = 0.0;
+        FitBox<df2> b;
+        FitBox<double> bd;
+        df2 Tt[10];
+        float eta0[10], spread;
+        Maxw<df2> g;
+        Maxw<double> gd;
+        FitCount fc = kNoCount, fd = kNoCount;
+        if (!closed_setup<df2>(t, a, u0, sg, b, Tt, eta0, spread) || !closed_setup<double>(t, fine, v0, s0, bd, Td, ed, spread) ||
+            !closed_fit<df2>(g, b, Tt, eta0, nullptr, t[0], a, fc) || !closed_fit<double>(gd, bd, Td, ed, nullptr, t[0], fine, fd))
+            continue;
+        o[0] = 1.0;
+        o[1] = std::fabs(wide_of(g.L) - gd.L);
+        for (int q = 0; q < 3; ++q)
+            o[1] = std::fmax(o[1], std::fabs((v0[q] - u0[q]) + s0[q] * gd.m[q] - sg[q] * wide_of(g.m[q])) / s0[q]);
+        for (int x = 0; x < 3; ++x)
+            for (int y = x; y < 3; ++y) {
+                const int q = sym(x, y);
+                const double f = (sg[x] / s0[x]) * (sg[y] / s0[y]);
+                o[2] = std::fmax(o[2], std::fabs(wide_of(g.P[q]) / f - gd.P[q]) / std::sqrt(gd.P[sym(x, x)] * gd.P[sym(y, y)]));
+            }
+        o[3] = fit_slack(fc, tol);
     }
 }
 

@@ -37,8 +37,10 @@ def fits(tmp_path_factory):
     def run(arith, N, targets, tol=None, max_iter=20):
         out = np.zeros((len(targets), 8))
         f = getattr(lib, "closed_fit_" + arith)
+        if arith == "apart":
+            out = np.zeros((len(targets), 4))
         f.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double, ctypes.c_int, ctypes.c_int, dp, dp]
-        f(N, 5.0, TOL[arith] if tol is None else tol, max_iter, len(targets), np.ascontiguousarray(targets), out)
+        f(N, 5.0, TOL.get(arith, 1e-11) if tol is None else tol, max_iter, len(targets), np.ascontiguousarray(targets), out)
         return out
 
     return run
@@ -113,3 +115,19 @@ def test_barely_resolved_in_fp64(host, fits, N):  # noqa: F811
     fit = fits("f64", N, tg)
     kept = fit[:, 0] == 1.0
     assert np.all(fit[kept, 2] <= TOL["f64"] + EVAL["f64"] * fit[kept, 4]), fit[kept, 2].max()
+
+
+@pytest.mark.parametrize("N", [12, 16, 20, 24])
+@pytest.mark.parametrize("cells", [(0.6, 1.2), (1.2, 2.5)])
+def test_fits_lie_within_their_slack(fits, N, cells):
+    """FP32 mode keeps a closed-form fit where no line parameter of the exchange can
+    round otherwise within fit_slack of it: 1.5 of it for L and the means, 3 for P
+    (rounds_alike). The exact fit has to lie that close, with Gram sums that leave
+    out up to 1e-3 of the density too."""
+    _, tg = near_faces(np.random.default_rng(47 * N), 1200 if N <= 16 else 300, N, *cells)
+    out = fits("apart", N, tg)
+    both = out[:, 0] == 1.0
+    assert both.sum() > len(tg) // 20
+    o = out[both]
+    assert np.all(o[:, 1] <= 1.5 * o[:, 3]), np.max(o[:, 1] / o[:, 3])
+    assert np.all(o[:, 2] <= 3.0 * o[:, 3]), np.max(o[:, 2] / o[:, 3])
