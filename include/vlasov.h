@@ -319,15 +319,17 @@ vl_status mlp_grad(vl_ctx* ctx, const float* samples_dev, long long n, float* gr
  * iterations, out[1] Newton fallbacks, out[2] clipped cells, out[3] fits
  * whose targets are invalid (empty, non-finite or not positive definite);
  * the work of the double-float 2D3V Newton fits (precision 32; each counted
- * once per fit and evaluation, over the whole velocity block): out[4]
- * double-float moment evaluations (recurrence path), out[5] FP32 Jacobian
+ * once per fit and evaluation): out[4] double-float moment evaluations (closed
+ * form, or recurrences over the whole velocity block), out[5] FP32 Jacobian
  * (Gram) evaluations, out[6] evaluations with one FP64 exponential per
  * velocity cell (wide exponent range), out[7] Newton steps with the FP64
  * Jacobian; out[8] asynchronous tile copies whose wait ran out of time (the
  * fused spatial sweep gives up on such a tile and leaves it unwritten: any
  * nonzero value means the result of that call is invalid); out[9] fits run
  * by the wide double-float kernel; the work of the FP64 fits (precision 64):
- * out[10] moment evaluations, out[11] of which with the Gram sums; out[12]
+ * out[10] moment evaluations, out[11] of which with the Gram sums (evaluations
+ * of a closed-form fit that a direct one replaces count too, its iterations do
+ * not; those of a start that another one replaces do); out[12]
  * fits started from the network's prediction (use_mlp, prediction accepted
  * by the network's input and output range guard). Synchronises the stream. */
 #define VL_NSTATS 13

@@ -109,7 +109,7 @@ CF_FN float log_of(float x) { return logf(x); }
 CF_FN double log_of(double x) { return log(x); }
 
 struct FitCount {
-    int iters;
+    int iters;              // Newton steps, evaluations and those with Gram sums, of every pass
     unsigned evals, grams;
     float last, before;     // size of the last Newton step and of the one before it
     float res, prev;        // residuals after and before the last step (relative to n)
@@ -179,7 +179,6 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
             L0 = L1;
         }
         if (gmax <= tolj) {
-            cnt.iters += it;
             cnt.res = (float)rel;
             return true;
         }
@@ -239,6 +238,7 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
             g.m[a] = add(g.m[a], from(dm[a], z));
         }
         g.L = add(g.L, from(dq, z));
+        ++cnt.iters;
     }
 }
 
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
             }
         }
         left = !good;
-        if (left) fc = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f, false};
+        if (left) fc.iters = 0;  // the direct kernel's are the fit's; evaluations done are work done
     }
     if (kF64) {
         if (left) a.todo[atomicAdd(a.ntodo, 1u)] = (unsigned long long)fit;

@@ -125,6 +125,35 @@ extern "C" void closed_fit_apart(int N, double half, double tol, int max_iter, i
     }
 }
 
+// Newton steps and evaluations of a fit from eta0 (out[0..2]: taken, steps,
+// evaluations) and of the same fit from eta0 + dw first (out[3..5]); the steps that
+// start alone takes with a cap of 40, or 0 where it fails (out[6]).
+extern "C" void closed_fit_started(int N, double half, double tol, int max_iter, int cases, const double* in, const float* dw,
+                                   double* out) {
+    FitArgs a;
+    box_of(N, half, tol, max_iter, a);
+    for (int c = 0; c < cases; ++c) {
+        double t[10], u0[3], sg[3], *o = out + 7 * c;
+        for (int q = 0; q < 10; ++q) t[q] = in[10 * c + q];
+        FitBox<df2> b;
+        df2 Tt[10];
+        float eta0[10], spread;
+        Maxw<df2> g;
+        for (int q = 0; q < 7; ++q) o[q] = 0.0;
+        if (!closed_setup<df2>(t, a, u0, sg, b, Tt, eta0, spread)) continue;
+        for (int start = 0; start < 2; ++start) {
+            FitCount fc = kNoCount;
+            o[3 * start] = closed_fit<df2>(g, b, Tt, eta0, start ? dw + 10 * c : nullptr, t[0], a, fc) ? 1.0 : 0.0;
+            o[3 * start + 1] = fc.iters;
+            o[3 * start + 2] = fc.evals;
+        }
+        float eta[10];
+        FitCount fc = kNoCount;
+        for (int q = 0; q < 10; ++q) eta[q] = eta0[q] + dw[10 * c + q];
+        if (from_eta<df2>(eta, g) && closed_newton<df2, false>(g, b, N, Tt, t[0], tol, 40, fc)) o[6] = fc.iters;
+    }
+}
+
 extern "C" void closed_fit_df2(int N, double half, double tol, int max_iter, int cases, const double* in, double* out) {
     run<df2>(N, half, tol, max_iter, cases, in, out);
 }

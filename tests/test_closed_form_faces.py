@@ -24,14 +24,18 @@ EVAL = {"df2": 5e-13, "f64": 2e-15}
 TOL = {"df2": 1e-11, "f64": 1e-13}
 
 
-@pytest.fixture(scope="module")
-def fits(tmp_path_factory):
+def build_fits(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("fits") / "fits.so")
     inc = tmp_path_factory.mktemp("inc")
     (inc / "cuda_runtime.h").write_text("")
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", str(inc),
                     os.path.join(HERE, "host", "closed_newton_host.cpp"), "-o", so], check=True)
-    lib = ctypes.CDLL(so)
+    return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def fits(tmp_path_factory):
+    lib = build_fits(tmp_path_factory)
     dp = np.ctypeslib.ndpointer(np.float64, flags="C_CONTIGUOUS")
 
     def run(arith, N, targets, tol=None, max_iter=20):
