@@ -22,8 +22,9 @@
 //     the corners' first few cells.
 // About 10 thousand operations instead of 37 N^3. closed_eval refuses (returns
 // false) whatever it cannot give to rounding: means near or beyond a face,
-// strongly correlated or very narrow covariances, heavy corners; such fits
-// take the direct sums (newton.cuh, newton64.cuh).
+// strongly correlated or very narrow covariances, heavy corners, narrow
+// Maxwellians close to a face in FP32 mode; such fits take the direct sums
+// (newton.cuh, newton64.cuh).
 //
 // T is the arithmetic: df2 (double-float pairs on the FP32 pipe, FP32 mode)
 // or double (FP64 mode). J is that of the Jacobian (Gram matrix): float with
@@ -32,8 +33,6 @@
 #pragma once
 
 #include <math.h>
-
-#include <type_traits>
 
 #include "df64.cuh"
 #include "fit_index.cuh"
@@ -482,12 +481,27 @@ CF_FN void far_mode(int q, int& x, int& y, int& z) {
 // They are the product of two small parts, so FP32 gives them where that
 // product is small enough (Limits::tail). A narrow Maxwellian next to a face
 // makes both parts large (0.7 cells per standard deviation, a face at 2: 1e-4 of
-// the density, of which FP32 loses 1e-10): those are summed in FP64, by the
-// evaluation's FINE form, whichever the arithmetic.
+// the density, of which FP32 loses 4e-11): FP64 mode sums those in FP64, and FP32
+// mode leaves such fits to the direct sums (an FP64 form of this kept for them cost
+// every other fit 1 to 4% by its registers).
 template <typename V>
 struct Tail {
     V f, ca, iv, tp, tm, h, ih[3], x[3], r[3], S[6];
 };
+
+template <typename V, typename T>
+CF_FN Tail<V> tail_of(T f, T ca, T iv, T tp, T tm, T h, const T (&ih)[3], const T (&x)[3], const T (&r)[3], const T (&S)[6]) {
+    Tail<V> q = {plain<V>(f), plain<V>(ca), plain<V>(iv), plain<V>(tp), plain<V>(tm), plain<V>(h)};
+    CF_UNROLL
+    for (int c = 0; c < 3; ++c) {
+        q.ih[c] = plain<V>(ih[c]);
+        q.x[c] = plain<V>(x[c]);
+        q.r[c] = plain<V>(r[c]);
+    }
+    CF_UNROLL
+    for (int c = 0; c < 6; ++c) q.S[c] = plain<V>(S[c]);
+    return q;
+}
 
 CF_FN void turn(float y, float& c, float& s) {
     y -= rintf(y);
@@ -501,6 +515,14 @@ CF_FN void tail_modes(int a, const Tail<V>& q, V cut, V (&out)[10]) {
     constexpr V two_pi = V(6.283185307179586476925);
     CF_UNROLL
     for (int d = 0; d < 10; ++d) out[d] = V(0);
+    // first cells, and the ratios to the next ones
+    const V t0[2] = {q.tp, q.tm}, rr = expj(-q.h * q.h * q.iv);
+    V w0[2], r0[2];
+    CF_UNROLL
+    for (int side = 0; side < 2; ++side) {
+        w0[side] = q.ca * expj(V(-0.5) * t0[side] * t0[side] * q.iv);
+        r0[side] = expj(-(t0[side] + V(0.5) * q.h) * q.h * q.iv);
+    }
     CF_LOOP
     for (int m = 0; m < 4; ++m) {
         const V kb = m == 1 ? V(0) : V(1), kc = m == 0 ? V(0) : (m == 3 ? V(-1) : V(1));
@@ -522,9 +544,9 @@ CF_FN void tail_modes(int a, const Tail<V>& q, V cut, V (&out)[10]) {
         turn(om * q.h, cr, sr);
         CF_LOOP
         for (int side = 0; side < 2; ++side) {
-            V t = side ? q.tm : q.tp;
-            V w = q.ca * expj(V(-0.5) * t * t * q.iv), rt = expj(-(t + V(0.5) * q.h) * q.h * q.iv);
-            const V rr = expj(-q.h * q.h * q.iv), sg = side ? V(-1) : V(1);
+            V t = side ? t0[1] : t0[0], w = side ? w0[1] : w0[0], rt = side ? r0[1] : r0[0];
+            if (!(w > cut)) continue;
+            const V sg = side ? V(-1) : V(1);
             V c, s;
             turn(ph + om * sg * t, c, s);
             CF_LOOP
@@ -557,7 +579,9 @@ CF_FN void tail_modes(int a, const Tail<V>& q, V cut, V (&out)[10]) {
         }
     }
 }
-// one far mode's moments 1, d, d d; false where it is below every rounding
+
+// One far mode's moments 1, d, d d. A mode weighs 2 exp(-ex) (1 + 2 ex) of the
+// density at most, of which FP32 loses some 4e-7.
 template <typename V>
 struct Far {
     V n, ih[3], x[3], S[6];
@@ -592,6 +616,29 @@ CF_FN bool far_part(int q, const Far<V>& f, V (&out)[10]) {
     }
     return true;
 }
+CF_FN float far_exponent(int q, const float (&ih)[3], const float (&S)[6]) {
+    int k[3];
+    far_mode(q, k[0], k[1], k[2]);
+    float ex = 0.f;
+    CF_UNROLL
+    for (int a = 0; a < 3; ++a)
+        CF_UNROLL
+        for (int c = 0; c < 3; ++c) ex += (k[a] * ih[a]) * S[sym(a, c)] * (k[c] * ih[c]);
+    return 19.7392088f * ex;
+}
+template <typename V, typename T>
+CF_FN Far<V> far_of(const T& n, const T (&ih)[3], const T (&x)[3], const T (&S)[6]) {
+    Far<V> f;
+    f.n = plain<V>(n);
+    CF_UNROLL
+    for (int a = 0; a < 3; ++a) {
+        f.ih[a] = plain<V>(ih[a]);
+        f.x[a] = plain<V>(x[a]);
+    }
+    CF_UNROLL
+    for (int q = 0; q < 6; ++q) f.S[q] = plain<V>(S[q]);
+    return f;
+}
 
 // limits of a closed-form evaluation, relative to the density: what may be
 // left out, and what may be summed in FP32
@@ -602,22 +649,22 @@ struct Limits<df2> {
     static constexpr float drop = 2e-15f;   // a neglected part
     static constexpr float cut = 1e-19f;    // smallest cell weight of a sum
     static constexpr float fp32 = 3e-7f;    // doubly outside cells (times t^2) summed in FP32
-    static constexpr float tail = 2e-8f;    // tails' and far Poisson modes (times t^2) summed in FP32
+    static constexpr float tail = 3e-7f;    // tails' Poisson modes (times t^2; FP32 loses 4e-7 of it) in FP32
+    static constexpr float far = 0.f;       // exponent of the far modes from which on FP32 does
 };
 template <>
 struct Limits<double> {
     static constexpr float drop = 1e-16f;
     static constexpr float cut = 1e-21f;
     static constexpr float fp32 = 1e-10f;
-    static constexpr float tail = 2e-11f;
+    static constexpr float tail = 1e-9f;
+    static constexpr float far = 26.f;
 };
 
 // Discrete moments (and with gram the Gram sums) of g over the N^3 cells of
-// the box, about its own mean. False where the closed form does not apply, or
-// (coarse) where it takes the FINE form, which sums small parts in FP64 that are
-// too large for FP32.
-template <typename T, bool FINE>
-CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, Eval<T>& e, bool& coarse) {
+// the box, about its own mean. False where the closed form does not apply.
+template <typename T>
+CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, Eval<T>& e) {
     typedef typename Jac<T>::type J;
     typedef Limits<T> Lim;
     const T* P = g.P;
@@ -677,10 +724,6 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
     const bool modes = modes1 > Lim::drop;
     if (modes && !(24.f * (1.f + 240.f * top) * expf(-6.f * kTwoPi2 * lam) <= 4.f * Lim::drop)) return false;
     e.omitted = modes ? 8.f * (1.f + 120.f * top) * expf(-3.f * kTwoPi2 * lam) : 0.f;
-    if (!FINE && e.omitted > Lim::tail) {
-        coarse = true;
-        return false;
-    }
 
     // lattice integral
     const T zero = num<T>(0.0);
@@ -766,29 +809,14 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
         const T nn = neg(np);
         const float weight = modes1 * fmaxf(f0, f2);
         e.omitted = fmaxf(e.omitted, weight);
-        if (!FINE && weight > Lim::tail) {
-            coarse = true;
-            return false;
-        }
-        if (weight > Lim::drop) {
-            typedef typename std::conditional<FINE, double, float>::type V;
-            Tail<V> q;
-            q.f = plain<V>(nn);
-            q.ca = plain<V>(ca);
-            q.iv = plain<V>(iv);
-            q.tp = plain<V>(sub(edge, off));
-            q.tm = plain<V>(add(edge, off));
-            q.h = plain<V>(h);
-            CF_UNROLL
-            for (int c = 0; c < 3; ++c) {
-                q.ih[c] = plain<V>(ihT[c]);
-                q.x[c] = plain<V>(x[c]);
-                q.r[c] = plain<V>(r[c]);
-            }
-            CF_UNROLL
-            for (int c = 0; c < 6; ++c) q.S[c] = plain<V>(Sc[c]);
-            V part[10];
-            tail_modes<V>(a, q, V(Lim::cut), part);
+        if (weight > Lim::tail) {
+            if (sizeof(J) == 4) return false;
+            double part[10];
+            tail_modes<double>(a, tail_of<double>(nn, ca, iv, sub(edge, off), add(edge, off), h, ihT, x, r, Sc), (double)Lim::cut, part);
+            add_moments(e, part);
+        } else if (weight > Lim::drop) {
+            float part[10];
+            tail_modes<float>(a, tail_of<float>(nn, ca, iv, sub(edge, off), add(edge, off), h, ihT, x, r, Sc), Lim::cut, part);
             add_moments(e, part);
         }
         add_low(e, mul(nn, t0), mul(nn, t1), mul(nn, t2), r, Sc);
@@ -1002,31 +1030,20 @@ CF_FN bool closed_sums(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
             }
         }
     }
-    if (modes && 3.f * kTwoPi2 * lam < 48.f) {  // far_part leaves out what is below e^-48
-        typedef typename std::conditional<FINE, double, float>::type V;
-        Far<V> f;
-        f.n = plain<V>(np);
-        CF_UNROLL
-        for (int a = 0; a < 3; ++a) {
-            f.ih[a] = plain<V>(ihT[a]);
-            f.x[a] = plain<V>(x[a]);
-        }
-        CF_UNROLL
-        for (int q = 0; q < 6; ++q) f.S[q] = plain<V>(S[q]);
+    if (modes && 3.f * kTwoPi2 * lam < 48.f) {
+        const Far<float> ff = far_of<float>(np, ihT, x, S);
         CF_LOOP
         for (int q = 0; q < kFarModes; ++q) {
-            V part[10];
-            if (far_part(q, f, part)) add_moments(e, part);
+            if (sizeof(J) == 8 && far_exponent(q, ih, sf) < Lim::far) {
+                double part[10];
+                if (far_part<double>(q, far_of<double>(np, ihT, x, S), part)) add_moments(e, part);
+            } else {
+                float part[10];
+                if (far_part<float>(q, ff, part)) add_moments(e, part);
+            }
         }
     }
     return true;
-}
-
-// either form
-template <typename T>
-CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, Eval<T>& e) {
-    bool coarse = false;
-    return closed_sums<T, false>(g, b, N, gram, e, coarse) || (coarse && closed_sums<T, true>(g, b, N, gram, e, coarse));
 }
 
 }  // namespace cf

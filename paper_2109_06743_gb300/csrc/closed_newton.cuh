@@ -34,12 +34,6 @@
 namespace vl {
 namespace cf {
 
-#ifdef __CUDACC__
-#define CF_CALL __device__ __noinline__
-#else
-#define CF_CALL inline
-#endif
-
 constexpr int kCoefC = 16;
 
 // dl = -J^-1 G, J the Gram matrix packed from the central sums C, by LDL^T
@@ -114,7 +108,6 @@ struct FitCount {
     float last, before;     // size of the last Newton step and of the one before it
     float res, prev;        // residuals after and before the last step (relative to n)
     float omitted;          // largest Eval::omitted of the pass
-    bool coarse;            // an evaluation asked for the FINE form
 };
 
 // thresholds of the direct kernels: damping test above kDamp n, Gram sums with
@@ -125,8 +118,8 @@ CF_FN bool more_steps(float rel, float, float) { return rel > 1e-5f; }
 CF_FN bool more_steps(double rel, double tol, double) { return 100.0 * rel * rel > tol; }
 
 // Newton iteration from g to max |D - Tt| <= tol n. Returns false when the
-// fit is left to the FINE form (cnt.coarse) or to the direct kernels.
-template <typename T, bool FINE>
+// fit is left to the direct kernels.
+template <typename T>
 CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10], double n, double tol,
                          int max_iter, FitCount& cnt) {
     typedef typename Jac<T>::type J;
@@ -137,7 +130,7 @@ CF_FN bool closed_newton(Maxw<T>& g, const FitBox<T>& b, int N, const T (&Tt)[10
     CF_LOOP
     for (int it = 0;; ++it) {
         Eval<T> e;
-        if (!closed_sums<T, FINE>(g, b, N, gram, e, cnt.coarse)) return false;
+        if (!closed_eval<T>(g, b, N, gram, e)) return false;
         ++cnt.evals;
         cnt.grams += gram ? 1u : 0u;
         cnt.omitted = it == 0 ? e.omitted : fmaxf(cnt.omitted, e.omitted);
@@ -341,62 +334,21 @@ CF_FN bool from_eta(const typename Jac<T>::type (&eta)[10], Maxw<T>& g) {
 // warp did not come together again (network-started fits 840 -> 1310 us).
 CF_FN bool predicted(const float* dw) { return dw && fabsf(dw[0]) < 1e30f; }
 
-template <typename T, bool FINE>
-CF_FN bool closed_solve(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const typename Jac<T>::type (&eta0)[10],
-                        const float* dw, double n, const FitArgs& a, FitCount& fc) {
+template <typename T>
+CF_FN bool closed_fit(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const typename Jac<T>::type (&eta0)[10],
+                      const float* dw, double n, const FitArgs& a, FitCount& fc) {
     typedef typename Jac<T>::type J;
     bool good = false;
     CF_LOOP
-    for (int pass = predicted(dw) ? 0 : 1; pass < 2 && !good && !fc.coarse; ++pass) {
+    for (int pass = predicted(dw) ? 0 : 1; pass < 2 && !good; ++pass) {
         J eta[10];
         CF_UNROLL
         for (int q = 0; q < 10; ++q) {
             const float d = pass == 0 ? dw[q] : 0.f;
             eta[q] = eta0[q] + (fabsf(d) < 1e30f ? (J)d : J(0));
         }
-        good = from_eta<T>(eta, g) && closed_newton<T, FINE>(g, b, a.nv, Tt, n, a.tol, a.max_iter, fc);
+        good = from_eta<T>(eta, g) && closed_newton<T>(g, b, a.nv, Tt, n, a.tol, a.max_iter, fc);
     }
-    return good;
-}
-
-// The same in the FINE form, out of line and on copies: few fits take it, and its
-// code and registers stay out of the common path (called from within the
-// evaluation it cost the other fits 4.5%, so less than 1%).
-template <typename T>
-struct FineFit {
-    Maxw<T> g;
-    FitBox<T> b;
-    T Tt[10];
-    typename Jac<T>::type eta0[10];
-    const float* dw;
-    double n;
-    FitCount fc;
-};
-template <typename T>
-CF_CALL bool closed_solve_fine(FineFit<T>& f, const FitArgs& a) {
-    return closed_solve<T, true>(f.g, f.b, f.Tt, f.eta0, f.dw, f.n, a, f.fc);
-}
-
-// the fit in the form it needs
-template <typename T>
-CF_FN bool closed_fit(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const typename Jac<T>::type (&eta0)[10],
-                      const float* dw, double n, const FitArgs& a, FitCount& fc) {
-    if (closed_solve<T, false>(g, b, Tt, eta0, dw, n, a, fc)) return true;
-    if (!fc.coarse) return false;
-    FineFit<T> f;
-    f.b = b;
-    CF_UNROLL
-    for (int q = 0; q < 10; ++q) {
-        f.Tt[q] = Tt[q];
-        f.eta0[q] = eta0[q];
-    }
-    f.dw = dw;
-    f.n = n;
-    f.fc = fc;
-    f.fc.coarse = false;
-    const bool good = closed_solve_fine<T>(f, a);
-    g = f.g;
-    fc = f.fc;
     return good;
 }
 
@@ -411,8 +363,9 @@ CF_FN bool closed_fit(Maxw<T>& g, const FitBox<T>& b, const T (&Tt)[10], const t
 // direct kernels over 1.6e5 fits of the workloads: 5e-13, 1.8e-6 of the step, the
 // residual or the step). Where the Gram sums leave out more than FP32 resolves
 // (Eval::omitted; narrow Maxwellians near a face, two faces at once), the last step
-// leaves a remainder of the size of the residual rather than 2e-6 of the step, and
-// the direct kernel may need a step less: what is left out, times the step before.
+// may leave a remainder of the size of the residual rather than 2e-6 of the step,
+// and the direct kernel may need a step less: what is left out, times the step
+// before.
 CF_FN double fit_slack(const FitCount& fc, double tol) {
     const double last = fc.last, res = fc.res;
     double eps = 8e-13 + 2e-6 * last;
@@ -462,7 +415,7 @@ CF_FN bool rounds_alike(const Maxw<T>& g, const FitBox<T>& b, const double (&u0)
 // direct kernels are appended to a.todo. With a.sel the kernel also reduces
 // what chooses the direct kernel (see kernels.cuh).
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 2) closed_fit_kernel(const __grid_constant__ FitArgs a) {
+__global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 2) closed_fit_kernel(FitArgs a) {
     typedef typename Jac<T>::type J;
     constexpr bool kF64 = sizeof(J) == 8;
     __shared__ unsigned long long cnt[VL_NSTATS];
@@ -470,7 +423,7 @@ __global__ void __launch_bounds__(128, sizeof(typename Jac<T>::type) == 4 ? 3 : 
     __syncthreads();
     const long long fit = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool have = fit < 2 * a.ncell;
-    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f, false};
+    FitCount fc = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f};
     bool left = false, empty = false;
     unsigned warm = 0u;
     unsigned long long top = 0ull, wide = 0ull;

@@ -15,7 +15,7 @@ using namespace vl;
 using namespace vl::cf;
 typedef long double LD;
 
-static const FitCount kNoCount = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f, false};
+static const FitCount kNoCount = {0, 0u, 0u, 0.f, 0.f, 0.f, 1.f, 0.f};
 
 static void box_of(int N, double half, double tol, int max_iter, FitArgs& a) {
     std::memset(&a, 0, sizeof a);
@@ -150,7 +150,7 @@ extern "C" void closed_fit_started(int N, double half, double tol, int max_iter,
         float eta[10];
         FitCount fc = kNoCount;
         for (int q = 0; q < 10; ++q) eta[q] = eta0[q] + dw[10 * c + q];
-        if (from_eta<df2>(eta, g) && closed_newton<df2, false>(g, b, N, Tt, t[0], tol, 40, fc)) o[6] = fc.iters;
+        if (from_eta<df2>(eta, g) && closed_newton<df2>(g, b, N, Tt, t[0], tol, 40, fc)) o[6] = fc.iters;
     }
 }
 
