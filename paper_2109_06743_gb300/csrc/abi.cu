@@ -597,7 +597,7 @@ vl_status moment_fit_solve(vl_ctx* ctx, int s, const double* vmom, int use_mlp, 
     // closed-form fits first, the direct kernels take what they leave; a
     // forced choice of the direct kernel (moment_fit_wide) runs it alone
     if (d.nvdim == 3 && (a.fp64 || a.wide < 0)) {
-        const bool closed = a.nv >= vl::kClosedMin;
+        const bool closed = vl::closed_first(a.nv, a.ncell, a.fp64 != 0);
         if (closed || !a.fp64) {
             st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 3 * sizeof(unsigned long long), cs),
                             "moment_fit (kernel choice)");

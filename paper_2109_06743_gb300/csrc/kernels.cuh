@@ -146,12 +146,30 @@ struct FitArgs {
                             // a target is not finite or has n < 0; may be null
 };
 cudaError_t launch_fit(const FitArgs& a, int nvdim, cudaStream_t st);
-// the closed-form fits (closed_fit.cu): sel, ntodo zeroed by the caller. For
-// blocks of kClosedMin^3 and more: an 8^3 block of +-5 thermal speeds resolves
-// them with 0.8 cells each, where the Poisson modes of the tails' corners
-// matter and most fits are refused (measured with the closed form tried first:
-// 8192 FP32 fits of Harris ions 222 -> 307 us, 16384 FP64 fits 3.34 -> 3.63 ms)
+// the closed-form fits (closed_fit.cu): sel, ntodo zeroed by the caller.
+//
+// closed_first: are a species' fits tried in closed form, or fitted by the direct
+// kernels at once?
+// * 8^3 blocks, direct: +-5 thermal speeds are resolved with 0.8 cells each, where
+//   the Poisson modes of the tails' corners matter and most fits are refused (closed
+//   form first: 8192 FP32 fits of Harris ions 222 -> 307 us, 16384 FP64 fits 3.34 ->
+//   3.63 ms).
+// * Few fits, direct: a thread per fit is a chain that takes as long for one fit as
+//   for ten thousand, eight lanes (FP64: a warp) per fit are done sooner while they
+//   all fit on the chip. us, closed form / direct, isotropic and strongly correlated
+//   (rho 0.3) Maxwellians, 2 fits a cell:
+//     FP64 12^3: 512 cells 566 / 386, 1697 / 385; 1024 cells 567 / 736, 1698 / 736
+//          16^3: 512 cells 452 / 429, 1620 / 428; 1024 cells 453 / 793, 1620 / 794
+//          20^3: 256 cells 510 / 437, 1903 / 435; 512 cells 514 / 697, 1964 / 698
+//          24^3: 256 cells 555 / 541, 2421 / 542; 512 cells 791 / 886, 2510 / 886
+//     FP32 12^3: 1024 cells 278 / 143, 388 / 764; 2048 cells 279 / 161; 4096 cells 281 /
+//          229, cold ones 372 / 391. Larger blocks: 16^3 at 256 cells 153 / 192.
 constexpr int kClosedMin = 12;
+inline bool closed_first(int nv, long long ncell, bool fp64) {
+    if (nv < kClosedMin) return false;
+    if (fp64) return ncell > (nv <= 16 ? 512 : 256);
+    return nv > 12 || ncell > 2048;
+}
 cudaError_t launch_closed_fit(const FitArgs& a, cudaStream_t st);
 
 // ---- MLP warm start (mlp.cu) ------------------------------------------------------

@@ -3,9 +3,9 @@
 // newton64.cuh: plain FP64); each size is instantiated in its own
 // translation unit (newton_<N>.cu) so that the build compiles them in
 // parallel. With a.ntodo the closed-form kernel (closed_fit.cu) runs first
-// and these direct kernels take the fits it leaves. Blocks of 8^3, which it
-// mostly refuses, go to the direct kernels at once (fit_select_kernel chooses
-// between the two double-float ones).
+// and these direct kernels take the fits it leaves. Blocks of 8^3 and few fits go to
+// the direct kernels at once (closed_first; fit_select_kernel chooses between the two
+// double-float ones).
 #include "kernels.cuh"
 
 namespace vl {

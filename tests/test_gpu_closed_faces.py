@@ -58,8 +58,8 @@ def test_converged_fits_meet_the_tolerance(fits, precision, nv):  # noqa: F811
     if not torch.cuda.is_available():
         pytest.fail("GPU tests need a CUDA device")
     arith = "df2" if precision == 32 else "f64"
-    # more cells than the direct kernels take at once in FP64 mode
-    cfg = W.harris(nx=64, ny=17, nv=nv, lx=3.2, ly=0.85, precision=precision)
+    # more cells than the direct kernels take at once
+    cfg = W.harris(nx=128, ny=17, nv=nv, lx=6.4, ly=0.85, precision=precision)
     cfg.fit_tol = TOL[arith]
     nc, k = cfg.ncell, 1
     sp = cfg.species[k]
