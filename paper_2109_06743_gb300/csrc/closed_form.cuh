@@ -451,6 +451,141 @@ CF_FN bool corner_sums(J ap, J am, J bp, J bm, J ha, J hb, J Qaa, J Qab, J Qbb, 
     return ok;
 }
 
+// a row of two corners from its cell v outward, ratio r to the next one
+struct Two {
+    float x, y;
+};
+CF_FN void light_row(Two v, Two r, float rr, float tb, float h, float cut, float (&s0)[2], float (&s1)[2], float (&s2)[2]) {
+    s0[0] = s0[1] = s1[0] = s1[1] = s2[0] = s2[1] = 0.f;
+    CF_LOOP
+    for (int j = 0; j < kMaxTail && larger(v.x, v.y) > cut; ++j) {
+        const float a = v.x * tb, b = v.y * tb;
+        s0[0] += v.x;
+        s0[1] += v.y;
+        s1[0] += a;
+        s1[1] += b;
+        s2[0] = fmaf(a, tb, s2[0]);
+        s2[1] = fmaf(b, tb, s2[1]);
+        v.x *= r.x;
+        v.y *= r.y;
+        r.x *= rr;
+        r.y *= rr;
+        tb += h;
+    }
+}
+
+// The same for heavy corners in FP64 mode: cells above heavy in FP64, lighter ones
+// (1e-11 of the lattice integral: FP32 rounds them at 1e-17) and what a row or a
+// corner has beyond them in FP32, whose chains are several times as short. All in
+// FP64 the corners of strongly correlated fits took three quarters of the time
+// (2048 fits of 16^3 1621 -> 1190 us, 24^3 2510 -> 1552).
+template <typename J>
+CF_FN bool corner_sums_mixed(J ap, J am, J bp, J bm, J ha, J hb, J Qaa, J Qab,
+                             J Qbb, const J (&w4)[4], float cut, J (&t)[6]) {
+    constexpr J heavy = J(1e-11);
+    CF_UNROLL
+    for (int q = 0; q < 6; ++q) t[q] = J(0);
+    const J raa = expj(-Qaa * ha * ha), rbb = expj(-Qbb * hb * hb), ea = expj(-Qab * ha * hb), eb = expj(Qab * ha * hb);
+    const float raaf = (float)raa, rbbf = (float)rbb, haf = (float)ha, hbf = (float)hb;
+    bool ok = true;
+    CF_LOOP
+    for (int side = 0; side < 2; ++side) {
+        const J tb0 = side ? bm : bp;
+        J w[2] = {side ? w4[2] : w4[0], side ? w4[3] : w4[1]};
+        J ta[2] = {ap, am}, ra[2], rb[2], rab[2] = {side ? eb : ea, side ? ea : eb};
+        CF_UNROLL
+        for (int c = 0; c < 2; ++c) {
+            const J qab = (c != side) ? -Qab : Qab;
+            const J la = -(Qaa * ta[c] + qab * tb0) * ha, lb = -(Qbb * tb0 + qab * ta[c]) * hb;
+            ok = ok && la < J(0) && lb < J(0);
+            ra[c] = expj(la - J(0.5) * Qaa * ha * ha);
+            rb[c] = expj(lb - J(0.5) * Qbb * hb * hb);
+        }
+        if (!ok) return false;
+        J c0[2] = {J(0), J(0)}, c1a[2] = {J(0), J(0)}, c1b[2] = {J(0), J(0)}, c2a[2] = {J(0), J(0)}, c2m[2] = {J(0), J(0)},
+               c2b[2] = {J(0), J(0)};
+        int i = 0;
+        CF_LOOP
+        for (; i < kMaxTail && larger(w[0], w[1]) > heavy; ++i) {
+            J v[2] = {w[0], w[1]}, r[2] = {rb[0], rb[1]}, tb = tb0;
+            J s0[2] = {J(0), J(0)}, s1[2] = {J(0), J(0)}, s2[2] = {J(0), J(0)};
+            int j = 0;
+            CF_LOOP
+            for (; j < kMaxTail && larger(v[0], v[1]) > heavy; ++j) {
+                CF_UNROLL
+                for (int c = 0; c < 2; ++c) {
+                    const J vt = v[c] * tb;
+                    s0[c] += v[c];
+                    s1[c] += vt;
+                    s2[c] += vt * tb;
+                    v[c] *= r[c];
+                    r[c] *= rbb;
+                }
+                tb += hb;
+            }
+            float f0[2], f1[2], f2[2];
+            light_row({(float)v[0], (float)v[1]}, {(float)r[0], (float)r[1]}, rbbf, (float)tb, hbf, cut, f0, f1, f2);
+            CF_UNROLL
+            for (int c = 0; c < 2; ++c) {
+                s0[c] += f0[c];
+                s1[c] += f1[c];
+                const J ts = ta[c] * s0[c];
+                c0[c] += s0[c];
+                c1a[c] += ts;
+                c1b[c] += s1[c];
+                c2a[c] += ta[c] * ts;
+                c2m[c] += ta[c] * s1[c];
+                c2b[c] += s2[c] + f2[c];
+                w[c] *= ra[c];
+                ra[c] *= raa;
+                rb[c] *= rab[c];
+                ta[c] += ha;
+            }
+        }
+        float wf[2], raf[2], rbf[2], rabf[2], taf[2];
+        CF_UNROLL
+        for (int c = 0; c < 2; ++c) {
+            wf[c] = (float)w[c];
+            raf[c] = (float)ra[c];
+            rbf[c] = (float)rb[c];
+            rabf[c] = (float)rab[c];
+            taf[c] = (float)ta[c];
+        }
+        float d0[2] = {0.f, 0.f}, d1a[2] = {0.f, 0.f}, d1b[2] = {0.f, 0.f}, d2a[2] = {0.f, 0.f}, d2m[2] = {0.f, 0.f},
+              d2b[2] = {0.f, 0.f};
+        CF_LOOP
+        for (; i < kMaxTail && larger(wf[0], wf[1]) > cut; ++i) {
+            float f0[2], f1[2], f2[2];
+            light_row({wf[0], wf[1]}, {rbf[0], rbf[1]}, rbbf, (float)tb0, hbf, cut, f0, f1, f2);
+            CF_UNROLL
+            for (int c = 0; c < 2; ++c) {
+                const float ts = taf[c] * f0[c];
+                d0[c] += f0[c];
+                d1a[c] += ts;
+                d1b[c] += f1[c];
+                d2a[c] += taf[c] * ts;
+                d2m[c] += taf[c] * f1[c];
+                d2b[c] += f2[c];
+                wf[c] *= raf[c];
+                raf[c] *= raaf;
+                rbf[c] *= rabf[c];
+                taf[c] += haf;
+            }
+        }
+        CF_UNROLL
+        for (int c = 0; c < 2; ++c) {
+            const J sa = c ? J(-1) : J(1), sb = side ? J(-1) : J(1);
+            t[0] += c0[c] + d0[c];
+            t[1] += sa * (c1a[c] + d1a[c]);
+            t[2] += sb * (c1b[c] + d1b[c]);
+            t[3] += c2a[c] + d2a[c];
+            t[4] += sa * sb * (c2m[c] + d2m[c]);
+            t[5] += c2b[c] + d2b[c];
+        }
+    }
+    return ok;
+}
+
 // modes beyond |k|^2 = 2, one of each pair +-k, with |k|^2 <= 5
 constexpr int kFarModes = 19;
 CF_FN void far_mode(int q, int& x, int& y, int& z) {
@@ -857,7 +992,7 @@ CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
             wtop = fmaxf(wtop, w4[c]);
         }
         const T Taa = a ? S[3] : S[0], Tbb = p == 0 ? S[3] : S[5], Tab = pick(p, S[1], S[2], S[4]);
-        if (wtop > 3e-10f) {
+        if (sizeof(J) == 4 && wtop > 3e-10f) {
             // heavy corners: the FP32 exponent (about 16, to 1e-6) is not enough
             const T di = inv(sub(mul(Taa, Tbb), mul(Tab, Tab)));
             const T qaa = mul(Tbb, di), qbb = mul(Taa, di), qab = neg(mul(Tab, di));
@@ -894,7 +1029,7 @@ CF_FN bool closed_eval(const Maxw<T>& g, const FitBox<T>& b, int N, bool gram, E
                 const J ta = (c & 1) ? jam : jap, tb = (c & 2) ? jbm : jbp, q2 = (c == 1 || c == 2) ? J(-2) * qab : J(2) * qab;
                 j4[c] = nrm * expj(J(-0.5) * (qaa * ta * ta + q2 * ta * tb + qbb * tb * tb));
             }
-            if (!corner_sums<J>(jap, jam, jbp, jbm, Ha, Hb, qaa, qab, qbb, j4, J(Lim::cut), t)) return false;
+            if (!corner_sums_mixed<J>(jap, jam, jbp, jbm, Ha, Hb, qaa, qab, qbb, j4, Lim::cut, t)) return false;
         } else {
             if (!(weight <= (sizeof(J) == 8 ? 1.f : Lim::fp32))) return false;
             CF_UNROLL
