@@ -103,7 +103,7 @@ Layout layout_of(const vl_desc& d) {
     L.u2 = off; off = align256(off + nc * 10 * sizeof(double));
     L.cur = off; off = align256(off + nc * 3 * sizeof(double));
     L.counters = off; off = align256(off + VL_NSTATS * sizeof(unsigned long long));
-    L.select = off; off = align256(off + 3 * sizeof(unsigned long long));
+    L.select = off; off = align256(off + 4 * sizeof(unsigned long long));
     L.todo = off; off = align256(off + nc * 2 * sizeof(unsigned long long));
     const size_t np = (size_t)VL_MLP_NPARAM * sizeof(float);
     L.mlp_w = off; off = align256(off + np);
@@ -593,13 +593,14 @@ vl_status moment_fit_solve(vl_ctx* ctx, int s, const double* vmom, int use_mlp, 
     a.sel = nullptr;
     a.todo = nullptr;
     a.ntodo = nullptr;
+    a.next = nullptr;
     cudaStream_t cs = (cudaStream_t)stream;
     // closed-form fits first, the direct kernels take what they leave; a
     // forced choice of the direct kernel (moment_fit_wide) runs it alone
     if (d.nvdim == 3 && (a.fp64 || a.wide < 0)) {
         const bool closed = vl::closed_first(a.nv, a.ncell, a.fp64 != 0);
         if (closed || !a.fp64) {
-            st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 3 * sizeof(unsigned long long), cs),
+            st = cuda_check(ctx, cudaMemsetAsync(ctx->ws.fit_select, 0, 4 * sizeof(unsigned long long), cs),
                             "moment_fit (kernel choice)");
             if (st != VL_OK) return st;
         }
@@ -607,6 +608,7 @@ vl_status moment_fit_solve(vl_ctx* ctx, int s, const double* vmom, int use_mlp, 
         if (closed) {
             a.todo = ctx->ws.fit_todo;
             a.ntodo = reinterpret_cast<unsigned*>(ctx->ws.fit_select + 2);
+            a.next = ctx->ws.fit_select + 3;
         }
     }
     if (use_mlp) {

@@ -41,8 +41,8 @@ struct Workspace {
     double* fluid_l;      // [ncell][10]
     double* cur;          // [ncell][3] current density at cell centres
     unsigned long long* counters;  // [VL_NSTATS]
-    unsigned long long* fit_select;  // [3] device-side choice of the direct fit kernel, then the number of
-                          // entries left to it
+    unsigned long long* fit_select;  // [4] device-side choice of the direct fit kernel, then the number of
+                          // entries left to it and the next of them
     unsigned long long* fit_todo;  // [2 ncell] those fits
     float* mlp;           // MLP weights and scratch
 };

@@ -140,13 +140,14 @@ struct FitArgs {
                             // fits, 2 cell + (0: V, 1: F). FP32 mode: units of four cells' V or F
                             // fits, (2 (cell / 4) + (0: V, 1: F)) * 16 + a bit per cell to be kept
     unsigned* ntodo;        // their number; null: the direct kernels fit every cell
+    unsigned long long* next;  // FP32 mode: the next entry of a long list
     double inv_dv[3];
     int fp64;               // 1: the plain FP64 fit (FP64 mode), 0: double-float on the FP32 pipe
     int* numeric;           // status word (device-visible host memory): set to VL_ENUMERIC when
                             // a target is not finite or has n < 0; may be null
 };
 cudaError_t launch_fit(const FitArgs& a, int nvdim, cudaStream_t st);
-// the closed-form fits (closed_fit.cu): sel, ntodo zeroed by the caller.
+// the closed-form fits (closed_fit.cu): sel, ntodo, next zeroed by the caller.
 //
 // closed_first: are a species' fits tried in closed form, or fitted by the direct
 // kernels at once?

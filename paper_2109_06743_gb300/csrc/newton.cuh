@@ -1631,7 +1631,10 @@ __global__ void __launch_bounds__(128, WIDE ? 3 : 4) newton_kernel(FitArgs a) {
 // hence the same bits, whoever asked for it. The list is usually short (a few
 // units in a thousand), and then what counts is the latency of one fit, a chain
 // of some 80 k instructions with eight lanes per cell: up to kShortList units
-// each get a CTA, a warp per cell. A longer list is fitted a warp per unit.
+// each get a CTA, a warp per cell. A longer list is fitted a warp per unit, and a
+// warp takes the next one when it is done: units take uneven time (131072 fits of
+// 12^3, all left: narrow ones 111 ms by equal shares, 93 now, 99 without a closed-form
+// attempt; correlated ones 47, 43 and 45).
 constexpr long long kShortList = 912;  // two waves of 3 CTAs per SM
 template <int N, bool WIDE>
 __global__ void __launch_bounds__(128, 3) newton_list_kernel(FitArgs a) {
@@ -1659,7 +1662,11 @@ __global__ void __launch_bounds__(128, 3) newton_list_kernel(FitArgs a) {
         }
     } else {
         const int slot = threadIdx.x / kG, c = slot & 3;
-        for (long long k = (long long)blockIdx.x * 4 + (threadIdx.x >> 5); k < units; k += (long long)gridDim.x * 4) {
+        for (;;) {
+            unsigned long long k = 0;
+            if ((threadIdx.x & 31) == 0) k = atomicAdd(a.next, 1ull);
+            k = __shfl_sync(0xffffffffu, k, 0);
+            if (k >= (unsigned long long)units) break;
             const unsigned long long entry = a.todo[k];
             const long long cell = (long long)(entry >> 5) * 4 + c;
             const bool have = cell < a.ncell, keep = have && ((entry >> c) & 1ull) != 0;
