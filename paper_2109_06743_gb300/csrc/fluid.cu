@@ -111,9 +111,8 @@ __device__ __forceinline__ void closure_e3(const R* s, R* e3) {
 // per stage however small the grid; here a point is formed 1.25-1.4 times and
 // 256 threads share a tile. Measured (GB300): one FP32 step (three stages) of
 // 128 x 64 cells 180 -> 37 us; the closure model's step of 64 x 64 cells in
-// FP64, both species and fields, 1257 -> 330 us; same bits. Tiles of 8 x 8
-// cells where they fill the chip twice (1.25 points formed per point used),
-// else 8 x 4 (1.38, but more CTAs).
+// FP64, both species and fields, 1257 -> 330 us; same bits. Shapes: tile_shape
+// (8 x 8 forms 1.25 points per point used, 8 x 4 1.38, 32 x 1 2.03).
 constexpr int kTileThreads = 256;
 template <typename R, int TX, int TY>
 struct FluidTile {
@@ -373,6 +372,30 @@ static cudaError_t launch_tile(const FluidArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <int TX, int TY>
+static cudaError_t launch_shape(const FluidArgs& a, cudaStream_t st) {
+    if (a.closure) return a.precision == 64 ? launch_tile<double, true, TX, TY>(a, st) : launch_tile<float, true, TX, TY>(a, st);
+    return a.precision == 64 ? launch_tile<double, false, TX, TY>(a, st) : launch_tile<float, false, TX, TY>(a, st);
+}
+
+// The shape of the tiles: the one that forms fewest points on this grid, once the
+// chip has work for two CTAs per SM, else 8 x 4 (more CTAs). A few rows or columns
+// of cells fill 8 x 8 tiles badly: one FP64 step of 65535 x 1 cells 14.1 ms, in 32 x
+// 1 tiles 3.1; 1 x 65535 14.2, in 1 x 32 3.1; 16384 x 3 3.7, in 8 x 4 2.1 (a thread per
+// cell: 3.7, 3.7 and 2.7).
+static int tile_shape(int nx, int ny) {
+    constexpr int tx[4] = {8, 8, 32, 1}, ty[4] = {4, 8, 1, 32};
+    int best = 0;
+    long long least = 0;
+    for (int q = 0; q < 4; ++q) {
+        const long long tiles = (long long)((nx + tx[q] - 1) / tx[q]) * ((ny + ty[q] - 1) / ty[q]);
+        const long long points = tiles * ((tx[q] + 2) * ty[q] + tx[q] * (ty[q] + 2));
+        if (q == 0) least = points;
+        if (q > 0 && tiles >= 2 * 152 && points <= least) least = points, best = q;
+    }
+    return best;
+}
+
 cudaError_t launch_fluid_stage(const FluidArgs& args, cudaStream_t st) {
     FluidArgs a = args;
     a.invdx = 1.0 / a.dx;
@@ -386,16 +409,12 @@ cudaError_t launch_fluid_stage(const FluidArgs& args, cudaStream_t st) {
         count_launch();
         return cudaGetLastError();
     }
-    // 8 x 8 tiles once there are two per SM
-    const bool large = (long long)((a.nx + 7) / 8) * ((a.ny + 7) / 8) >= 2 * 152;
-    if (a.closure) {
-        if (a.precision == 64)
-            return large ? launch_tile<double, true, 8, 8>(a, st) : launch_tile<double, true, 8, 4>(a, st);
-        return large ? launch_tile<float, true, 8, 8>(a, st) : launch_tile<float, true, 8, 4>(a, st);
+    switch (tile_shape(a.nx, a.ny)) {
+        case 0: return launch_shape<8, 4>(a, st);
+        case 1: return launch_shape<8, 8>(a, st);
+        case 2: return launch_shape<32, 1>(a, st);
+        default: return launch_shape<1, 32>(a, st);
     }
-    if (a.precision == 64)
-        return large ? launch_tile<double, false, 8, 8>(a, st) : launch_tile<double, false, 8, 4>(a, st);
-    return large ? launch_tile<float, false, 8, 8>(a, st) : launch_tile<float, false, 8, 4>(a, st);
 }
 
 }  // namespace vl
