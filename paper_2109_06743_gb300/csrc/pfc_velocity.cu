@@ -921,8 +921,15 @@ __global__ void moments_kernel(MomentArgs a) {
 // One warp per spatial cell (lines of at most 64 velocities, two to a lane): a
 // thread per cell was a chain of some 500 FP64 instructions for 32 velocities
 // on two warps of one SM (64 cells: the step 24 us, 5 now; the moments 13 us,
-// 4 now).
+// 4 now). A thread per cell again where there are cells enough to fill the chip
+// with threads: a warp leaves most lanes idle on short lines, and its shuffles
+// cost more than the sums. us, warps / threads, FP64:
+//   4 velocities:  512 cells step 6 / 8, moments 4 / 4; 1024 10 / 8, 6 / 4; 4096 25 / 8, 10 / 4
+//   16: 2048 cells 14 / 21, 8 / 8; 4096 25 / 21, 10 / 8; 65535 330 / 64, 126 / 27
+//   32: 4096 cells 25 / 37, 10 / 14; 16384 87 / 40, 35 / 17; 65535 330 / 115, 126 / 48
+//   64: 4096 cells 31 / 68, 12 / 25; 16384 107 / 70, 44 / 27; 65535 412 / 218, 160 / 89
 constexpr int kLine1d = 64, kWarps1d = 4;
+static bool threads1d(long long ncell, int nv) { return ncell >= 512 + 128LL * nv; }
 
 // moments 1, v, v^2, v^3 of the line x(q), q = 0 .. n - 1
 template <typename F>
@@ -938,6 +945,16 @@ __device__ __forceinline__ void line_moments1d(F x, int n, double vmin, double d
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m[p] += __shfl_xor_sync(0xffffffffu, m[p], o);
     if (lane < 4) out[lane] = (lane == 0 ? m[0] : (lane == 1 ? m[1] : (lane == 2 ? m[2] : m[3]))) * dv;
+}
+
+template <typename T>
+__device__ __forceinline__ void cell_moments1d(const T* f, int n, double vmin, double dv, double* out) {
+    double m[4] = {0, 0, 0, 0};
+    for (int q = 0; q < n; ++q) {
+        const double v = vmin + (q + 0.5) * dv, x = (double)f[q];
+        m[0] += x; m[1] += v * x; m[2] += v * v * x; m[3] += v * v * v * x;
+    }
+    for (int p = 0; p < 4; ++p) out[p] = m[p] * dv;
 }
 
 // zero-flux PFC step of the velocity line with c = (q/m) E dt / dv
@@ -991,6 +1008,49 @@ __global__ void __launch_bounds__(32 * kWarps1d) moments1d_kernel(MomentArgs a) 
     if (c >= a.ncell) return;
     const T* f = reinterpret_cast<const T*>(a.f) + c * a.nv;
     line_moments1d([&](int q) { return f[q]; }, a.nv, a.vmin[0], a.dv[0], a.mom_out + c * 4);
+}
+
+// the same by a thread per cell, straight from global memory
+template <typename T>
+__global__ void velocity1d_cells_kernel(VelocityArgs a) {
+    long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (c >= a.ncell) return;
+    T* f = reinterpret_cast<T*>(a.f) + c * a.nv;
+    const int n = a.nv;
+    double cc = a.qm * a.eb[c * 6] * a.dt / a.dv[0];
+    bool fwd = cc >= 0.0;
+    double ca = fwd ? cc : -cc;
+    if (!(ca < (double)n)) ca = (double)n;
+    int s = (int)floor(ca);
+    T alpha = (T)(ca - s);
+    const T A = (T(1) - alpha) * (T(2) - alpha) / T(6);
+    const T B = (T(1) - alpha) * (T(1) + alpha) / T(6);
+    T g[kLine1d];
+    auto at = [&](int q) -> T { return (q < 0 || q >= n) ? T(0) : f[fwd ? q : n - 1 - q]; };
+    T phi_prev = T(0), phi = T(0);
+    for (int q = 0; q < n; ++q) {
+        phi = phi_lim<T>(alpha, A, B, at(q - 1), at(q), at(q + 1));
+        g[q] = at(q) - phi + phi_prev;
+        phi_prev = phi;
+    }
+    T acc = T(0);
+    for (int p = 0; p < n; ++p) {
+        int q = p - s;
+        T v = (q >= 0) ? g[q] : T(0);
+        if (p == n - 1) {
+            for (int qq = (q >= 0 ? q : 0); qq < n; ++qq) acc += g[qq];
+            v = acc + phi;
+        }
+        f[fwd ? p : n - 1 - p] = v;
+    }
+    if (a.mom_out) cell_moments1d(f, n, a.vmin[0], a.dv[0], a.mom_out + c * 4);
+}
+
+template <typename T>
+__global__ void moments1d_cells_kernel(MomentArgs a) {
+    long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (c >= a.ncell) return;
+    cell_moments1d(reinterpret_cast<const T*>(a.f) + c * a.nv, a.nv, a.vmin[0], a.dv[0], a.mom_out + c * 4);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -1066,6 +1126,13 @@ static cudaError_t launch_moments_n(const MomentArgs& a, cudaStream_t st) {
     }
 
 cudaError_t launch_velocity(const VelocityArgs& a, int nvdim, int precision, cudaStream_t st) {
+    if (nvdim == 1 && threads1d(a.ncell, a.nv)) {
+        const unsigned grid = (unsigned)((a.ncell + 127) / 128);
+        if (precision == 64) velocity1d_cells_kernel<double><<<grid, 128, 0, st>>>(a);
+        else velocity1d_cells_kernel<float><<<grid, 128, 0, st>>>(a);
+        count_launch();
+        return cudaGetLastError();
+    }
     if (nvdim == 1) {
         const unsigned grid = (unsigned)((a.ncell + kWarps1d - 1) / kWarps1d);
         if (precision == 64) velocity1d_kernel<double><<<grid, 32 * kWarps1d, 0, st>>>(a);
@@ -1093,6 +1160,13 @@ cudaError_t launch_velocity(const VelocityArgs& a, int nvdim, int precision, cud
 }
 
 cudaError_t launch_moments(const MomentArgs& a, int nvdim, int precision, cudaStream_t st) {
+    if (nvdim == 1 && threads1d(a.ncell, a.nv)) {
+        const unsigned grid = (unsigned)((a.ncell + 127) / 128);
+        if (precision == 64) moments1d_cells_kernel<double><<<grid, 128, 0, st>>>(a);
+        else moments1d_cells_kernel<float><<<grid, 128, 0, st>>>(a);
+        count_launch();
+        return cudaGetLastError();
+    }
     if (nvdim == 1) {
         const unsigned grid = (unsigned)((a.ncell + kWarps1d - 1) / kWarps1d);
         if (precision == 64) moments1d_kernel<double><<<grid, 32 * kWarps1d, 0, st>>>(a);
