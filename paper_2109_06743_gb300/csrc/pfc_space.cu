@@ -244,8 +244,9 @@ cudaError_t launch_pfc_space(const SpaceSweepArgs& a, int precision, cudaStream_
     // than SMs (1D1V, smallest grids) segments of 4: there the FP64 pipe of the few
     // SMs at work and the depth of a segment bound the sweep (64 cells of 32
     // velocities: one tile of 32 columns in segments of 16 13.5 us, four tiles in
-    // segments of 16 15.5, in segments of 4 9.5)
-    const int cells = precision == 64 && ntiles < 152 ? 4 : 16;
+    // segments of 16 15.5, in segments of 4 9.5; 512 cells 20.6 against 30.9; a line of
+    // 1024 cells keeps the pipe busy with 16, 30.9 against 32.9)
+    const int cells = precision == 64 && ntiles < 152 && a.n < 1024 ? 4 : 16;
     int nseg = (a.n + cells - 1) / cells;
     if (nseg > 1024 / a.ncol) nseg = 1024 / a.ncol;
     if (nseg < 1) nseg = 1;
