@@ -443,14 +443,13 @@ vl_status pfc_advect_xy(vl_ctx* ctx, int s, double dt, void* f_out, vl_stream_t 
     const bool fused = a.tx && a.ty && a.hy <= 8 && a.hy <= d.ny && ntiles < (1LL << 31);
     cudaStream_t cs = (cudaStream_t)stream;
     cudaError_t e = cudaErrorNotSupported;
-    if (d.precision == 32 && fused && vl::march_fits(a)) {
-        // Whole 16 x 16 tiles with shifts up to 2 cells add an update's two
-        // products in physical order, other grids in the order of the sweep's
-        // direction: the roundings pfc_advect_xy has had on either kind of
-        // grid, so that a run keeps its bits
-        const bool frame = !(a.hx <= 4 && a.hy <= 4 && d.nx % 16 == 0 && d.ny % 16 == 0);
+    // Whole 16 x 16 tiles with shifts up to 2 cells add an update's two
+    // products in physical order, other grids in the order of the sweep's
+    // direction: the roundings pfc_advect_xy has had on either kind of
+    // grid, so that a run keeps its bits
+    const bool frame = !(a.hx <= 4 && a.hy <= 4 && d.nx % 16 == 0 && d.ny % 16 == 0);
+    if (d.precision == 32 && fused && vl::march_fits(a) && !(frame && vl::march_late(a, ntiles)))
         e = vl::launch_pfc_space_march(a, frame, cs);
-    }
     if (e != cudaErrorNotSupported) {
         st = cuda_check(ctx, e, "pfc_advect_xy");
     } else if (fused) {

@@ -68,9 +68,12 @@ struct SpaceXYArgs {
 };
 size_t pfc_space_xy_smem(const SpaceXYArgs& a, int precision);
 cudaError_t launch_pfc_space_xy(const SpaceXYArgs& a, int precision, cudaStream_t st);
-// the streamed form in FP32 (pfc_space_march.cu), any grid; frame: products
-// added in the single-axis sweeps' order. cudaErrorNotSupported: not taken
+// the streamed form in FP32 (pfc_space_march.cu); frame: products added in the
+// single-axis sweeps' order. cudaErrorNotSupported: not taken. march_fits: can it
+// take the call (rows of whole 8-cell groups, any number of rows)? march_late: is
+// pfc_space_xy_kernel, which has frame's roundings, done sooner?
 bool march_fits(const SpaceXYArgs& a);
+bool march_late(const SpaceXYArgs& a, long long ntiles);
 cudaError_t launch_pfc_space_march(const SpaceXYArgs& a, bool frame, cudaStream_t st);
 
 // ---- velocity-space PFC pass (+ fused moments) -----------------------------

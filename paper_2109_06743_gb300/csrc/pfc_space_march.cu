@@ -394,6 +394,19 @@ bool march_fits(const SpaceXYArgs& a) {
            a.counters != nullptr;
 }
 
+// Small grids of one or two groups of cells in x with long shifts, and 8 x 8 cells: a
+// march starts with a ring to set up and 2 hy rows that emit nothing, and a few
+// CTAs have little to hide them behind. us, march / tiles: 8 x 8 cells of 12^3 8.3 /
+// 6.3 at half a cell, 12.5 / 8.4 at 6; 16 x 16 of 16^3 10.4 / 10.4 at 2 cells, 14.5 / 10.4
+// at 4, 16.5 / 12.4 at 6; of 24^3 16.6 / 20.7 at 1, 26.7 / 22.7 at 4; 8 x 128 of 12^3 16.6 /
+// 18.6 at 3, 20.7 / 18.6 at 5. Wider than high it is the other way: 64 x 8 of 12^3 14.5 /
+// 18.6 at 6.
+bool march_late(const SpaceXYArgs& a, long long ntiles) {
+    if (a.nx > 16 || a.ny < a.nx) return false;
+    if (ntiles <= 128 && (a.hx >= 5 || a.nx * a.ny <= 64)) return true;
+    return ntiles <= 448 && a.hx >= 6;
+}
+
 cudaError_t launch_pfc_space_march(const SpaceXYArgs& a, bool frame, cudaStream_t st) {
     return frame ? launch_t<true>(a, st) : launch_t<false>(a, st);
 }
