@@ -23,7 +23,8 @@ spatial cells x velocity cells) x steps / time, over all ranks.
 project; the paper has no code) on a bounded sample of the same workload on
 the host cores. Under torchrun each rank runs an independent replica
 (replicas only: the method's spatial decomposition is not needed on one
-GPU), the slowest rank's time is used and rank 0 prints one JSON line.
+GPU), the slowest rank's time is used and rank 0 prints one JSON line; --record
+PATH keeps the full record (every block of every workload).
 """
 from __future__ import annotations
 
@@ -963,6 +964,38 @@ def shear_ablation(device, steps=100):
     return out
 
 
+# what the printed line keeps of each block, in full or by key
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "roofline", "phases_ms_per_step", "newton_iterations_per_fit",
+             "gpu_launches", "clocks")
+LINE_PARTS = {"e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps", "ms_per_step", "run_reported"),
+              "mlp": ("newton_iterations_per_fit", "fits_started_warm"),
+              "cpu_baseline": ("value", "unit", "cores", "kind"),
+              "fp64_form": ("value", "unit", "ms_per_step"),
+              "newton_roofline": ("bound", "frac", "unit")}
+LINE_NESTED = ("value", "unit", "ms_per_step", "steps")
+
+
+def printed_line(record):
+    """The record's line on standard output: the contract's keys and one figure per
+    block, some 2500 characters. The record itself is ten times as long (every run
+    of the end-to-end leg, the other workloads' blocks) and goes to --record PATH: a
+    reader that keeps the end of a line only, or bounds its length, lost the value."""
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    for key, parts in LINE_PARTS.items():
+        if record.get(key):
+            line[key] = {k: record[key][k] for k in parts if k in record[key]}
+    cold = (record.get("mlp") or {}).get("cold_start")
+    if cold:
+        line["mlp"]["cold_start_ms_per_step"] = cold["ms_per_step"]
+    for name, block in (record.get("workloads") or {}).items():
+        short = {k: block[k] for k in LINE_NESTED if k in block}
+        if block.get("e2e"):
+            short["e2e_value"] = block["e2e"]["value"]
+        line.setdefault("workloads", {})[name] = short
+    return line
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -983,6 +1016,7 @@ def main():
     ap.add_argument("--no-extra", action="store_true",
                     help="only the named workload: no nested lines of the other workloads, no network transfer, "
                          "no shear ablation")
+    ap.add_argument("--record", default=None, metavar="PATH", help="write the full record (every block) to PATH")
     args = ap.parse_args()
 
     rank = int(os.environ.get("RANK", "0"))
@@ -1046,7 +1080,10 @@ def main():
                 device, res["ms_per_step"], {k: v["ms_per_launch"] for k, v in res["hbm_phases"].items()})
         line["workloads"] = nested
     if rank == 0:
-        print(json.dumps(line))
+        if args.record:
+            with open(args.record, "w") as fh:
+                json.dump(line, fh, indent=1)
+        print(json.dumps(printed_line(line)))
     if dist:
         dist.destroy_process_group()
     return 0
